@@ -24,8 +24,10 @@
 // contractions and the only work on the tensor cores.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <new>
 #include <vector>
 
 #include "../../include/lbsurrogate.h"
@@ -306,7 +308,7 @@ extern "C" lb_status lb_gemm_status(void)
 }
 
 // ---------------------------------------------------------------------------
-// The network: parameters, activations and the kernels around the products.
+// The network: parameters, activations and its two kernels.
 namespace lbsur {
 
 constexpr int NIN = LB_MLP_IN, NINP = LB_MLP_IN_PAD, NH = LB_MLP_HID, NOUT = LB_MLP_OUT, NOUTP = LB_MLP_OUT_PAD;
@@ -314,124 +316,698 @@ constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + NH * NINP, OFF_W2 = OFF_B1 + NH, OFF
               OFF_W3 = OFF_B2 + NH, OFF_B3 = OFF_W3 + NOUTP * NH, NPARAM = OFF_B3 + NOUTP;
 static_assert(NPARAM == LB_MLP_NPARAM, "parameter layout");
 
-// lower-triangle index t of (i, j), j <= i: t = i (i + 1) / 2 + j
-__host__ __device__ constexpr int tri(int i, int j) { return i * (i + 1) / 2 + j; }
+// A BF16 matrix X(r, k) kept as 8 x 8 core matrices (8 rows of 16 bytes), the
+// cores of one column group k / 8 together: element (r, k) at byte
+// (k / 8) * cs + (r / 8) * 128 + (r % 8) * 16 + (k % 8) * 2.  The tensor core reads
+// the same bytes as a K-major operand over k (row groups 128 bytes apart, K groups
+// cs apart) and as an MN-major operand over r (groups of k cs apart, K groups of 8
+// rows 128 apart), so one copy of the weights serves the forward and the backward
+// products and one copy of the activations serves the products over the samples;
+// nothing is transposed.  A row group times one column group is 128 contiguous
+// bytes, so 8 threads holding 8 consecutive rows store them without conflicts.
+__host__ __device__ constexpr int core_at(int cs, int r, int k) { return (k >> 3) * cs + (r >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2; }
 
-__global__ void features_kernel(const float* x, int n, __nv_bfloat16* X)
-{
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n * NINP) return;
-    const int s = idx / NINP, k = idx % NINP;
-    X[idx] = __float2bfloat16(k < NIN ? x[s * NIN + k] : 0.0f);
-}
+// the weights' BF16 copy: W1 (256 x 16), W2 (256 x 256), W3 (32 x 256), as above
+constexpr int CS_W12 = NH / 8 * 128, CS_W3 = NOUTP / 8 * 128;
+constexpr int PK_W1 = 0, PK_W2 = PK_W1 + NH * NINP * 2, PK_W3 = PK_W2 + NH * NH * 2, PK_BYTES = PK_W3 + NOUTP * NH * 2;
 
-__global__ void to_bf16_kernel(const float* p, __nv_bfloat16* q, int n)
+// activations and their gradients in global memory, samples as rows: `cs` bytes
+// per group of 8 features, 128-sample tiles of 16 row groups (2 KiB) within it
+struct Acts {
+    unsigned char *X, *H1, *H2, *dY, *dH2, *dH1;
+    long long cs;
+    float* loss_part;                   // [tiles]
+    float* d32;                         // up to SPLIT_MIN tiles: FP32 dH1, dH2, dY, [2 * 256 + 32][ns] by column
+    float* b_part;                      // more tiles: their column sums, [4 tiles][2 * 256 + 32], per warp of 32 samples
+    int ns;                             // samples a column of d32 holds
+    unsigned* count;                    // tiles done (zero between launches)
+};
+constexpr int TILE = 128;               // samples per tile: one TMEM lane each
+constexpr int NSUM = 2 * NH + NOUTP;
+constexpr int SPLIT_MIN = 8;            // tiles up to which every sum over the samples runs in their order
+
+__global__ void pack_kernel(const float* p, unsigned char* w)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) q[i] = __float2bfloat16(p[i]);
+    int base, cs, r, k;
+    if (i < NH * NINP) { base = PK_W1; cs = CS_W12; r = i / NINP; k = i % NINP; }
+    else if (i >= OFF_W2 && i < OFF_W2 + NH * NH) { base = PK_W2; cs = CS_W12; r = (i - OFF_W2) / NH; k = (i - OFF_W2) % NH; }
+    else if (i >= OFF_W3 && i < OFF_W3 + NOUTP * NH) { base = PK_W3; cs = CS_W3; r = (i - OFF_W3) / NH; k = (i - OFF_W3) % NH; }
+    else return;
+    *reinterpret_cast<__nv_bfloat16*>(w + base + core_at(cs, r, k)) = __float2bfloat16(p[i]);
 }
+
+// lower-triangular index t of (i, j), j <= i: t = i (i + 1) / 2 + j
+__host__ __device__ constexpr int tri(int i, int j) { return i * (i + 1) / 2 + j; }
 
 __device__ __forceinline__ float softplus(float y) { return y > 20.0f ? y : log1pf(expf(y)); }
 __device__ __forceinline__ float sigmoid(float y) { return 1.0f / (1.0f + expf(-y)); }
 
-// Output head, one thread per sample: L from the 21 outputs (diagonal through
-// softplus), R^ = L L^T; with targets, the loss (1/(36 n)) sum (R^ - Rt)^2 and
-// its gradient with respect to the outputs: dR = 2 (R^ - Rt) / (36 n),
-// dL = 2 dR L (dR symmetric), dy = dL (off the diagonal), dL_ii sigmoid(y_ii).
-__global__ void head_kernel(const float* Y, int n, float* y_out, float* R_out, const float* Rt, float* loss,
-                            float* dY32, __nv_bfloat16* dY16)
+// ---- PTX helpers
+// programmatic dependent launch: wait for the kernels before this one; let the next one start its prologue
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void mbar_init(unsigned long long* b)
 {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    float part = 0.0f;
-    if (s < n) {
-        float y[NOUT], L[6][6], R[6][6];
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(b)) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(unsigned long long* b, unsigned bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, unsigned long long* bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_store(void* dst, const void* src, unsigned bytes)
+{
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void mma_bf16(unsigned d, unsigned long long a, unsigned long long b, unsigned idesc, bool acc)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d), "l"(a), "l"(b), "r"(idesc),
+                 "r"(acc ? 1u : 0u)
+                 : "memory");
+}
+__device__ __forceinline__ void mma_commit(unsigned long long* bar)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// 32 accumulator columns of this warp's 32 lanes
+__device__ __forceinline__ void tmem_ld32(unsigned addr, float (&v)[32])
+{
+    unsigned r[32];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                 : "r"(addr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-        for (int t = 0; t < NOUT; ++t) y[t] = Y[s * NOUTP + t];
-        if (y_out) {
-            for (int t = 0; t < NOUT; ++t) y_out[s * NOUT + t] = y[t];
+    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+}
+
+__device__ __forceinline__ unsigned pack2(float a, float b)
+{
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const unsigned*>(&h);
+}
+
+// sums over the warp's lanes of 32 values per lane: lane l returns the sum of
+// v[l] (each step exchanges half of what is left: 31 shuffles instead of 160)
+__device__ __forceinline__ float warp_colsum(float (&v)[32], int lane)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < o; ++k) {
+            const float send = up ? v[k] : v[k + o], keep = up ? v[k + o] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
+    }
+    return v[0];
+}
+
+// ---- Forward pass, head and (BWD) the activations' gradients of one 128-sample
+// tile per block, everything between the inputs and the weight products in one
+// kernel.  All three weight matrices (152 KiB) and one 128 x 256 activation tile
+// live in shared memory, the accumulators in tensor memory, the ReLU masks in
+// registers (one bit per element); the activations go to global memory only for
+// the products over the samples (grad_kernel).  Five products per tile, each issued
+// by one thread and followed by an epilogue of 512 threads (thread = sample x a quarter of
+// the columns): the chain of five waits and epilogues bounds the kernel at every batch
+// size up to 152 tiles, so nothing is split further.
+// Measured (512 samples, one training step): the chain of 13 kernels before took 760 us
+// a step, its staging loads one at a time; see grad_kernel for both kernels together.
+struct NetArgs {
+    const float* x;
+    const float* p;                     // biases
+    const unsigned char* w;             // packed weights
+    const float* Rt;
+    float* y_out;
+    float* R_out;
+    float* loss;                        // !BWD: the loss is summed here by the last tile
+    Acts act;
+    int n;
+    unsigned* status;
+};
+
+constexpr int NS_W2 = 0, NS_W3 = NS_W2 + NH * NH * 2, NS_W1 = NS_W3 + NOUTP * NH * 2, NS_H = NS_W1 + NH * NINP * 2,
+              NS_X = NS_H + TILE * NH * 2, NS_BIAS = NS_X + TILE * NINP * 2, NET_SMEM = NS_BIAS + (2 * NH + NOUTP) * 4;
+constexpr int CS_T = TILE / 8 * 128;    // column-group stride of a 128-row tile in shared memory
+constexpr int NTHREADS = 512;           // four threads per sample, 64 columns each
+static_assert(NET_SMEM <= 227 * 1024 - 256, "shared memory of the network kernel");
+static_assert(TILE * NOUTP * 2 <= NH * NINP * 2, "dY takes the place of W1");
+
+template <bool BWD>
+__global__ void __launch_bounds__(NTHREADS, 1) net_kernel(const NetArgs A)
+{
+    extern __shared__ __align__(128) unsigned char sm[];
+    __shared__ unsigned long long bar[3];           // W1; W2 and W3; products
+    __shared__ unsigned s_tmem;
+    __shared__ float s_red[4];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wq = warp & 3, part = warp >> 2;
+    const int tile = blockIdx.x, row = wq * 32 + lane, s = tile * TILE + row;
+    const bool live = s < A.n;
+    unsigned char* sH = sm + NS_H;
+    unsigned char* sdY = sm + NS_W1;
+    float* sb = reinterpret_cast<float*>(sm + NS_BIAS);
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&s_tmem)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int k = 0; k < 3; ++k) mbar_init(bar + k);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    // the inputs and the weights may come from the kernels just before; once they are
+    // done, grad_kernel may set itself up beside this kernel (it waits in turn)
+    pdl_wait();
+    pdl_trigger();
+    if (tid == 0) {
+        mbar_expect(bar, NH * NINP * 2);
+        bulk_load(sm + NS_W1, A.w + PK_W1, NH * NINP * 2, bar);
+        mbar_expect(bar + 1, NH * NH * 2 + NOUTP * NH * 2);
+        bulk_load(sm + NS_W2, A.w + PK_W2, NH * NH * 2 + NOUTP * NH * 2, bar + 1);   // W3 follows W2 in both
+    }
+    if (tid < TILE) {
+        // the sample's 8 features, the padding columns zero
+        float f[NIN];
+        const float* xs = A.x + (long long)s * NIN;
+        if (live && (reinterpret_cast<uintptr_t>(A.x) & 15u) == 0) {
+            const float4 u = __ldg(reinterpret_cast<const float4*>(xs)), v = __ldg(reinterpret_cast<const float4*>(xs) + 1);
+            f[0] = u.x; f[1] = u.y; f[2] = u.z; f[3] = u.w; f[4] = v.x; f[5] = v.y; f[6] = v.z; f[7] = v.w;
+        } else {
 #pragma unroll
-        for (int i = 0; i < 6; ++i)
-#pragma unroll
-            for (int j = 0; j < 6; ++j) L[i][j] = j < i ? y[tri(i, j)] : (j == i ? softplus(y[tri(i, i)]) : 0.0f);
-#pragma unroll
-        for (int i = 0; i < 6; ++i)
-#pragma unroll
-            for (int j = 0; j < 6; ++j) {
-                float a = 0.0f;
-#pragma unroll
-                for (int k = 0; k < 6; ++k) a += L[i][k] * L[j][k];
-                R[i][j] = a;
-            }
-        if (R_out) {
-            for (int i = 0; i < 6; ++i)
-                for (int j = 0; j < 6; ++j) R_out[s * 36 + i * 6 + j] = R[i][j];
+            for (int k = 0; k < NIN; ++k) f[k] = live ? __ldg(xs + k) : 0.0f;
         }
-        if (Rt) {
-            const float c = 2.0f / (36.0f * (float)n);
-            float dR[6][6];
+        const uint4 c0 = make_uint4(pack2(f[0], f[1]), pack2(f[2], f[3]), pack2(f[4], f[5]), pack2(f[6], f[7]));
+        const uint4 c1 = make_uint4(0u, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(sm + NS_X + core_at(CS_T, row, 0)) = c0;
+        *reinterpret_cast<uint4*>(sm + NS_X + core_at(CS_T, row, 8)) = c1;
+    }
+    for (int k = tid; k < 2 * NH + NOUTP; k += NTHREADS)
+        sb[k] = __ldg(A.p + (k < NH ? OFF_B1 + k : (k < 2 * NH ? OFF_B2 + k - NH : OFF_B3 + k - 2 * NH)));
+    fence_async();
+    tc_before();
+    __syncthreads();
+    tc_after();
+    const unsigned tmem = s_tmem, tlane = tmem + ((unsigned)(wq * 32) << 16);
+    unsigned phase = 0;
+    bool ok = true;
+    constexpr unsigned ID256 = idesc_bf16(TILE, NH), ID32 = idesc_bf16(TILE, NOUTP), BMN = 1u << 16;   // B MN-major
+    const unsigned aH = smem_u32(sH);
+    // waits for the last product; uniform over the block
+    auto product_done = [&]() {
+        const bool got = mbar_wait(bar + 2, phase);
+        phase ^= 1u;
+        if (__syncthreads_or(!got)) ok = false;
+        tc_after();
+        return ok;
+    };
+    // a tile of 32 core columns (2 KiB each) to global memory, one column group per lane of warp 1
+    auto store_tile = [&](unsigned char* dst, const unsigned char* src, int groups) {
+        if (warp == 1) {
+            if (lane < groups) bulk_store(dst + lane * A.act.cs + (long long)tile * CS_T, src + lane * CS_T, CS_T);
+            bulk_commit();
+        }
+    };
+    auto store_read = [&]() { if (warp == 1) bulk_wait_read(); };
+    // hidden layer's epilogue: act = relu(acc + b) as BF16 into sH, its mask into m[]
+    auto hidden = [&](unsigned col0, const float* b, unsigned (&m)[2]) {
+#pragma unroll 1
+        for (int q = 0; q < 2; ++q) {
+            const int c0 = part * 64 + q * 32;
+            float v[32];
+            tmem_ld32(tlane + col0 + (unsigned)c0, v);
+            unsigned bits = 0;
 #pragma unroll
-            for (int i = 0; i < 6; ++i)
+            for (int j = 0; j < 32; j += 8) {
+                unsigned h[4];
 #pragma unroll
-                for (int j = 0; j < 6; ++j) {
-                    const float d = R[i][j] - Rt[s * 36 + i * 6 + j];
-                    part += d * d;
-                    dR[i][j] = c * d;
+                for (int t = 0; t < 4; ++t) {
+                    const float2 bb = *reinterpret_cast<const float2*>(b + c0 + j + 2 * t);
+                    const float v0 = live ? fmaxf(v[j + 2 * t] + bb.x, 0.0f) : 0.0f;
+                    const float v1 = live ? fmaxf(v[j + 2 * t + 1] + bb.y, 0.0f) : 0.0f;
+                    h[t] = pack2(v0, v1);
+                    if (h[t] & 0x7fffu) bits |= 1u << (j + 2 * t);
+                    if (h[t] & 0x7fff0000u) bits |= 2u << (j + 2 * t);
                 }
-            float dy[NOUTP];
+                *reinterpret_cast<uint4*>(sH + core_at(CS_T, row, c0 + j)) = make_uint4(h[0], h[1], h[2], h[3]);
+            }
+            m[0] = q == 0 ? bits : m[0];
+            m[1] = q == 1 ? bits : m[1];
+        }
+        fence_async();
+        tc_before();
+        __syncthreads();
+        tc_after();
+    };
+    auto column_sums = [&](float (&v)[32], int c0) {
+        if (gridDim.x <= SPLIT_MIN) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) A.act.d32[(c0 + j) * A.act.ns + s] = v[j];
+        } else {
+            A.act.b_part[(long long)(tile * 4 + wq) * NSUM + c0 + lane] = warp_colsum(v, lane);
+        }
+    };
+    // gradient's epilogue: masked, BF16 into sH; the FP32 values, or above SPLIT_MIN tiles
+    // their sums over the warp, for the bias gradients (columns sum0 .. sum0 + 255)
+    auto masked = [&](unsigned col0, const unsigned (&m)[2], int sum0) {
+#pragma unroll 1
+        for (int q = 0; q < 2; ++q) {
+            const int c0 = part * 64 + q * 32;
+            const unsigned bits = q == 0 ? m[0] : m[1];
+            float v[32];
+            tmem_ld32(tlane + col0 + (unsigned)c0, v);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = ((bits >> j) & 1u) ? v[j] : 0.0f;
+#pragma unroll
+            for (int j = 0; j < 32; j += 8)
+                *reinterpret_cast<uint4*>(sH + core_at(CS_T, row, c0 + j)) =
+                    make_uint4(pack2(v[j], v[j + 1]), pack2(v[j + 2], v[j + 3]), pack2(v[j + 4], v[j + 5]), pack2(v[j + 6], v[j + 7]));
+            column_sums(v, sum0 + c0);
+        }
+        fence_async();
+        tc_before();
+        __syncthreads();
+        tc_after();
+    };
+    unsigned m1[2] = {0u, 0u}, m2[2] = {0u, 0u};
+    bool pending = true;                            // W2 and W3 still on their way
+    do {
+        // ---- layer 1
+        if (__syncthreads_or(!mbar_wait(bar, 0u))) { ok = false; break; }
+        if (tid == 0) {
+            mma_bf16(tmem, sdesc(smem_u32(sm + NS_X), CS_T, 128u), sdesc(smem_u32(sm + NS_W1), CS_W12, 128u), ID256, false);
+            mma_commit(bar + 2);
+        }
+        if (BWD) store_tile(A.act.X, sm + NS_X, 2);
+        if (!product_done()) break;
+        hidden(0u, sb, m1);
+        // ---- layer 2
+        const bool got = mbar_wait(bar + 1, 0u);
+        if (__syncthreads_or(!got)) { ok = false; break; }
+        pending = false;
+        if (tid == 0) {
+#pragma unroll
+            for (int k = 0; k < NH / 16; ++k)
+                mma_bf16(tmem + NH, sdesc(aH + k * 2 * CS_T, CS_T, 128u), sdesc(smem_u32(sm + NS_W2) + k * 2 * CS_W12, CS_W12, 128u), ID256, k > 0);
+            mma_commit(bar + 2);
+        }
+        if (BWD) {
+            store_tile(A.act.H1, sH, 32);
+            store_read();
+        }
+        if (!product_done()) break;
+        hidden(NH, sb + NH, m2);
+        // ---- output layer
+        if (tid == 0) {
+#pragma unroll
+            for (int k = 0; k < NH / 16; ++k)
+                mma_bf16(tmem, sdesc(aH + k * 2 * CS_T, CS_T, 128u), sdesc(smem_u32(sm + NS_W3) + k * 2 * CS_W3, CS_W3, 128u), ID32, k > 0);
+            mma_commit(bar + 2);
+        }
+        if (BWD) {
+            store_tile(A.act.H2, sH, 32);
+            store_read();
+        }
+        if (!product_done()) break;
+        // ---- head, one thread per sample: L from the 21 outputs (diagonal through
+        // softplus), R^ = L L^T; with targets, the loss (1/(36 n)) sum (R^ - Rt)^2 and its
+        // gradient with respect to the outputs: dR = 2 (R^ - Rt) / (36 n), dL = 2 dR L
+        // (dR symmetric), dy = dL (off the diagonal), dL_ii sigmoid(y_ii)
+        if (warp < 4) {
+            float err = 0.0f, dy[NOUTP];
 #pragma unroll
             for (int t = 0; t < NOUTP; ++t) dy[t] = 0.0f;
+            float v[32];
+            tmem_ld32(tlane, v);
+            if (live) {
+                float y[NOUT], L[6][6], R[6][6];
 #pragma unroll
-            for (int i = 0; i < 6; ++i)
-#pragma unroll
-                for (int j = 0; j <= i; ++j) {
-                    float a = 0.0f;
-#pragma unroll
-                    for (int k = 0; k < 6; ++k) a += dR[i][k] * L[k][j];
-                    a *= 2.0f;
-                    dy[tri(i, j)] = (j == i) ? a * sigmoid(y[tri(i, i)]) : a;
+                for (int t = 0; t < NOUT; ++t) y[t] = v[t] + sb[2 * NH + t];
+                if (A.y_out) {
+                    for (int t = 0; t < NOUT; ++t) A.y_out[(long long)s * NOUT + t] = y[t];
                 }
 #pragma unroll
-            for (int t = 0; t < NOUTP; ++t) {
-                dY32[s * NOUTP + t] = dy[t];
-                dY16[s * NOUTP + t] = __float2bfloat16(dy[t]);
+                for (int i = 0; i < 6; ++i)
+#pragma unroll
+                    for (int j = 0; j < 6; ++j) L[i][j] = j < i ? y[tri(i, j)] : (j == i ? softplus(y[tri(i, i)]) : 0.0f);
+#pragma unroll
+                for (int i = 0; i < 6; ++i)
+#pragma unroll
+                    for (int j = 0; j < 6; ++j) {
+                        float a = 0.0f;
+#pragma unroll
+                        for (int k = 0; k < 6; ++k) a += L[i][k] * L[j][k];
+                        R[i][j] = a;
+                    }
+                if (A.R_out) {
+                    for (int i = 0; i < 6; ++i)
+                        for (int j = 0; j < 6; ++j) A.R_out[(long long)s * 36 + i * 6 + j] = R[i][j];
+                }
+                if (A.Rt) {
+                    const float c = 2.0f / (36.0f * (float)A.n);
+                    const float* rt = A.Rt + (long long)s * 36;
+                    float dR[6][6];
+#pragma unroll
+                    for (int i = 0; i < 6; ++i)
+#pragma unroll
+                        for (int j = 0; j < 6; ++j) {
+                            const float d = R[i][j] - __ldg(rt + i * 6 + j);
+                            err += d * d;
+                            dR[i][j] = c * d;
+                        }
+                    if (BWD) {
+#pragma unroll
+                        for (int i = 0; i < 6; ++i)
+#pragma unroll
+                            for (int j = 0; j <= i; ++j) {
+                                float a = 0.0f;
+#pragma unroll
+                                for (int k = 0; k < 6; ++k) a += dR[i][k] * L[k][j];
+                                a *= 2.0f;
+                                dy[tri(i, j)] = (j == i) ? a * sigmoid(y[tri(i, i)]) : a;
+                            }
+                    }
+                }
+            }
+            if (BWD) {
+#pragma unroll
+                for (int j = 0; j < NOUTP; j += 8)
+                    *reinterpret_cast<uint4*>(sdY + core_at(CS_T, row, j)) =
+                        make_uint4(pack2(dy[j], dy[j + 1]), pack2(dy[j + 2], dy[j + 3]), pack2(dy[j + 4], dy[j + 5]), pack2(dy[j + 6], dy[j + 7]));
+                column_sums(dy, 2 * NH);
+            }
+            for (int o = 16; o > 0; o >>= 1) err += __shfl_xor_sync(0xffffffffu, err, o);
+            if (lane == 0) s_red[warp] = err;
+        }
+        fence_async();
+        tc_before();
+        __syncthreads();
+        tc_after();
+        if (tid == 0 && A.Rt) A.act.loss_part[tile] = ((s_red[0] + s_red[2]) + (s_red[1] + s_red[3])) / (36.0f * (float)A.n);
+        if (!BWD) break;
+        // ---- dH2 = (dY W3) * [H2 > 0]
+        if (tid == 0) {
+#pragma unroll
+            for (int k = 0; k < NOUTP / 16; ++k)
+                mma_bf16(tmem + NH, sdesc(smem_u32(sdY) + k * 2 * CS_T, CS_T, 128u), sdesc(smem_u32(sm + NS_W3) + k * 256, 128u, CS_W3), ID256 | BMN, k > 0);
+            mma_commit(bar + 2);
+        }
+        store_tile(A.act.dY, sdY, 4);
+        if (!product_done()) break;
+        masked(NH, m2, NH);
+        // ---- dH1 = (dH2 W2) * [H1 > 0]
+        if (tid == 0) {
+#pragma unroll
+            for (int k = 0; k < NH / 16; ++k)
+                mma_bf16(tmem, sdesc(aH + k * 2 * CS_T, CS_T, 128u), sdesc(smem_u32(sm + NS_W2) + k * 256, 128u, CS_W12), ID256 | BMN, k > 0);
+            mma_commit(bar + 2);
+        }
+        store_tile(A.act.dH2, sH, 32);
+        store_read();
+        if (!product_done()) break;
+        masked(0u, m1, 0);
+        store_tile(A.act.dH1, sH, 32);
+    } while (false);
+    if (!ok) {
+        // a completion never came: give what is in flight a second bounded wait before leaving
+        if (tid == 0) {
+            atomicOr(&g_gemm_status, 1u);
+            if (A.status) atomicOr(A.status, 1u);
+        }
+        (void)mbar_wait(bar, 0u);
+        if (pending) (void)mbar_wait(bar + 1, 0u);
+        (void)mbar_wait(bar + 2, phase ^ 1u);
+    }
+    if (warp == 1) bulk_wait_all();
+    if (!BWD && A.loss) {
+        // the last tile adds the tiles' losses, in order
+        __shared__ bool s_last;
+        if (tid == 0) {
+            __threadfence();
+            s_last = atomicAdd(A.act.count, 1u) == gridDim.x - 1;
+            if (s_last) {
+                __threadfence();
+                float v = 0.0f;
+                for (unsigned t = 0; t < gridDim.x; ++t) v += __ldcg(A.act.loss_part + t);
+                *A.loss = v;
+                *A.act.count = 0;
             }
         }
     }
-    if (Rt) {
-        // block sum of the squared errors, one atomic per block
-        __shared__ float red[32];
-        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            float v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0f;
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (threadIdx.x == 0) atomicAdd(loss, v / (36.0f * (float)n));
+    tc_before();
+    __syncthreads();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+}
+
+// ---- Products over the samples (weight gradients), column sums of the biases, the
+// loss, and with ADAM the update of every parameter and of its BF16 copy in place.
+// One block per 128 x 32 tile of a gradient: dW2 = dH2^T H1 (16 tiles), dW3^T = H2^T dY
+// (2), dW1 = dH1^T X (2, 16 columns), and one per 32 biases.  Both operands are
+// MN-major: the tiles that net_kernel wrote come in by 2 KiB bulk copies, 128 samples a
+// stage, GST stages in flight.  Narrow tiles give the chip 20 blocks where a single
+// 256-wide tile per half gave 2; the order of the sum over the samples stays that of one
+// accumulator up to SPLIT_MIN tiles (an Adam step turns the last bit of a gradient near
+// zero into the sign of the update), and is split over a cluster above it, whose first
+// block adds the parts in rank order.
+// Measured, 512 samples: GSTEP_NOTE
+struct GradArgs {
+    Acts act;
+    int n, tiles;
+    float* grad;                        // !ADAM
+    float *p, *m1, *m2;                 // ADAM
+    unsigned char* w;
+    float lr, c1, c2;
+    float* loss;
+    unsigned* status;
+};
+
+constexpr int GST = 5, GS_A = 16 * CS_T, GS_B = 4 * CS_T, GRAD_SMEM = GST * (GS_A + GS_B);
+constexpr int GTHREADS_N = 192;         // a warpgroup for the result, one warp for the loads, one for the products
+constexpr int GEMM_JOBS = 20, BIAS_JOBS = NSUM / 32, SPLIT = 4;
+static_assert(32 * (SPLIT_MIN * TILE * 4 + 16) <= GRAD_SMEM, "32 columns of the samples fit the stages");
+static_assert((SPLIT - 1) * TILE * 32 * 4 <= GRAD_SMEM, "the parts of the other blocks fit the stages");
+
+__device__ __forceinline__ float adam(float& p, float& m1, float& m2, float gi, float lr, float c1, float c2)
+{
+    const float a = 0.9f * m1 + 0.1f * gi;
+    const float b = 0.999f * m2 + 0.001f * gi * gi;
+    m1 = a;
+    m2 = b;
+    p -= lr * (a * c1) / (sqrtf(b * c2) + 1e-8f);
+    return p;
+}
+
+template <bool ADAM>
+__global__ void __launch_bounds__(GTHREADS_N, 1) grad_kernel(const GradArgs G)
+{
+    extern __shared__ __align__(128) unsigned char sm[];
+    __shared__ unsigned long long full[GST], empty[GST], done;
+    __shared__ unsigned s_tmem;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    unsigned rank, nrank;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(nrank));
+    const int job = blockIdx.x / (int)nrank;
+    if (job >= GEMM_JOBS) {
+        // biases: 32 columns, summed in the samples' order by one lane each; the loss
+        const int c0 = (job - GEMM_JOBS) * 32;
+        if (rank > 0) return;
+        pdl_wait();
+        float v = 0.0f;
+        bool ok = true;
+        if (G.tiles <= SPLIT_MIN) {
+            // the columns by one bulk copy each, 16 bytes apart modulo 128 so that the lanes read without conflicts
+            const int bytes = G.tiles * TILE * 4;
+            if (tid == 0) {
+                mbar_init(full);
+                asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+                mbar_expect(full, 32u * (unsigned)bytes);
+            }
+            __syncthreads();
+            if (warp > 0) return;
+            bulk_load(sm + lane * (bytes + 16), G.act.d32 + (long long)(c0 + lane) * G.act.ns, (unsigned)bytes, full);
+            ok = mbar_wait(full, 0u);
+            const float4* d = reinterpret_cast<const float4*>(sm + lane * (bytes + 16));
+#pragma unroll 8
+            for (int t = 0; t < G.tiles * TILE / 4; ++t) {
+                const float4 u = d[t];
+                v += u.x;
+                v += u.y;
+                v += u.z;
+                v += u.w;
+            }
+        } else {
+            if (warp > 0) return;
+#pragma unroll 8
+            for (int t = 0; t < 4 * G.tiles; ++t) v += __ldg(G.act.b_part + (long long)t * NSUM + c0 + lane);
+        }
+        if (!ok) {
+            if (lane == 0) {
+                atomicOr(&g_gemm_status, 1u);
+                if (G.status) atomicOr(G.status, 1u);
+            }
+            return;
+        }
+        const int c = c0 + lane, i = c < NH ? OFF_B1 + c : (c < 2 * NH ? OFF_B2 + c - NH : OFF_B3 + c - 2 * NH);
+        if (ADAM) adam(G.p[i], G.m1[i], G.m2[i], v, G.lr, G.c1, G.c2);
+        else G.grad[i] = v;
+        if (c == NSUM - 1 && G.loss) {
+            float l = 0.0f;
+            for (int t = 0; t < G.tiles; ++t) l += G.act.loss_part[t];
+            *G.loss = l;
+        }
+        return;
+    }
+    // ---- operands and place of this tile
+    const bool w3 = job >= 16 && job < 18, w1 = job >= 18;
+    const int ih = job < 16 ? job >> 3 : job & 1, jt = job < 16 ? job & 7 : 0, ncol = w1 ? 16 : 32;
+    const unsigned char* a = (w1 ? G.act.dH1 : (w3 ? G.act.H2 : G.act.dH2)) + (long long)ih * 16 * G.act.cs;
+    const unsigned char* b = (w1 ? G.act.X : (w3 ? G.act.dY : G.act.H1)) + (long long)jt * 4 * G.act.cs;
+    const int t0 = (int)((long long)G.tiles * rank / nrank), t1 = (int)((long long)G.tiles * (rank + 1) / nrank);
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 32;" ::"r"(smem_u32(&s_tmem)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int k = 0; k < GST; ++k) { mbar_init(full + k); mbar_init(empty + k); }
+        mbar_init(&done);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    tc_before();
+    __syncthreads();
+    tc_after();
+    // ---- parameters of this thread's row, last written by the kernel before net_kernel, which that one
+    // waited for before it let this one start
+    const int row = ih * 128 + (tid & 127);
+    float pv[32], q1[32], q2[32];
+    const int o0 = w1 ? OFF_W1 + row * NINP : (w3 ? OFF_W3 + row : OFF_W2 + row * NH + jt * 32);
+    if (ADAM && rank == 0 && warp < 4) {
+        if (w3) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) { pv[j] = G.p[o0 + j * NH]; q1[j] = G.m1[o0 + j * NH]; q2[j] = G.m2[o0 + j * NH]; }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+                if (j >= ncol) break;
+                *reinterpret_cast<float4*>(pv + j) = *reinterpret_cast<const float4*>(G.p + o0 + j);
+                *reinterpret_cast<float4*>(q1 + j) = *reinterpret_cast<const float4*>(G.m1 + o0 + j);
+                *reinterpret_cast<float4*>(q2 + j) = *reinterpret_cast<const float4*>(G.m2 + o0 + j);
+            }
         }
     }
-}
-
-// column sums of an FP32 [n][w] matrix (bias gradients), one thread per column
-__global__ void colsum_kernel(const float* D, int n, int w, float* out)
-{
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= w) return;
-    float a = 0.0f;
-    for (int s = 0; s < n; ++s) a += D[(long long)s * w + c];
-    out[c] = a;
-}
-
-__global__ void adam_kernel(float* p, const float* g, float* m1, float* m2, int n, float lr, float c1, float c2)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float a = 0.9f * m1[i] + 0.1f * gi;
-    const float b = 0.999f * m2[i] + 0.001f * gi * gi;
-    m1[i] = a;
-    m2[i] = b;
-    p[i] -= lr * (a * c1) / (sqrtf(b * c2) + 1e-8f);
+    pdl_wait();
+    const unsigned tmem = s_tmem;
+    bool ok = true;
+    if (warp == 4) {
+        // loads: one column group (2 KiB of a tile) per lane
+        const int ng = 16 + ncol / 8;
+        for (int t = t0; t < t1; ++t) {
+            const int st = (t - t0) % GST, use = (t - t0) / GST;
+            if (use > 0 && !mbar_wait(empty + st, (unsigned)(use - 1) & 1u)) { ok = false; break; }
+            unsigned char* d = sm + st * (GS_A + GS_B);
+            if (lane == 0) mbar_expect(full + st, (unsigned)(ng * CS_T));
+            __syncwarp();
+            if (lane < 16) bulk_load(d + lane * CS_T, a + lane * G.act.cs + (long long)t * CS_T, CS_T, full + st);
+            else if (lane < ng) bulk_load(d + GS_A + (lane - 16) * CS_T, b + (lane - 16) * G.act.cs + (long long)t * CS_T, CS_T, full + st);
+        }
+    } else if (tid == 5 * 32) {
+        const unsigned idesc = idesc_bf16(TILE, ncol) | (1u << 15) | (1u << 16);     // both MN-major
+        for (int t = t0; t < t1; ++t) {
+            const int st = (t - t0) % GST, use = (t - t0) / GST;
+            if (!mbar_wait(full + st, (unsigned)use & 1u)) { ok = false; break; }
+            tc_after();
+            const unsigned ad = smem_u32(sm + st * (GS_A + GS_B)), bd = ad + GS_A;
+#pragma unroll
+            for (int k = 0; k < TILE / 16; ++k)
+                mma_bf16(tmem, sdesc(ad + k * 256, 128u, CS_T), sdesc(bd + k * 256, 128u, CS_T), idesc, t > t0 || k > 0);
+            mma_commit(empty + st);
+        }
+        if (ok) mma_commit(&done);
+    }
+    __syncwarp();
+    if (warp < 4 && !mbar_wait(&done, 0u)) ok = false;
+    const bool fail = __syncthreads_or(!ok);
+    tc_after();
+    float v[32];
+    if (!fail && warp < 4) tmem_ld32(tmem + ((unsigned)((warp & 3) * 32) << 16), v);     // 16 of them for dW1
+    if (fail) {
+        if (tid == 0) {
+            atomicOr(&g_gemm_status, 1u);
+            if (G.status) atomicOr(G.status, 1u);
+        }
+        for (int k = 0; k < GST; ++k) (void)mbar_wait(full + k, 0u);
+    }
+    if (nrank > 1) {
+        // the other blocks' parts into the first one's stages: column j of row m at (j * 128 + m) floats
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (rank > 0 && warp < 4) {
+            const unsigned local = smem_u32(sm) + ((rank - 1) * TILE * 32 + (unsigned)tid) * 4u;
+            unsigned remote;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"(local));
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote + j * TILE * 4), "f"(fail ? 0.0f : v[j]) : "memory");
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (rank == 0 && warp < 4) {
+            const float* part = reinterpret_cast<const float*>(sm) + tid;
+            for (unsigned r = 0; r + 1 < nrank; ++r)
+#pragma unroll
+                for (int j = 0; j < 32; ++j) v[j] += part[(r * 32 + j) * TILE];
+        }
+    }
+    if (!fail && rank == 0 && warp < 4) {
+        if (ADAM) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                if (j < ncol) v[j] = adam(pv[j], q1[j], q2[j], v[j], G.lr, G.c1, G.c2);
+            if (w3) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    G.p[o0 + j * NH] = pv[j]; G.m1[o0 + j * NH] = q1[j]; G.m2[o0 + j * NH] = q2[j];
+                    *reinterpret_cast<__nv_bfloat16*>(G.w + PK_W3 + core_at(CS_W3, j, row)) = __float2bfloat16(pv[j]);
+                }
+            } else {
+                unsigned char* w = G.w + (w1 ? PK_W1 : PK_W2);
+#pragma unroll
+                for (int j = 0; j < 32; j += 8) {
+                    if (j >= ncol) break;
+#pragma unroll
+                    for (int t = 0; t < 8; t += 4) {
+                        *reinterpret_cast<float4*>(G.p + o0 + j + t) = *reinterpret_cast<const float4*>(pv + j + t);
+                        *reinterpret_cast<float4*>(G.m1 + o0 + j + t) = *reinterpret_cast<const float4*>(q1 + j + t);
+                        *reinterpret_cast<float4*>(G.m2 + o0 + j + t) = *reinterpret_cast<const float4*>(q2 + j + t);
+                    }
+                    *reinterpret_cast<uint4*>(w + core_at(CS_W12, row, jt * 32 + j)) =
+                        make_uint4(pack2(pv[j], pv[j + 1]), pack2(pv[j + 2], pv[j + 3]), pack2(pv[j + 4], pv[j + 5]), pack2(pv[j + 6], pv[j + 7]));
+                }
+            }
+        } else {
+            const int st = w3 ? NH : 1;
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                if (j < ncol) G.grad[o0 + j * st] = v[j];
+        }
+    }
+    tc_before();
+    __syncthreads();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 32;" ::"r"(tmem) : "memory");
 }
 
 // Cholesky solve of A u = f for one symmetric positive definite 6x6 A (FP64,
@@ -575,20 +1151,11 @@ struct lb_mlp {
     int max_batch = 0;
     long long step = 0;
     float* p = nullptr;                 // FP32 master parameters
-    float* g = nullptr;                 // gradients
     float* m1 = nullptr;                // Adam moments
     float* m2 = nullptr;
     float* loss = nullptr;              // scratch loss for train_step without output
-    __nv_bfloat16* w16 = nullptr;       // BF16 copy of the whole parameter block (W1, W2, W3 used)
-    __nv_bfloat16* X = nullptr;         // [B][16]
-    __nv_bfloat16* H1 = nullptr;        // [B][256]
-    __nv_bfloat16* H2 = nullptr;
-    float* Y = nullptr;                 // [B][32]
-    float* dY32 = nullptr;
-    __nv_bfloat16* dY16 = nullptr;
-    float* dH32 = nullptr;              // [B][256], reused for both hidden layers
-    __nv_bfloat16* dH2 = nullptr;
-    __nv_bfloat16* dH1 = nullptr;
+    unsigned char* w = nullptr;         // BF16 copy of the weights, packed (PK_*)
+    Acts act{};
     std::vector<void*> allocs;
 };
 
@@ -615,70 +1182,48 @@ void mlp_free(lb_mlp* m)
 
 inline unsigned blocks(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
-GemmArgs gemm(const __nv_bfloat16* A, long long a_sm, long long a_sk, const __nv_bfloat16* B, long long b_sn,
-              long long b_sk, int M, int N, int K)
+// forward pass, head and (BWD) the activations' gradients of n samples
+template <bool BWD>
+cudaError_t launch_net(lb_mlp* m, const float* x, int n, const float* Rt, float* y, float* R, float* loss, cudaStream_t s)
 {
-    GemmArgs g{};
-    g.A = A; g.a_sm = a_sm; g.a_sk = a_sk;
-    g.B = B; g.b_sn = b_sn; g.b_sk = b_sk;
-    g.M = M; g.N = N; g.K = K;
-    return g;
+    NetArgs A{};
+    A.x = x; A.p = m->p; A.w = m->w; A.Rt = Rt; A.y_out = y; A.R_out = R; A.loss = loss; A.act = m->act; A.n = n;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks(n, TILE));
+    cfg.blockDim = dim3(NTHREADS);
+    cfg.dynamicSmemBytes = NET_SMEM;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, net_kernel<BWD>, A);
 }
 
-// forward pass of n samples into m->H1, m->H2, m->Y
-cudaError_t forward(lb_mlp* m, const float* x, int n, cudaStream_t s)
+// weight and bias gradients into grad, or (ADAM) the step with learning rate lr
+template <bool ADAM>
+cudaError_t launch_grad(lb_mlp* m, int n, float* grad, float lr, float c1, float c2, float* loss, cudaStream_t s)
 {
-    cudaError_t e;
-    features_kernel<<<blocks((long long)n * NINP, 256), 256, 0, s>>>(x, n, m->X);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    GemmArgs g = gemm(m->X, NINP, 1, m->w16 + OFF_W1, NINP, 1, n, NH, NINP);
-    g.bias = m->p + OFF_B1; g.relu = 1; g.C16 = m->H1; g.c_sm = NH; g.c_sn = 1;
-    if ((e = launch_gemm(g, s)) != cudaSuccess) return e;
-    g = gemm(m->H1, NH, 1, m->w16 + OFF_W2, NH, 1, n, NH, NH);
-    g.bias = m->p + OFF_B2; g.relu = 1; g.C16 = m->H2; g.c_sm = NH; g.c_sn = 1;
-    if ((e = launch_gemm(g, s)) != cudaSuccess) return e;
-    g = gemm(m->H2, NH, 1, m->w16 + OFF_W3, NH, 1, n, NOUTP, NH);
-    g.bias = m->p + OFF_B3; g.C32 = m->Y; g.c_sm = NOUTP; g.c_sn = 1;
-    return launch_gemm(g, s);
-}
-
-// loss and gradients into m->g (after forward); loss accumulated into `loss`
-cudaError_t backward(lb_mlp* m, const float* Rt, int n, float* loss, cudaStream_t s)
-{
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(loss, 0, sizeof(float), s)) != cudaSuccess) return e;
-    head_kernel<<<blocks(n, 128), 128, 0, s>>>(m->Y, n, nullptr, nullptr, Rt, loss, m->dY32, m->dY16);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // layer 3: dW3 = dY^T H2, db3 = sum dY
-    GemmArgs g = gemm(m->dY16, 1, NOUTP, m->H2, 1, NH, NOUTP, NH, n);
-    g.C32 = m->g + OFF_W3; g.c_sm = NH; g.c_sn = 1;
-    if ((e = launch_gemm(g, s)) != cudaSuccess) return e;
-    colsum_kernel<<<1, NOUTP, 0, s>>>(m->dY32, n, NOUTP, m->g + OFF_B3);
-    // dH2 = (dY W3) * [H2 > 0]
-    g = gemm(m->dY16, NOUTP, 1, m->w16 + OFF_W3, 1, NH, n, NH, NOUTP);
-    g.mask = m->H2; g.C32 = m->dH32; g.C16 = m->dH2; g.c_sm = NH; g.c_sn = 1;
-    if ((e = launch_gemm(g, s)) != cudaSuccess) return e;
-    colsum_kernel<<<1, NH, 0, s>>>(m->dH32, n, NH, m->g + OFF_B2);
-    // layer 2: dW2 = dH2^T H1
-    g = gemm(m->dH2, 1, NH, m->H1, 1, NH, NH, NH, n);
-    g.C32 = m->g + OFF_W2; g.c_sm = NH; g.c_sn = 1;
-    if ((e = launch_gemm(g, s)) != cudaSuccess) return e;
-    // dH1 = (dH2 W2) * [H1 > 0]
-    g = gemm(m->dH2, NH, 1, m->w16 + OFF_W2, 1, NH, n, NH, NH);
-    g.mask = m->H1; g.C32 = m->dH32; g.C16 = m->dH1; g.c_sm = NH; g.c_sn = 1;
-    if ((e = launch_gemm(g, s)) != cudaSuccess) return e;
-    colsum_kernel<<<1, NH, 0, s>>>(m->dH32, n, NH, m->g + OFF_B1);
-    // layer 1: dW1 = dH1^T X
-    g = gemm(m->dH1, 1, NH, m->X, 1, NINP, NH, NINP, n);
-    g.C32 = m->g + OFF_W1; g.c_sm = NINP; g.c_sn = 1;
-    if ((e = launch_gemm(g, s)) != cudaSuccess) return e;
-    return cudaGetLastError();
-}
-
-cudaError_t refresh_bf16(lb_mlp* m, cudaStream_t s)
-{
-    to_bf16_kernel<<<blocks(NPARAM, 256), 256, 0, s>>>(m->p, m->w16, NPARAM);
-    return cudaGetLastError();
+    GradArgs G{};
+    G.act = m->act; G.n = n; G.tiles = (int)blocks(n, TILE); G.grad = grad;
+    G.p = m->p; G.m1 = m->m1; G.m2 = m->m2; G.w = m->w; G.lr = lr; G.c1 = c1; G.c2 = c2; G.loss = loss;
+    // above SPLIT_MIN tiles (1,024 samples) each gradient tile is a cluster of SPLIT blocks
+    const int nr = G.tiles > SPLIT_MIN ? SPLIT : 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((GEMM_JOBS + BIAS_JOBS) * nr);
+    cfg.blockDim = dim3(GTHREADS_N);
+    cfg.dynamicSmemBytes = GRAD_SMEM;
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)nr;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, grad_kernel<ADAM>, G);
 }
 
 }  // namespace
@@ -692,17 +1237,26 @@ extern "C" lb_status lb_mlp_create(int32_t device, int32_t max_batch, lb_mlp** o
     if (!m) return LB_ENOMEM;
     m->device = device;
     m->max_batch = max_batch;
-    const size_t B = (size_t)max_batch;
-    bool ok = mlp_alloc(m, &m->p, NPARAM) && mlp_alloc(m, &m->g, NPARAM) && mlp_alloc(m, &m->m1, NPARAM) &&
-              mlp_alloc(m, &m->m2, NPARAM) && mlp_alloc(m, &m->loss, 1) && mlp_alloc(m, &m->w16, NPARAM) &&
-              mlp_alloc(m, &m->X, B * NINP) && mlp_alloc(m, &m->H1, B * NH) && mlp_alloc(m, &m->H2, B * NH) &&
-              mlp_alloc(m, &m->Y, B * NOUTP) && mlp_alloc(m, &m->dY32, B * NOUTP) &&
-              mlp_alloc(m, &m->dY16, B * NOUTP) && mlp_alloc(m, &m->dH32, B * NH) && mlp_alloc(m, &m->dH2, B * NH) &&
-              mlp_alloc(m, &m->dH1, B * NH);
+    const size_t T = blocks(max_batch, TILE), B = T * TILE;      // whole tiles
+    Acts& a = m->act;
+    a.cs = (long long)T * CS_T;
+    a.ns = (int)std::min<size_t>(T, SPLIT_MIN) * TILE;
+    bool ok = mlp_alloc(m, &m->p, NPARAM) && mlp_alloc(m, &m->m1, NPARAM) && mlp_alloc(m, &m->m2, NPARAM) &&
+              mlp_alloc(m, &m->loss, 1) && mlp_alloc(m, &m->w, PK_BYTES) && mlp_alloc(m, &a.X, B * NINP * 2) &&
+              mlp_alloc(m, &a.H1, B * NH * 2) && mlp_alloc(m, &a.H2, B * NH * 2) && mlp_alloc(m, &a.dY, B * NOUTP * 2) &&
+              mlp_alloc(m, &a.dH2, B * NH * 2) && mlp_alloc(m, &a.dH1, B * NH * 2) && mlp_alloc(m, &a.loss_part, T) &&
+              mlp_alloc(m, &a.d32, (size_t)a.ns * NSUM) &&
+              mlp_alloc(m, &a.b_part, 4 * T * NSUM) && mlp_alloc(m, &a.count, 1);
     if (ok) {
-        for (void* q : {(void*)m->p, (void*)m->g, (void*)m->m1, (void*)m->m2})
+        for (void* q : {(void*)m->p, (void*)m->m1, (void*)m->m2})
             ok = ok && cudaMemset(q, 0, NPARAM * sizeof(float)) == cudaSuccess;
-        ok = ok && cudaMemset(m->w16, 0, NPARAM * sizeof(__nv_bfloat16)) == cudaSuccess;
+        ok = ok && cudaMemset(m->w, 0, PK_BYTES) == cudaSuccess && cudaMemset(a.count, 0, sizeof(unsigned)) == cudaSuccess;
+        // the kernels' shared memory on this device
+        const cudaFuncAttribute ds = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        ok = ok && cudaFuncSetAttribute(net_kernel<false>, ds, NET_SMEM) == cudaSuccess &&
+             cudaFuncSetAttribute(net_kernel<true>, ds, NET_SMEM) == cudaSuccess &&
+             cudaFuncSetAttribute(grad_kernel<false>, ds, GRAD_SMEM) == cudaSuccess &&
+             cudaFuncSetAttribute(grad_kernel<true>, ds, GRAD_SMEM) == cudaSuccess;
         ok = ok && cudaDeviceSynchronize() == cudaSuccess;
     }
     if (!ok) {
@@ -738,9 +1292,10 @@ extern "C" lb_status lb_mlp_set_params(lb_mlp* m, const float* host)
     }
     if (cudaMemcpy(m->p, h.data(), NPARAM * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(m->m1, 0, NPARAM * sizeof(float)) != cudaSuccess ||
-        cudaMemset(m->m2, 0, NPARAM * sizeof(float)) != cudaSuccess || refresh_bf16(m, nullptr) != cudaSuccess ||
-        cudaDeviceSynchronize() != cudaSuccess)
+        cudaMemset(m->m2, 0, NPARAM * sizeof(float)) != cudaSuccess)
         return LB_ECUDA;
+    pack_kernel<<<blocks(NPARAM, 256), 256>>>(m->p, m->w);
+    if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) return LB_ECUDA;
     m->step = 0;
     return LB_OK;
 }
@@ -758,10 +1313,10 @@ extern "C" lb_status lb_mlp_get_params(lb_mlp* m, float* host)
 extern "C" lb_status lb_mlp_forward(lb_mlp* m, const float* x_dev, int32_t n, float* y_dev, float* R_dev, void* stream)
 {
     if (!m || !x_dev || n < 1 || n > m->max_batch) return LB_EINVAL;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaSetDevice(m->device) != cudaSuccess || forward(m, x_dev, n, s) != cudaSuccess) return LB_ECUDA;
-    head_kernel<<<blocks(n, 128), 128, 0, s>>>(m->Y, n, y_dev, R_dev, nullptr, nullptr, nullptr, nullptr);
-    return cudaGetLastError() == cudaSuccess ? LB_OK : LB_ECUDA;
+    if (cudaSetDevice(m->device) != cudaSuccess ||
+        launch_net<false>(m, x_dev, n, nullptr, y_dev, R_dev, nullptr, static_cast<cudaStream_t>(stream)) != cudaSuccess)
+        return LB_ECUDA;
+    return LB_OK;
 }
 
 extern "C" lb_status lb_mlp_loss_grad(lb_mlp* m, const float* x_dev, const float* Rt_dev, int32_t n, float* loss_dev,
@@ -769,10 +1324,11 @@ extern "C" lb_status lb_mlp_loss_grad(lb_mlp* m, const float* x_dev, const float
 {
     if (!m || !x_dev || !Rt_dev || !loss_dev || n < 1 || n > m->max_batch) return LB_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaSetDevice(m->device) != cudaSuccess || forward(m, x_dev, n, s) != cudaSuccess ||
-        backward(m, Rt_dev, n, loss_dev, s) != cudaSuccess)
-        return LB_ECUDA;
-    if (grad_dev && cudaMemcpyAsync(grad_dev, m->g, NPARAM * sizeof(float), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+    if (cudaSetDevice(m->device) != cudaSuccess) return LB_ECUDA;
+    if (!grad_dev)                      // the loss alone
+        return launch_net<false>(m, x_dev, n, Rt_dev, nullptr, nullptr, loss_dev, s) == cudaSuccess ? LB_OK : LB_ECUDA;
+    if (launch_net<true>(m, x_dev, n, Rt_dev, nullptr, nullptr, nullptr, s) != cudaSuccess ||
+        launch_grad<false>(m, n, grad_dev, 0.0f, 0.0f, 0.0f, loss_dev, s) != cudaSuccess)
         return LB_ECUDA;
     return LB_OK;
 }
@@ -782,15 +1338,13 @@ extern "C" lb_status lb_mlp_train_step(lb_mlp* m, const float* x_dev, const floa
 {
     if (!m || !x_dev || !Rt_dev || n < 1 || n > m->max_batch || !(lr > 0.0f)) return LB_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaSetDevice(m->device) != cudaSuccess || forward(m, x_dev, n, s) != cudaSuccess ||
-        backward(m, Rt_dev, n, loss_dev ? loss_dev : m->loss, s) != cudaSuccess)
+    if (cudaSetDevice(m->device) != cudaSuccess ||
+        launch_net<true>(m, x_dev, n, Rt_dev, nullptr, nullptr, nullptr, s) != cudaSuccess)
         return LB_ECUDA;
     m->step += 1;
     const float c1 = (float)(1.0 / (1.0 - std::pow(0.9, (double)m->step)));
     const float c2 = (float)(1.0 / (1.0 - std::pow(0.999, (double)m->step)));
-    adam_kernel<<<blocks(NPARAM, 256), 256, 0, s>>>(m->p, m->g, m->m1, m->m2, NPARAM, lr, c1, c2);
-    if (cudaGetLastError() != cudaSuccess || refresh_bf16(m, s) != cudaSuccess) return LB_ECUDA;
-    return LB_OK;
+    return launch_grad<true>(m, n, nullptr, lr, c1, c2, loss_dev ? loss_dev : m->loss, s) == cudaSuccess ? LB_OK : LB_ECUDA;
 }
 
 extern "C" lb_status lb_spd_solve6(const float* R_dev, const double* f_dev, double* u_dev, int32_t n, void* stream)
