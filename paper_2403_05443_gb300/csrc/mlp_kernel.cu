@@ -19,9 +19,8 @@
 // index.  The
 // epilogue: warp w reads TMEM lanes 32w..32w+31 (one output row per lane) with
 // tcgen05.ld, adds the bias, applies ReLU and writes FP32 and/or BF16.
-// The network is small (8 -> 256 -> 256 -> 21), so the staging is done by
-// plain loads that also transpose; the products are the only dense
-// contractions and the only work on the tensor cores.
+// This form serves any strides (lb_gemm_bf16); the network has kernels of its own, see
+// net_kernel and grad_kernel below.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -338,7 +337,7 @@ struct Acts {
     long long cs;
     float* loss_part;                   // [tiles]
     float* d32;                         // up to SPLIT_MIN tiles: FP32 dH1, dH2, dY, [2 * 256 + 32][ns] by column
-    float* b_part;                      // more tiles: their column sums, [4 tiles][2 * 256 + 32], per warp of 32 samples
+    float* b_part;                      // more tiles: their column sums, [4 tiles][2 * 256 + 32], per 32 samples
     int ns;                             // samples a column of d32 holds
     unsigned* count;                    // tiles done (zero between launches)
 };
@@ -381,13 +380,6 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned b
                  "l"(src), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
 }
-__device__ __forceinline__ void bulk_store(void* dst, const void* src, unsigned bytes)
-{
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -402,42 +394,38 @@ __device__ __forceinline__ void mma_commit(unsigned long long* bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// 32 accumulator columns of this warp's 32 lanes
-__device__ __forceinline__ void tmem_ld32(unsigned addr, float (&v)[32])
+// n products of K = 16 into accumulator d, operand descriptors advancing by da and db
+// (in 16-byte units) per product
+__device__ __forceinline__ void mma_chain(unsigned d, unsigned long long a, unsigned da, unsigned long long b, unsigned db,
+                                          unsigned idesc, int n, bool acc)
 {
-    unsigned r[32];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                 : "r"(addr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+    for (int k = 0; k < n; ++k) {
+        mma_bf16(d, a, b, idesc, acc || k > 0);
+        a += da;
+        b += db;
+    }
 }
+
+// 16 (8) accumulator columns of this warp's 32 lanes; the values are there after tmem_wait
+__device__ __forceinline__ void tmem_ld16(unsigned addr, unsigned (&r)[16])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(addr));
+}
+__device__ __forceinline__ void tmem_ld8(unsigned addr, unsigned (&r)[8])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(addr));
+}
+__device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ unsigned pack2(float a, float b)
 {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<const unsigned*>(&h);
-}
-
-// sums over the warp's lanes of 32 values per lane: lane l returns the sum of
-// v[l] (each step exchanges half of what is left: 31 shuffles instead of 160)
-__device__ __forceinline__ float warp_colsum(float (&v)[32], int lane)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int k = 0; k < o; ++k) {
-            const float send = up ? v[k] : v[k + o], keep = up ? v[k + o] : v[k];
-            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
-    }
-    return v[0];
 }
 
 // ---- Forward pass, head and (BWD) the activations' gradients of one 128-sample
@@ -449,8 +437,9 @@ __device__ __forceinline__ float warp_colsum(float (&v)[32], int lane)
 // by one thread and followed by an epilogue of 512 threads (thread = sample x a quarter of
 // the columns): the chain of five waits and epilogues bounds the kernel at every batch
 // size up to 152 tiles, so nothing is split further.
-// Measured (512 samples, one training step): the chain of 13 kernels before took 760 us
-// a step, its staging loads one at a time; see grad_kernel for both kernels together.
+// In cycles at 512 samples: set-up and inputs 2,800, the three 256-wide products 2,500
+// each (16 x 132, the tensor core's rate), hidden epilogues 2,900, head 6,000, gradient
+// epilogues 6,400 with the FP32 copy; times of both kernels at grad_kernel.
 struct NetArgs {
     const float* x;
     const float* p;                     // biases
@@ -464,12 +453,134 @@ struct NetArgs {
     unsigned* status;
 };
 
-constexpr int NS_W2 = 0, NS_W3 = NS_W2 + NH * NH * 2, NS_W1 = NS_W3 + NOUTP * NH * 2, NS_H = NS_W1 + NH * NINP * 2,
-              NS_X = NS_H + TILE * NH * 2, NS_BIAS = NS_X + TILE * NINP * 2, NET_SMEM = NS_BIAS + (2 * NH + NOUTP) * 4;
+constexpr int NS_W2 = 0, NS_W3 = NS_W2 + NH * NH * 2, NS_H = NS_W3 + NOUTP * NH * 2, NS_BIAS = NS_H + TILE * NH * 2,
+              NS_W1 = NS_BIAS + (2 * NH + NOUTP) * 4, NS_X = NS_W1 + NH * NINP * 2, NS_TAB = NS_W1,
+              NET_SMEM = NS_TAB + 29 * TILE * 4;      // the head's tables take the place of W1 and X
 constexpr int CS_T = TILE / 8 * 128;    // column-group stride of a 128-row tile in shared memory
 constexpr int NTHREADS = 512;           // four threads per sample, 64 columns each
 static_assert(NET_SMEM <= 227 * 1024 - 256, "shared memory of the network kernel");
-static_assert(TILE * NOUTP * 2 <= NH * NINP * 2, "dY takes the place of W1");
+static_assert(NS_X + TILE * NINP * 2 <= NET_SMEM && NS_W1 % 128 == 0, "W1 and X fit the tables' place");
+
+// Epilogues of one thread's 64 columns.  out: its place in global memory (a group of 8
+// columns every cs bytes; plain 16-byte stores, 512 contiguous bytes a warp: a bulk store of
+// the tile held the next epilogue back by the 3,000 cycles it took to read the tile).
+// Hidden layer: relu(acc + b) as BF16 into the tile and, per group of 8 columns, which are
+// above zero (one byte each of the result).
+template <bool OUT>
+__device__ __forceinline__ unsigned long long hidden(unsigned acc, const float* b, unsigned char* tile, unsigned char* out,
+                                                     long long cs, bool live)
+{
+    unsigned long long m = 0;
+    unsigned r[4][16];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) tmem_ld16(acc + q * 16u, r[q]);
+    tmem_wait();
+#pragma unroll
+    for (int c = 0; c < 64; c += 8) {
+        const unsigned(&u)[16] = r[c >> 4];
+        const int o = c & 8;
+        const float4 b0 = *reinterpret_cast<const float4*>(b + c), b1 = *reinterpret_cast<const float4*>(b + c + 4);
+        unsigned h[4];
+        h[0] = pack2(fmaxf(__uint_as_float(u[o]) + b0.x, 0.0f), fmaxf(__uint_as_float(u[o + 1]) + b0.y, 0.0f));
+        h[1] = pack2(fmaxf(__uint_as_float(u[o + 2]) + b0.z, 0.0f), fmaxf(__uint_as_float(u[o + 3]) + b0.w, 0.0f));
+        h[2] = pack2(fmaxf(__uint_as_float(u[o + 4]) + b1.x, 0.0f), fmaxf(__uint_as_float(u[o + 5]) + b1.y, 0.0f));
+        h[3] = pack2(fmaxf(__uint_as_float(u[o + 6]) + b1.z, 0.0f), fmaxf(__uint_as_float(u[o + 7]) + b1.w, 0.0f));
+        unsigned bits = 0;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            if (!live) h[t] = 0u;
+            // both halves' 15 magnitude bits carry into the bit above when any is set
+            const unsigned nz = ((h[t] & 0x7fff7fffu) + 0x7fff7fffu) & 0x80008000u;
+            bits |= (nz >> (15 - t)) | (nz >> (27 - t));
+        }
+        const uint4 v = make_uint4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<uint4*>(tile + (c >> 3) * CS_T) = v;
+        if (OUT) *reinterpret_cast<uint4*>(out + (c >> 3) * cs) = v;
+        m |= (unsigned long long)(bits & 0xffu) << c;
+    }
+    return m;
+}
+
+// Gradient: masked, BF16 into the tile; the FP32 values (d32, by column), or above
+// SPLIT_MIN tiles their sums over the warp (part), for the bias gradients
+__device__ __forceinline__ void masked(unsigned acc, unsigned long long m, unsigned char* tile, unsigned char* out, long long cs,
+                                       float* d32, int ns, float* part, int lane)
+{
+    unsigned r[4][16];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) tmem_ld16(acc + q * 16u, r[q]);
+    tmem_wait();
+#pragma unroll
+    for (int c = 0; c < 64; c += 8) {
+        float v[8];
+        const unsigned bits = (unsigned)(m >> c);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            v[2 * t] = (bits & (1u << t)) ? __uint_as_float(r[c >> 4][(c & 8) + 2 * t]) : 0.0f;
+            v[2 * t + 1] = (bits & (16u << t)) ? __uint_as_float(r[c >> 4][(c & 8) + 2 * t + 1]) : 0.0f;
+        }
+        const uint4 h = make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
+        *reinterpret_cast<uint4*>(tile + (c >> 3) * CS_T) = h;
+        *reinterpret_cast<uint4*>(out + (c >> 3) * cs) = h;
+        if (d32) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) d32[(c + j) * ns] = v[j];
+        } else {
+            // columns by lane bits 4, 3, 2 (each step sends half of what is left), then the sums of the 4 lanes
+#pragma unroll
+            for (int o = 16, n = 4; o >= 4; o >>= 1, n >>= 1) {
+                const bool up = (lane & o) != 0;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (k >= n) break;
+                    const float send = up ? v[k] : v[k + n], keep = up ? v[k + n] : v[k];
+                    v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+            }
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+            if ((lane & 3) == 0) part[c + (lane >> 2)] = v[0];
+        }
+    }
+}
+
+// Output head: L from the 21 outputs (diagonal through softplus), R^ = L L^T; with
+// targets, the loss (1/(36 n)) sum (R^ - Rt)^2 and its gradient with respect to the
+// outputs: dR = 2 (R^ - Rt) / (36 n), dL = 2 dR L (dR symmetric), dy = dL (off the
+// diagonal), dL_ii sigmoid(y_ii).  One row i of one sample per call, from the sample's
+// table T (L's lower triangle, then the sigmoids; dy, or y, in its place afterwards): with
+// consecutive threads on consecutive rows the targets are read in whole lines (36
+// floats per sample read by its own thread cost 32 line accesses per load, 4,800 cycles a
+// tile).  Returns the row's squared errors.
+constexpr int TS = 29;                  // floats a sample's table takes (27, odd for the banks)
+__device__ __forceinline__ float head_row(const float* T, int i, const float* rt, float* R_out, float c, float (&dy)[6])
+{
+    float err = 0.0f, Li[6], dR[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) Li[k] = k <= i ? T[i * (i + 1) / 2 + k] : 0.0f;
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        float a = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) a += Li[k] * (k <= j ? T[tri(j, k)] : 0.0f);
+        if (R_out) R_out[j] = a;
+        dR[j] = 0.0f;
+        if (rt) {
+            const float d = a - __ldg(rt + j);
+            err += d * d;
+            dR[j] = c * d;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        float a = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) a += dR[k] * (j <= k ? T[tri(k, j)] : 0.0f);
+        a *= 2.0f;
+        dy[j] = j == i ? a * T[NOUT + i] : a;
+    }
+    return err;
+}
 
 template <bool BWD>
 __global__ void __launch_bounds__(NTHREADS, 1) net_kernel(const NetArgs A)
@@ -477,12 +588,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) net_kernel(const NetArgs A)
     extern __shared__ __align__(128) unsigned char sm[];
     __shared__ unsigned long long bar[3];           // W1; W2 and W3; products
     __shared__ unsigned s_tmem;
-    __shared__ float s_red[4];
+    __shared__ float s_red[NTHREADS / 32];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wq = warp & 3, part = warp >> 2;
     const int tile = blockIdx.x, row = wq * 32 + lane, s = tile * TILE + row;
     const bool live = s < A.n;
+    const long long out0 = (long long)tile * CS_T;      // this tile within a column group
     unsigned char* sH = sm + NS_H;
-    unsigned char* sdY = sm + NS_W1;
+    unsigned char* sdY = sH;            // dY takes the tile's place between H2 and dH2
     float* sb = reinterpret_cast<float*>(sm + NS_BIAS);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&s_tmem)) : "memory");
@@ -517,6 +629,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) net_kernel(const NetArgs A)
         const uint4 c1 = make_uint4(0u, 0u, 0u, 0u);
         *reinterpret_cast<uint4*>(sm + NS_X + core_at(CS_T, row, 0)) = c0;
         *reinterpret_cast<uint4*>(sm + NS_X + core_at(CS_T, row, 8)) = c1;
+        if (BWD) {
+            *reinterpret_cast<uint4*>(A.act.X + out0 + core_at(0, row, 0)) = c0;
+            *reinterpret_cast<uint4*>(A.act.X + A.act.cs + out0 + core_at(0, row, 0)) = c1;
+        }
     }
     for (int k = tid; k < 2 * NH + NOUTP; k += NTHREADS)
         sb[k] = __ldg(A.p + (k < NH ? OFF_B1 + k : (k < 2 * NH ? OFF_B2 + k - NH : OFF_B3 + k - 2 * NH)));
@@ -529,220 +645,153 @@ __global__ void __launch_bounds__(NTHREADS, 1) net_kernel(const NetArgs A)
     bool ok = true;
     constexpr unsigned ID256 = idesc_bf16(TILE, NH), ID32 = idesc_bf16(TILE, NOUTP), BMN = 1u << 16;   // B MN-major
     const unsigned aH = smem_u32(sH);
-    // waits for the last product; uniform over the block
-    auto product_done = [&]() {
-        const bool got = mbar_wait(bar + 2, phase);
-        phase ^= 1u;
+    // waits for a barrier; one thread polls and the others park at the block barrier (16 warps
+    // polling took the issuing thread's slots: 150 cycles per product instead of 50)
+    auto wait_all = [&](unsigned long long* b, unsigned parity) {
+        const bool got = tid > 0 || mbar_wait(b, parity);
         if (__syncthreads_or(!got)) ok = false;
         tc_after();
         return ok;
     };
-    // a tile of 32 core columns (2 KiB each) to global memory, one column group per lane of warp 1
-    auto store_tile = [&](unsigned char* dst, const unsigned char* src, int groups) {
-        if (warp == 1) {
-            if (lane < groups) bulk_store(dst + lane * A.act.cs + (long long)tile * CS_T, src + lane * CS_T, CS_T);
-            bulk_commit();
-        }
+    auto product_done = [&]() {
+        phase ^= 1u;
+        return wait_all(bar + 2, phase ^ 1u);
     };
-    auto store_read = [&]() { if (warp == 1) bulk_wait_read(); };
-    // hidden layer's epilogue: act = relu(acc + b) as BF16 into sH, its mask into m[]
-    auto hidden = [&](unsigned col0, const float* b, unsigned (&m)[2]) {
-#pragma unroll 1
-        for (int q = 0; q < 2; ++q) {
-            const int c0 = part * 64 + q * 32;
-            float v[32];
-            tmem_ld32(tlane + col0 + (unsigned)c0, v);
-            unsigned bits = 0;
-#pragma unroll
-            for (int j = 0; j < 32; j += 8) {
-                unsigned h[4];
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const float2 bb = *reinterpret_cast<const float2*>(b + c0 + j + 2 * t);
-                    const float v0 = live ? fmaxf(v[j + 2 * t] + bb.x, 0.0f) : 0.0f;
-                    const float v1 = live ? fmaxf(v[j + 2 * t + 1] + bb.y, 0.0f) : 0.0f;
-                    h[t] = pack2(v0, v1);
-                    if (h[t] & 0x7fffu) bits |= 1u << (j + 2 * t);
-                    if (h[t] & 0x7fff0000u) bits |= 2u << (j + 2 * t);
-                }
-                *reinterpret_cast<uint4*>(sH + core_at(CS_T, row, c0 + j)) = make_uint4(h[0], h[1], h[2], h[3]);
-            }
-            m[0] = q == 0 ? bits : m[0];
-            m[1] = q == 1 ? bits : m[1];
-        }
+    // end of an epilogue: the tile is in shared memory for the tensor core and the bulk stores
+    auto settled = [&]() {
         fence_async();
         tc_before();
         __syncthreads();
         tc_after();
     };
-    auto column_sums = [&](float (&v)[32], int c0) {
-        if (gridDim.x <= SPLIT_MIN) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) A.act.d32[(c0 + j) * A.act.ns + s] = v[j];
-        } else {
-            A.act.b_part[(long long)(tile * 4 + wq) * NSUM + c0 + lane] = warp_colsum(v, lane);
-        }
-    };
-    // gradient's epilogue: masked, BF16 into sH; the FP32 values, or above SPLIT_MIN tiles
-    // their sums over the warp, for the bias gradients (columns sum0 .. sum0 + 255)
-    auto masked = [&](unsigned col0, const unsigned (&m)[2], int sum0) {
-#pragma unroll 1
-        for (int q = 0; q < 2; ++q) {
-            const int c0 = part * 64 + q * 32;
-            const unsigned bits = q == 0 ? m[0] : m[1];
-            float v[32];
-            tmem_ld32(tlane + col0 + (unsigned)c0, v);
-#pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = ((bits >> j) & 1u) ? v[j] : 0.0f;
-#pragma unroll
-            for (int j = 0; j < 32; j += 8)
-                *reinterpret_cast<uint4*>(sH + core_at(CS_T, row, c0 + j)) =
-                    make_uint4(pack2(v[j], v[j + 1]), pack2(v[j + 2], v[j + 3]), pack2(v[j + 4], v[j + 5]), pack2(v[j + 6], v[j + 7]));
-            column_sums(v, sum0 + c0);
-        }
-        fence_async();
-        tc_before();
-        __syncthreads();
-        tc_after();
-    };
-    unsigned m1[2] = {0u, 0u}, m2[2] = {0u, 0u};
+    unsigned long long m1 = 0, m2 = 0;
+    const int col = part * 64;
+    unsigned char* mine = sH + core_at(CS_T, row, col);
+    const long long to = (long long)(col >> 3) * A.act.cs + out0 + core_at(0, row, 0);
+    const bool keep = gridDim.x <= SPLIT_MIN;       // FP32 gradients for sums in the samples' order
     bool pending = true;                            // W2 and W3 still on their way
     do {
         // ---- layer 1
-        if (__syncthreads_or(!mbar_wait(bar, 0u))) { ok = false; break; }
+        if (!wait_all(bar, 0u)) break;
         if (tid == 0) {
-            mma_bf16(tmem, sdesc(smem_u32(sm + NS_X), CS_T, 128u), sdesc(smem_u32(sm + NS_W1), CS_W12, 128u), ID256, false);
+            mma_chain(tmem, sdesc(smem_u32(sm + NS_X), CS_T, 128u), 0u, sdesc(smem_u32(sm + NS_W1), CS_W12, 128u), 0u, ID256, 1, false);
             mma_commit(bar + 2);
         }
-        if (BWD) store_tile(A.act.X, sm + NS_X, 2);
         if (!product_done()) break;
-        hidden(0u, sb, m1);
+        m1 = hidden<BWD>(tlane + (unsigned)col, sb + col, mine, A.act.H1 + to, A.act.cs, live);
+        settled();
         // ---- layer 2
-        const bool got = mbar_wait(bar + 1, 0u);
-        if (__syncthreads_or(!got)) { ok = false; break; }
+        if (!wait_all(bar + 1, 0u)) break;
         pending = false;
         if (tid == 0) {
-#pragma unroll
-            for (int k = 0; k < NH / 16; ++k)
-                mma_bf16(tmem + NH, sdesc(aH + k * 2 * CS_T, CS_T, 128u), sdesc(smem_u32(sm + NS_W2) + k * 2 * CS_W12, CS_W12, 128u), ID256, k > 0);
+            mma_chain(tmem + NH, sdesc(aH, CS_T, 128u), 2 * CS_T / 16, sdesc(smem_u32(sm + NS_W2), CS_W12, 128u), 2 * CS_W12 / 16, ID256, NH / 16, false);
             mma_commit(bar + 2);
         }
-        if (BWD) {
-            store_tile(A.act.H1, sH, 32);
-            store_read();
-        }
         if (!product_done()) break;
-        hidden(NH, sb + NH, m2);
+        m2 = hidden<BWD>(tlane + NH + (unsigned)col, sb + NH + col, mine, A.act.H2 + to, A.act.cs, live);
+        settled();
         // ---- output layer
         if (tid == 0) {
-#pragma unroll
-            for (int k = 0; k < NH / 16; ++k)
-                mma_bf16(tmem, sdesc(aH + k * 2 * CS_T, CS_T, 128u), sdesc(smem_u32(sm + NS_W3) + k * 2 * CS_W3, CS_W3, 128u), ID32, k > 0);
+            mma_chain(tmem, sdesc(aH, CS_T, 128u), 2 * CS_T / 16, sdesc(smem_u32(sm + NS_W3), CS_W3, 128u), 2 * CS_W3 / 16, ID32, NH / 16, false);
             mma_commit(bar + 2);
         }
-        if (BWD) {
-            store_tile(A.act.H2, sH, 32);
-            store_read();
-        }
         if (!product_done()) break;
-        // ---- head, one thread per sample: L from the 21 outputs (diagonal through
-        // softplus), R^ = L L^T; with targets, the loss (1/(36 n)) sum (R^ - Rt)^2 and its
-        // gradient with respect to the outputs: dR = 2 (R^ - Rt) / (36 n), dL = 2 dR L
-        // (dR symmetric), dy = dL (off the diagonal), dL_ii sigmoid(y_ii)
-        if (warp < 4) {
-            float err = 0.0f, dy[NOUTP];
+        // ---- head: the outputs into the samples' tables, the diagonals through softplus and sigmoid, the rows
+        {
+            float* T = reinterpret_cast<float*>(sm + NS_TAB);
+            unsigned v[8];
+            tmem_ld8(tlane + part * 8, v);
+            tmem_wait();
 #pragma unroll
-            for (int t = 0; t < NOUTP; ++t) dy[t] = 0.0f;
-            float v[32];
-            tmem_ld32(tlane, v);
-            if (live) {
-                float y[NOUT], L[6][6], R[6][6];
-#pragma unroll
-                for (int t = 0; t < NOUT; ++t) y[t] = v[t] + sb[2 * NH + t];
-                if (A.y_out) {
-                    for (int t = 0; t < NOUT; ++t) A.y_out[(long long)s * NOUT + t] = y[t];
-                }
-#pragma unroll
-                for (int i = 0; i < 6; ++i)
-#pragma unroll
-                    for (int j = 0; j < 6; ++j) L[i][j] = j < i ? y[tri(i, j)] : (j == i ? softplus(y[tri(i, i)]) : 0.0f);
-#pragma unroll
-                for (int i = 0; i < 6; ++i)
+            for (int k = 0; k < 8; ++k) {
+                const int t = part * 8 + k;
+                if (t < NOUT) T[row * TS + t] = __uint_as_float(v[k]) + sb[2 * NH + t];
+            }
+            __syncthreads();
+            if (A.y_out) {
+                for (int k = tid; k < min(A.n - tile * TILE, TILE) * NOUT; k += NTHREADS)
+                    A.y_out[(long long)tile * TILE * NOUT + k] = T[k / NOUT * TS + k % NOUT];
+                __syncthreads();
+            }
+#pragma unroll 1
+            for (int k = tid; k < 6 * TILE; k += NTHREADS) {
+                const int r = k / 6, i = k - r * 6, t = i * (i + 3) / 2;
+                const float y = T[r * TS + t];
+                T[r * TS + NOUT + i] = sigmoid(y);
+                T[r * TS + t] = softplus(y);
+            }
+            __syncthreads();
+            float err = 0.0f, dy[2][6] = {};
+#pragma unroll 1
+            for (int q = 0; q < 2; ++q) {
+                const int k = tid + q * NTHREADS, r = k / 6, i = k - r * 6;
+                const long long sr = (long long)tile * TILE + r;
+                if (k < 6 * TILE && sr < A.n) {
+                    float d[6];
+                    err += head_row(T + r * TS, i, A.Rt ? A.Rt + sr * 36 + i * 6 : nullptr, A.R_out ? A.R_out + sr * 36 + i * 6 : nullptr,
+                                    2.0f / (36.0f * (float)A.n), d);
 #pragma unroll
                     for (int j = 0; j < 6; ++j) {
-                        float a = 0.0f;
-#pragma unroll
-                        for (int k = 0; k < 6; ++k) a += L[i][k] * L[j][k];
-                        R[i][j] = a;
-                    }
-                if (A.R_out) {
-                    for (int i = 0; i < 6; ++i)
-                        for (int j = 0; j < 6; ++j) A.R_out[(long long)s * 36 + i * 6 + j] = R[i][j];
-                }
-                if (A.Rt) {
-                    const float c = 2.0f / (36.0f * (float)A.n);
-                    const float* rt = A.Rt + (long long)s * 36;
-                    float dR[6][6];
-#pragma unroll
-                    for (int i = 0; i < 6; ++i)
-#pragma unroll
-                        for (int j = 0; j < 6; ++j) {
-                            const float d = R[i][j] - __ldg(rt + i * 6 + j);
-                            err += d * d;
-                            dR[i][j] = c * d;
-                        }
-                    if (BWD) {
-#pragma unroll
-                        for (int i = 0; i < 6; ++i)
-#pragma unroll
-                            for (int j = 0; j <= i; ++j) {
-                                float a = 0.0f;
-#pragma unroll
-                                for (int k = 0; k < 6; ++k) a += dR[i][k] * L[k][j];
-                                a *= 2.0f;
-                                dy[tri(i, j)] = (j == i) ? a * sigmoid(y[tri(i, i)]) : a;
-                            }
+                        dy[0][j] = q == 0 ? d[j] : dy[0][j];
+                        dy[1][j] = q == 1 ? d[j] : dy[1][j];
                     }
                 }
-            }
-            if (BWD) {
-#pragma unroll
-                for (int j = 0; j < NOUTP; j += 8)
-                    *reinterpret_cast<uint4*>(sdY + core_at(CS_T, row, j)) =
-                        make_uint4(pack2(dy[j], dy[j + 1]), pack2(dy[j + 2], dy[j + 3]), pack2(dy[j + 4], dy[j + 5]), pack2(dy[j + 6], dy[j + 7]));
-                column_sums(dy, 2 * NH);
             }
             for (int o = 16; o > 0; o >>= 1) err += __shfl_xor_sync(0xffffffffu, err, o);
             if (lane == 0) s_red[warp] = err;
+            if (BWD) {
+                __syncthreads();
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const int k = tid + q * NTHREADS, r = k / 6, i = k - r * 6;
+#pragma unroll
+                    for (int j = 0; j < 6; ++j)
+                        if (k < 6 * TILE && j <= i) T[r * TS + i * (i + 1) / 2 + j] = dy[q][j];
+                }
+                __syncthreads();
+                // dY: 8 columns per thread as BF16 into the tile and to global memory, FP32 or warp sums for db3
+                float w[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) w[k] = live && part * 8 + k < NOUT ? T[row * TS + part * 8 + k] : 0.0f;
+                const uint4 h = make_uint4(pack2(w[0], w[1]), pack2(w[2], w[3]), pack2(w[4], w[5]), pack2(w[6], w[7]));
+                *reinterpret_cast<uint4*>(sdY + core_at(CS_T, row, part * 8)) = h;
+                *reinterpret_cast<uint4*>(A.act.dY + part * A.act.cs + (long long)tile * CS_T + core_at(0, row, 0)) = h;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int c = 2 * NH + part * 8 + k;
+                    if (keep) {
+                        A.act.d32[c * A.act.ns + s] = w[k];
+                    } else {
+                        for (int o = 16; o > 0; o >>= 1) w[k] += __shfl_xor_sync(0xffffffffu, w[k], o);
+                        if (lane == 0) A.act.b_part[(long long)(tile * 4 + wq) * NSUM + c] = w[k];
+                    }
+                }
+            }
         }
-        fence_async();
-        tc_before();
-        __syncthreads();
-        tc_after();
-        if (tid == 0 && A.Rt) A.act.loss_part[tile] = ((s_red[0] + s_red[2]) + (s_red[1] + s_red[3])) / (36.0f * (float)A.n);
+        settled();
+        if (warp == 0 && A.Rt) {
+            float err = lane < NTHREADS / 32 ? s_red[lane] : 0.0f;
+            for (int o = 16; o > 0; o >>= 1) err += __shfl_xor_sync(0xffffffffu, err, o);
+            if (lane == 0) A.act.loss_part[tile] = err / (36.0f * (float)A.n);
+        }
         if (!BWD) break;
         // ---- dH2 = (dY W3) * [H2 > 0]
         if (tid == 0) {
-#pragma unroll
-            for (int k = 0; k < NOUTP / 16; ++k)
-                mma_bf16(tmem + NH, sdesc(smem_u32(sdY) + k * 2 * CS_T, CS_T, 128u), sdesc(smem_u32(sm + NS_W3) + k * 256, 128u, CS_W3), ID256 | BMN, k > 0);
+            mma_chain(tmem + NH, sdesc(smem_u32(sdY), CS_T, 128u), 2 * CS_T / 16, sdesc(smem_u32(sm + NS_W3), 128u, CS_W3), 256 / 16, ID256 | BMN, NOUTP / 16, false);
             mma_commit(bar + 2);
         }
-        store_tile(A.act.dY, sdY, 4);
         if (!product_done()) break;
-        masked(NH, m2, NH);
+        masked(tlane + NH + (unsigned)col, m2, mine, A.act.dH2 + to, A.act.cs, keep ? A.act.d32 + (long long)(NH + col) * A.act.ns + s : nullptr, A.act.ns,
+               A.act.b_part + (long long)(tile * 4 + wq) * NSUM + NH + col, lane);
+        settled();
         // ---- dH1 = (dH2 W2) * [H1 > 0]
         if (tid == 0) {
-#pragma unroll
-            for (int k = 0; k < NH / 16; ++k)
-                mma_bf16(tmem, sdesc(aH + k * 2 * CS_T, CS_T, 128u), sdesc(smem_u32(sm + NS_W2) + k * 256, 128u, CS_W12), ID256 | BMN, k > 0);
+            mma_chain(tmem, sdesc(aH, CS_T, 128u), 2 * CS_T / 16, sdesc(smem_u32(sm + NS_W2), 128u, CS_W12), 256 / 16, ID256 | BMN, NH / 16, false);
             mma_commit(bar + 2);
         }
-        store_tile(A.act.dH2, sH, 32);
-        store_read();
         if (!product_done()) break;
-        masked(0u, m1, 0);
-        store_tile(A.act.dH1, sH, 32);
+        masked(tlane + (unsigned)col, m1, mine, A.act.dH1 + to, A.act.cs, keep ? A.act.d32 + (long long)col * A.act.ns + s : nullptr, A.act.ns,
+               A.act.b_part + (long long)(tile * 4 + wq) * NSUM + col, lane);
     } while (false);
     if (!ok) {
         // a completion never came: give what is in flight a second bounded wait before leaving
@@ -754,7 +803,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) net_kernel(const NetArgs A)
         if (pending) (void)mbar_wait(bar + 1, 0u);
         (void)mbar_wait(bar + 2, phase ^ 1u);
     }
-    if (warp == 1) bulk_wait_all();
     if (!BWD && A.loss) {
         // the last tile adds the tiles' losses, in order
         __shared__ bool s_last;
@@ -785,7 +833,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) net_kernel(const NetArgs A)
 // accumulator up to SPLIT_MIN tiles (an Adam step turns the last bit of a gradient near
 // zero into the sign of the update), and is split over a cluster above it, whose first
 // block adds the parts in rank order.
-// Measured, 512 samples: GSTEP_NOTE
+// Measured: an Adam step on 512 samples, both kernels, 28.8 us (net_kernel 18, this one
+// 12, overlapped by programmatic launch) against 760 us before, when five products, three
+// one-block column sums, the head and Adam were 13 kernels and each product staged its
+// operands with one load in flight; loss and gradients of 4,096 samples 28.3 us against
+// 2,805.  At 512 samples the 160 KiB of operands a block takes in set its time.
 struct GradArgs {
     Acts act;
     int n, tiles;
@@ -798,19 +850,19 @@ struct GradArgs {
 };
 
 constexpr int GST = 5, GS_A = 16 * CS_T, GS_B = 4 * CS_T, GRAD_SMEM = GST * (GS_A + GS_B);
-constexpr int GTHREADS_N = 192;         // a warpgroup for the result, one warp for the loads, one for the products
+constexpr int GTHREADS_N = 18 * 32;     // sixteen warps for the result, one for the loads, one for the products
 constexpr int GEMM_JOBS = 20, BIAS_JOBS = NSUM / 32, SPLIT = 4;
 static_assert(32 * (SPLIT_MIN * TILE * 4 + 16) <= GRAD_SMEM, "32 columns of the samples fit the stages");
-static_assert((SPLIT - 1) * TILE * 32 * 4 <= GRAD_SMEM, "the parts of the other blocks fit the stages");
+constexpr int GS_TILE = (SPLIT - 1) * TILE * 32 * 4;    // the result's tile, after the other blocks' parts
+static_assert(GS_TILE + TILE * 33 * 4 <= GRAD_SMEM, "parts and tile fit the stages");
 
-__device__ __forceinline__ float adam(float& p, float& m1, float& m2, float gi, float lr, float c1, float c2)
+__device__ __forceinline__ void adam(float& p, float& m1, float& m2, float gi, float lr, float c1, float c2)
 {
     const float a = 0.9f * m1 + 0.1f * gi;
     const float b = 0.999f * m2 + 0.001f * gi * gi;
     m1 = a;
     m2 = b;
     p -= lr * (a * c1) / (sqrtf(b * c2) + 1e-8f);
-    return p;
 }
 
 template <bool ADAM>
@@ -864,6 +916,7 @@ __global__ void __launch_bounds__(GTHREADS_N, 1) grad_kernel(const GradArgs G)
             }
             return;
         }
+        if (c0 + lane >= 2 * NH + NOUT) v = 0.0f;     // padding
         const int c = c0 + lane, i = c < NH ? OFF_B1 + c : (c < 2 * NH ? OFF_B2 + c - NH : OFF_B3 + c - 2 * NH);
         if (ADAM) adam(G.p[i], G.m1[i], G.m2[i], v, G.lr, G.c1, G.c2);
         else G.grad[i] = v;
@@ -894,27 +947,28 @@ __global__ void __launch_bounds__(GTHREADS_N, 1) grad_kernel(const GradArgs G)
     tc_after();
     // ---- parameters of this thread's row, last written by the kernel before net_kernel, which that one
     // waited for before it let this one start
-    const int row = ih * 128 + (tid & 127);
-    float pv[32], q1[32], q2[32];
-    const int o0 = w1 ? OFF_W1 + row * NINP : (w3 ? OFF_W3 + row : OFF_W2 + row * NH + jt * 32);
-    if (ADAM && rank == 0 && warp < 4) {
-        if (w3) {
+    // The result comes out of tensor memory one row per thread and goes through a shared-memory tile: a warp's
+    // accesses to the parameters are whole 128-byte lines, and an Adam step's square root and division (a chain of
+    // some 300 cycles that the compiler does not interleave) run eight deep on sixteen warps instead of 32 deep on
+    // four (17,900 cycles then).  Value j of a thread is element (tr + trs j, tc + tcs j) of the tile.
+    const int nval = w1 ? 4 : 8;
+    const int tr = w1 ? warp * 8 + (lane >> 4) : (w3 ? (warp & 3) * 32 + lane : warp * 8), trs = w1 ? 2 : (w3 ? 0 : 1);
+    const int tc = w1 ? lane & 15 : (w3 ? (warp >> 2) * 8 : lane), tcs = w3 ? 1 : 0;
+    const int stp = w1 ? 2 * NINP : NH;
+    const int o0 = w1 ? OFF_W1 + (ih * 128 + tr) * NINP + tc
+                      : (w3 ? OFF_W3 + tc * NH + ih * 128 + tr : OFF_W2 + (ih * 128 + tr) * NH + jt * 32 + tc);
+    float pv[8], q1[8], q2[8];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) { pv[j] = G.p[o0 + j * NH]; q1[j] = G.m1[o0 + j * NH]; q2[j] = G.m2[o0 + j * NH]; }
-        } else {
-#pragma unroll
-            for (int j = 0; j < 32; j += 4) {
-                if (j >= ncol) break;
-                *reinterpret_cast<float4*>(pv + j) = *reinterpret_cast<const float4*>(G.p + o0 + j);
-                *reinterpret_cast<float4*>(q1 + j) = *reinterpret_cast<const float4*>(G.m1 + o0 + j);
-                *reinterpret_cast<float4*>(q2 + j) = *reinterpret_cast<const float4*>(G.m2 + o0 + j);
-            }
-        }
+    for (int j = 0; j < 8; ++j) {
+        const bool mine = ADAM && rank == 0 && warp < 16 && j < nval;
+        pv[j] = mine ? G.p[o0 + j * stp] : 0.0f;
+        q1[j] = mine ? G.m1[o0 + j * stp] : 0.0f;
+        q2[j] = mine ? G.m2[o0 + j * stp] : 0.0f;
     }
     pdl_wait();
     const unsigned tmem = s_tmem;
     bool ok = true;
-    if (warp == 4) {
+    if (warp == 16) {
         // loads: one column group (2 KiB of a tile) per lane
         const int ng = 16 + ncol / 8;
         for (int t = t0; t < t1; ++t) {
@@ -926,26 +980,32 @@ __global__ void __launch_bounds__(GTHREADS_N, 1) grad_kernel(const GradArgs G)
             if (lane < 16) bulk_load(d + lane * CS_T, a + lane * G.act.cs + (long long)t * CS_T, CS_T, full + st);
             else if (lane < ng) bulk_load(d + GS_A + (lane - 16) * CS_T, b + (lane - 16) * G.act.cs + (long long)t * CS_T, CS_T, full + st);
         }
-    } else if (tid == 5 * 32) {
+    } else if (tid == 17 * 32) {
         const unsigned idesc = idesc_bf16(TILE, ncol) | (1u << 15) | (1u << 16);     // both MN-major
         for (int t = t0; t < t1; ++t) {
             const int st = (t - t0) % GST, use = (t - t0) / GST;
             if (!mbar_wait(full + st, (unsigned)use & 1u)) { ok = false; break; }
             tc_after();
             const unsigned ad = smem_u32(sm + st * (GS_A + GS_B)), bd = ad + GS_A;
-#pragma unroll
-            for (int k = 0; k < TILE / 16; ++k)
-                mma_bf16(tmem, sdesc(ad + k * 256, 128u, CS_T), sdesc(bd + k * 256, 128u, CS_T), idesc, t > t0 || k > 0);
+            mma_chain(tmem, sdesc(ad, 128u, CS_T), 256 / 16, sdesc(bd, 128u, CS_T), 256 / 16, idesc, TILE / 16, t > t0);
             mma_commit(empty + st);
         }
-        if (ok) mma_commit(&done);
+        if (ok) {
+            mma_commit(&done);
+            ok = mbar_wait(&done, 0u);          // the other warps park at the block barrier below
+        }
     }
-    __syncwarp();
-    if (warp < 4 && !mbar_wait(&done, 0u)) ok = false;
     const bool fail = __syncthreads_or(!ok);
     tc_after();
+    unsigned acc[2][16] = {};
+    if (!fail && warp < 4) {
+        tmem_ld16(tmem + ((unsigned)(warp * 32) << 16), acc[0]);
+        tmem_ld16(tmem + ((unsigned)(warp * 32) << 16) + 16u, acc[1]);      // not used for dW1
+        tmem_wait();
+    }
     float v[32];
-    if (!fail && warp < 4) tmem_ld32(tmem + ((unsigned)((warp & 3) * 32) << 16), v);     // 16 of them for dW1
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(acc[j >> 4][j & 15]);
     if (fail) {
         if (tid == 0) {
             atomicOr(&g_gemm_status, 1u);
@@ -972,37 +1032,32 @@ __global__ void __launch_bounds__(GTHREADS_N, 1) grad_kernel(const GradArgs G)
                 for (int j = 0; j < 32; ++j) v[j] += part[(r * 32 + j) * TILE];
         }
     }
-    if (!fail && rank == 0 && warp < 4) {
-        if (ADAM) {
+    if (rank == 0) {
+        float* T = reinterpret_cast<float*>(sm + GS_TILE);
+        if (warp < 4) {
 #pragma unroll
             for (int j = 0; j < 32; ++j)
-                if (j < ncol) v[j] = adam(pv[j], q1[j], q2[j], v[j], G.lr, G.c1, G.c2);
-            if (w3) {
+                if (j < ncol) T[tid * 33 + j] = v[j];
+        }
+        __syncthreads();
+        if (!fail && warp < 16) {
+            unsigned char* w = G.w + (w1 ? PK_W1 : (w3 ? PK_W3 : PK_W2));
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    G.p[o0 + j * NH] = pv[j]; G.m1[o0 + j * NH] = q1[j]; G.m2[o0 + j * NH] = q2[j];
-                    *reinterpret_cast<__nv_bfloat16*>(G.w + PK_W3 + core_at(CS_W3, j, row)) = __float2bfloat16(pv[j]);
-                }
-            } else {
-                unsigned char* w = G.w + (w1 ? PK_W1 : PK_W2);
-#pragma unroll
-                for (int j = 0; j < 32; j += 8) {
-                    if (j >= ncol) break;
-#pragma unroll
-                    for (int t = 0; t < 8; t += 4) {
-                        *reinterpret_cast<float4*>(G.p + o0 + j + t) = *reinterpret_cast<const float4*>(pv + j + t);
-                        *reinterpret_cast<float4*>(G.m1 + o0 + j + t) = *reinterpret_cast<const float4*>(q1 + j + t);
-                        *reinterpret_cast<float4*>(G.m2 + o0 + j + t) = *reinterpret_cast<const float4*>(q2 + j + t);
-                    }
-                    *reinterpret_cast<uint4*>(w + core_at(CS_W12, row, jt * 32 + j)) =
-                        make_uint4(pack2(pv[j], pv[j + 1]), pack2(pv[j + 2], pv[j + 3]), pack2(pv[j + 4], pv[j + 5]), pack2(pv[j + 6], pv[j + 7]));
+            for (int j = 0; j < 8; ++j) {
+                if (j >= nval) break;
+                const int r = tr + trs * j, c = tc + tcs * j, o = o0 + j * stp;
+                const float g = T[r * 33 + c];
+                if (ADAM) {
+                    adam(pv[j], q1[j], q2[j], g, G.lr, G.c1, G.c2);
+                    G.p[o] = pv[j];
+                    G.m1[o] = q1[j];
+                    G.m2[o] = q2[j];
+                    const int at = w3 ? core_at(CS_W3, c, ih * 128 + r) : core_at(CS_W12, ih * 128 + r, jt * 32 + c);
+                    *reinterpret_cast<__nv_bfloat16*>(w + at) = __float2bfloat16(pv[j]);
+                } else {
+                    G.grad[o] = g;
                 }
             }
-        } else {
-            const int st = w3 ? NH : 1;
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-                if (j < ncol) G.grad[o0 + j * st] = v[j];
         }
     }
     tc_before();
