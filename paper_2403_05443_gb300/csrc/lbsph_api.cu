@@ -36,8 +36,8 @@ cudaError_t launch_links(const PartDev* pd, const PartK* pk, const uint64_t* row
 cudaError_t launch_init_fluid(const BoxDev& B, int precision, void* fbuf, const float* u, const float* drho,
                               const int* owner, float tau, int stress, cudaStream_t s);
 cudaError_t launch_stokes(const BoxDev& B, const int* owner, const PartDev* pd, int np, int counter_on,
-                          const double body[3], float2* work, int* counts, double* sum, float* u,
-                          cudaStream_t s);
+                          const double body[3], float2* z, int* shell, int* counts, float* table, double* sum,
+                          float* u, float* drho, cudaStream_t s);
 }  // namespace lbsph
 
 using namespace lbsph;
@@ -70,8 +70,8 @@ struct lb_ctx {
     int links_cap = 0;
     int* d_count = nullptr;
     float* d_tmp = nullptr;
-    float2* d_stokes = nullptr;         // lb_stokes_field: two complex [3][N] buffers of the largest box
-    int* d_counts = nullptr;
+    float2* d_stokes = nullptr;         // lb_stokes_field: complex [2][N] and int [N] of the largest box
+    double* d_sums = nullptr;           // its sums, shifts and counters, then node counts and force values per particle
     double* d_rec = nullptr;
     size_t tmp_bytes = 0;
     bool collided = false;
@@ -1286,12 +1286,18 @@ extern "C" lb_status lb_init_fluid(lb_ctx* ctx, int32_t box, const float* u, siz
     }
     float* ud = ctx->d_tmp + B.N;                      // [3][N] after the owner field, then drho [N]
     float* dd = drho ? ctx->d_tmp + 4 * B.N : nullptr;
-    const cudaMemcpyKind kind = is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     CK(cudaStreamWaitEvent(s, ctx->ev_done, 0));
-    CK(cudaMemcpyAsync(ud, u, u_bytes, kind, s));
-    if (dd) CK(cudaMemcpyAsync(dd, drho, (size_t)B.N * sizeof(float), kind, s));
+    const float *us = ud, *ds = dd;
+    if (is_device && ((uintptr_t)u | (uintptr_t)drho) % sizeof(float) == 0) {
+        us = u;                                        // read where they are
+        ds = drho;
+    } else {
+        const cudaMemcpyKind kind = is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+        CK(cudaMemcpyAsync(ud, u, u_bytes, kind, s));
+        if (dd) CK(cudaMemcpyAsync(dd, drho, (size_t)B.N * sizeof(float), kind, s));
+    }
     CK(owner_field(ctx, box, s));
-    CK(launch_init_fluid(B, ctx->opt.precision, ctx->fbuf[ctx->cur], ud, dd, reinterpret_cast<int*>(ctx->d_tmp),
+    CK(launch_init_fluid(B, ctx->opt.precision, ctx->fbuf[ctx->cur], us, ds, reinterpret_cast<int*>(ctx->d_tmp),
                          (float)ctx->desc[box].tau, with_stress != 0, s));
     CK(cudaStreamSynchronize(s));
     return read_status(ctx);
@@ -1316,19 +1322,25 @@ extern "C" lb_status lb_stokes_field(lb_ctx* ctx, int32_t box, float* u_dev, flo
     if (!ctx->d_stokes) {
         long long nmax = 0;
         for (auto& h : ctx->hbox) nmax = std::max(nmax, h.N);
-        ctx->d_stokes = (float2*)dev_alloc(ctx, sizeof(float2) * 8 * (size_t)nmax);
-        // np + 1 counts, then (8-byte aligned) 4 double sums
-        ctx->d_counts = (int*)dev_alloc(ctx, sizeof(double) * ((size_t)(ctx->maxp + 2) / 2 + 4));
-        if (!ctx->d_stokes || !ctx->d_counts) return fail(ctx, LB_ENOMEM, "Stokes work buffers");
+        ctx->d_stokes = (float2*)dev_alloc(ctx, (2 * sizeof(float2) + sizeof(int)) * (size_t)nmax);
+        // 4 sums, 4 shifts, 2 counters (8 doubles' room), np + 1 counts, 3 (np + 1) force values
+        ctx->d_sums = (double*)dev_alloc(ctx, 8 * sizeof(double) + 4 * sizeof(int) * ((size_t)ctx->maxp + 1));
+        if (!ctx->d_stokes || !ctx->d_sums) return fail(ctx, LB_ENOMEM, "Stokes work buffers");
     }
     CK(cudaStreamWaitEvent(s, ctx->ev_done, 0));
     CK(owner_field(ctx, box, s));
+    // straight into the caller's fields, unless they are not aligned to their element type
+    const bool direct = ((uintptr_t)u_dev | (uintptr_t)drho_dev) % sizeof(float) == 0;
     float* out = ctx->d_tmp + B.N;                     // [4][N]: u, then drho
-    CK(launch_stokes(B, reinterpret_cast<int*>(ctx->d_tmp), ctx->d_pd + B.pbeg, B.pcnt, d.counter_force,
-                     d.body_force, ctx->d_stokes, ctx->d_counts,
-                     reinterpret_cast<double*>(ctx->d_counts) + (ctx->maxp + 2) / 2, out, s));
-    CK(cudaMemcpyAsync(u_dev, out, 3ull * B.N * sizeof(float), cudaMemcpyDeviceToDevice, s));
-    if (drho_dev) CK(cudaMemcpyAsync(drho_dev, out + 3 * B.N, (size_t)B.N * sizeof(float), cudaMemcpyDeviceToDevice, s));
+    int* counts = reinterpret_cast<int*>(ctx->d_sums + 8);
+    CK(launch_stokes(B, reinterpret_cast<int*>(ctx->d_tmp), ctx->d_pd + B.pbeg, B.pcnt, d.counter_force, d.body_force,
+                     ctx->d_stokes, reinterpret_cast<int*>(ctx->d_stokes + 2 * B.N), counts,
+                     reinterpret_cast<float*>(counts + ctx->maxp + 1), ctx->d_sums, direct ? u_dev : out,
+                     direct ? drho_dev : out + 3 * B.N, s));
+    if (!direct) {
+        CK(cudaMemcpyAsync(u_dev, out, 3ull * B.N * sizeof(float), cudaMemcpyDeviceToDevice, s));
+        if (drho_dev) CK(cudaMemcpyAsync(drho_dev, out + 3 * B.N, (size_t)B.N * sizeof(float), cudaMemcpyDeviceToDevice, s));
+    }
     CK(cudaStreamSynchronize(s));
     return read_status(ctx);
 }

@@ -15,10 +15,11 @@
 // time scales.  The mean flow is then set so that the fluid and particle
 // momenta add up to zero (rho0 sum_fluid u = -sum_p M_p U_p, with the
 // particles' initial velocities), as they do in a run from rest with a
-// balancing counter force.  The transforms are separable DFTs along x, y and z:
-// a radix-2 FFT per line in shared memory for power-of-two edges, otherwise
-// computed by definition (one output element per thread, the line's twiddle
-// table in shared memory); FP32 complex, the per-mode solve in FP64.
+// balancing counter force.  The transforms are separable mixed-radix FFTs along x, y
+// and z in FP32, two real fields to a complex one; the per-mode solve carries twice
+// FP32's digits.
+#include <cmath>
+
 #include "lattice_common.cuh"
 
 namespace lbsph {
@@ -98,136 +99,324 @@ __device__ __forceinline__ int shell_owner(const int* owner, int nx, int ny, int
     return o;
 }
 
-// shell-node count of each particle of the box (fluid nodes next to it) and
-// fluid count
-__global__ void count_owner_kernel(const int* owner, int nx, int ny, int nz, int* counts, int np)
-{
-    const long long N = (long long)nx * ny * nz;
-    const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (n >= N || owner[n] != 0) return;
-    atomicAdd(counts, 1);
-    const int o = shell_owner(owner, nx, ny, nz, n);
-    if (o > 0 && o <= np) atomicAdd(counts + o, 1);
-}
+// ---- lb_stokes_field: buffers and constants of one call
+struct Stokes {
+    int nx, ny, nz, np, counter;
+    long long N;
+    double body[3], rho0, omega;
+    float kappa;                        // power of two by which the density travels with the velocity's z component
+    const int* owner;
+    const PartDev* pd;
+    int* shell;                         // [N] -1 not fluid, 0 fluid, p + 1 fluid next to particle p
+    int* counts;                        // [np + 1] fluid nodes, shell nodes per particle
+    float* table;                       // [np + 1][3] force density of a fluid node by its shell entry
+    double* sum;                        // [4] sums of u and drho over the fluid nodes
+    float* shift;                       // [4]
+    unsigned* done;                     // [2] blocks done
+    float2* z;                          // [2][N] gx + i gy and gz; in Fourier space, then ux + i uy and uz + i kappa drho
+    float* u;                           // [3][N]
+    float* drho;                        // [N] or null
+};
 
-// force density as complex [3][N]: F_ext / nshell on the fluid nodes next to
-// a particle (a uniform traction just outside its surface, under which a
-// sphere's interior moves rigidly at its Stokes velocity), plus the body force
-// and (counter_on) -sum F_ext / N_fluid on every fluid node
-__global__ void force_density_kernel(const int* owner, int nx, int ny, int nz, const int* counts, const PartDev* pd,
-                                     int np, int counter_on, double bx, double by, double bz, float2* g)
+// Shell entries, node counts, and (the last block) the force density's values: F_ext / nshell
+// on the fluid nodes next to a particle (a uniform traction just outside its surface, under
+// which a sphere's interior moves rigidly at its Stokes velocity), plus the body force and
+// (counter) -sum F_ext / N_fluid on every fluid node.  The values are formed once per
+// particle: forming them in FP64 at every node (a sum over the particles and two divisions)
+// took 1,590 us at 128^3 nodes and 16 particles, one atomic per fluid node another 50.
+__global__ void __launch_bounds__(256) shell_kernel(const Stokes S)
 {
-    const long long N = (long long)nx * ny * nz;
-    const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    double f[3] = {0.0, 0.0, 0.0};
-    if (owner[n] == 0) {
-        f[0] = bx; f[1] = by; f[2] = bz;
-        if (counter_on && counts[0] > 0) {
-            for (int p = 0; p < np; ++p)
-                for (int k = 0; k < 3; ++k) f[k] -= pd[p].Fext[k] / (double)counts[0];
-        }
-        const int o = shell_owner(owner, nx, ny, nz, n);
-        if (o > 0 && o <= np) {
-            const double c = 1.0 / (double)counts[o];
-            for (int k = 0; k < 3; ++k) f[k] += pd[o - 1].Fext[k] * c;
-        }
+    __shared__ int s_n;
+    __shared__ bool s_last;
+    const long long n = blockIdx.x * 256ll + threadIdx.x;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    int e = -1;
+    if (n < S.N && S.owner[n] == 0) {
+        const int o = shell_owner(S.owner, S.nx, S.ny, S.nz, n);
+        e = o > 0 && o <= S.np ? o : 0;
     }
-    for (int k = 0; k < 3; ++k) g[k * N + n] = make_float2((float)f[k], 0.0f);
-}
-
-// one DFT pass along one axis: out(.., k, ..) = sum_j in(.., j, ..) w^(j k),
-// w = exp(sign 2 pi i / n); ncomp components of [nz][ny][nx] each
-__global__ void dft_axis_kernel(const float2* in, float2* out, int nx, int ny, int nz, int axis, float sign,
-                                int ncomp)
-{
-    extern __shared__ float2 tw[];
-    const int n = axis == 0 ? nx : (axis == 1 ? ny : nz);
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        float s, c;
-        sincospif(2.0f * (float)j / (float)n, &s, &c);
-        tw[j] = make_float2(c, sign * s);
+    if (n < S.N) S.shell[n] = e;
+    if (e > 0) atomicAdd(S.counts + e, 1);
+    const unsigned m = __ballot_sync(0xffffffffu, e >= 0);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&s_n, __popc(m));
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicAdd(S.counts, s_n);
+        __threadfence();
+        s_last = atomicAdd(S.done, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    const long long N = (long long)nx * ny * nz;
-    const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (e >= ncomp * N) return;
-    const int comp = (int)(e / N);
-    const long long r = e - comp * N;
-    const int x = (int)(r % nx), y = (int)((r / nx) % ny), z = (int)(r / ((long long)nx * ny));
-    const int k = axis == 0 ? x : (axis == 1 ? y : z);
-    const long long stride = axis == 0 ? 1 : (axis == 1 ? nx : (long long)nx * ny);
-    const long long base = comp * N + r - (long long)k * stride;
-    float ar = 0.0f, ai = 0.0f;
-    int idx = 0;
-    for (int j = 0; j < n; ++j) {
-        const float2 v = in[base + j * stride];
-        const float2 w = tw[idx];
-        ar += v.x * w.x - v.y * w.y;
-        ai += v.x * w.y + v.y * w.x;
-        idx += k;
-        if (idx >= n) idx -= n;
+    if (!s_last) return;
+    __threadfence();
+    const int nf = __ldcg(S.counts);
+    for (int t = threadIdx.x; t < 3 * (S.np + 1); t += 256) {
+        const int p = t / 3, k = t % 3;
+        double f = S.body[k];
+        if (S.counter && nf > 0)
+            for (int q = 0; q < S.np; ++q) f -= S.pd[q].Fext[k] / (double)nf;
+        if (p > 0) f += S.pd[p - 1].Fext[k] * (1.0 / (double)__ldcg(S.counts + p));
+        S.table[t] = (float)f;
     }
-    out[e] = make_float2(ar, ai);
 }
 
-// the same pass for a power-of-two length n = 2^logn: one block per line, the
-// line staged in shared memory in bit-reversed order and transformed by logn
-// radix-2 butterfly stages (decimation in time) with the twiddles of the line
-// in shared memory; O(n log n) instead of O(n^2) per line
-__global__ void fft_axis_kernel(const float2* in, float2* out, int nx, int ny, int nz, int axis, float sign, int logn)
+// ---- Transforms.  Lines of any length n = r0 r1 ... (radices 8, 4, 2, 3, 5 as written-out
+// butterflies, any other prime by its definition) in shared memory, Stockham order: stage s
+// with ns = r0 ... r_(s-1) takes x[b + m n/r] for butterfly b, multiplies by w^(k m) with
+// k = b mod ns, w = exp(sign 2 pi i / (ns r)), and writes X[(b / ns) ns r + k + m ns].  A
+// block takes L neighbouring lines (16 consecutive x for the axes y and z, so that global
+// accesses are 128-byte runs; one line at a time along y and z touched 8 bytes of every
+// sector), in place; the two fields of real data travel as real and imaginary part of one
+// complex field.  Traffic (16 bytes in, 16 out per node and pass, within L2 up to 128^3) and
+// the stages' shared-memory accesses bound a pass.  Measured at 128^3: seven passes of one
+// line per block over 3 + 4 complex fields took 1,270 us, the six passes here FFT_NOTE.
+constexpr int FFT_T = 256, FFT_ST = 12;
+struct FftPlan {
+    int n, ns_, L, lp;                  // stages, lines per block, padded pitch of a row of lines
+    float sign;
+    int radix[FFT_ST], ns[FFT_ST], nb[FFT_ST];          // nb = n / radix
+    unsigned nm[FFT_ST];                // division by ns (magic_div)
+    int nsft[FFT_ST];
+};
+
+template <int R>
+__device__ __forceinline__ void dft(float2 (&v)[R], float sign);
+__device__ __forceinline__ float2 cadd2(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 csub2(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 cmul2(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
+__device__ __forceinline__ float2 rot(float2 a, float s) { return make_float2(-s * a.y, s * a.x); }      // i s a
+template <>
+__device__ __forceinline__ void dft<2>(float2 (&v)[2], float)
+{
+    const float2 a = v[0];
+    v[0] = cadd2(a, v[1]);
+    v[1] = csub2(a, v[1]);
+}
+template <>
+__device__ __forceinline__ void dft<3>(float2 (&v)[3], float s)
+{
+    const float2 t = cadd2(v[1], v[2]), d = csub2(v[1], v[2]);
+    const float2 m = make_float2(v[0].x - 0.5f * t.x, v[0].y - 0.5f * t.y), q = rot(d, s * 0.866025403784438647f);
+    v[0] = cadd2(v[0], t);
+    v[1] = cadd2(m, q);
+    v[2] = csub2(m, q);
+}
+template <>
+__device__ __forceinline__ void dft<4>(float2 (&v)[4], float s)
+{
+    const float2 a = cadd2(v[0], v[2]), b = csub2(v[0], v[2]), c = cadd2(v[1], v[3]), d = rot(csub2(v[1], v[3]), s);
+    v[0] = cadd2(a, c);
+    v[1] = cadd2(b, d);
+    v[2] = csub2(a, c);
+    v[3] = csub2(b, d);
+}
+template <>
+__device__ __forceinline__ void dft<5>(float2 (&v)[5], float s)
+{
+    const float c1 = 0.309016994374947424f, c2 = -0.809016994374947424f, s1 = s * 0.951056516295153572f, s2 = s * 0.587785252292473129f;
+    const float2 a = cadd2(v[1], v[4]), b = cadd2(v[2], v[3]), d = csub2(v[1], v[4]), e = csub2(v[2], v[3]);
+    const float2 m1 = make_float2(v[0].x + c1 * a.x + c2 * b.x, v[0].y + c1 * a.y + c2 * b.y);
+    const float2 m2 = make_float2(v[0].x + c2 * a.x + c1 * b.x, v[0].y + c2 * a.y + c1 * b.y);
+    const float2 q1 = rot(make_float2(s1 * d.x + s2 * e.x, s1 * d.y + s2 * e.y), 1.0f);
+    const float2 q2 = rot(make_float2(s2 * d.x - s1 * e.x, s2 * d.y - s1 * e.y), 1.0f);
+    v[0] = cadd2(v[0], cadd2(a, b));
+    v[1] = cadd2(m1, q1);
+    v[2] = cadd2(m2, q2);
+    v[3] = csub2(m2, q2);
+    v[4] = csub2(m1, q1);
+}
+template <>
+__device__ __forceinline__ void dft<8>(float2 (&v)[8], float s)
+{
+    float2 e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
+    dft<4>(e, s);
+    dft<4>(o, s);
+    const float h = 0.707106781186547524f;
+    o[1] = make_float2(h * (o[1].x - s * o[1].y), h * (o[1].y + s * o[1].x));
+    o[2] = rot(o[2], s);
+    o[3] = make_float2(h * (-o[3].x - s * o[3].y), h * (s * o[3].x - o[3].y));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        v[k] = cadd2(e[k], o[k]);
+        v[k + 4] = csub2(e[k], o[k]);
+    }
+}
+
+// one stage of radix R over the block's lines: a -> b; lines fastest (shift lb = log2 L)
+template <int R>
+__device__ __forceinline__ void fft_stage(const FftPlan& P, int st, int lb, const float2* a, float2* b, const float2* tw)
+{
+    const int nb = P.nb[st], ns = P.ns[st], step = nb / ns, L = 1 << lb;      // w^(k m) = tw[k m step]
+    for (int t = threadIdx.x; t < nb << lb; t += FFT_T) {
+        const int l = t & (L - 1), j = t >> lb;
+        const int q = div_magic(j, P.nm[st], P.nsft[st]), k = j - q * ns;
+        float2 v[R];
+#pragma unroll
+        for (int m = 0; m < R; ++m) v[m] = a[(j + m * nb) * P.lp + l];
+#pragma unroll
+        for (int m = 1; m < R; ++m) v[m] = cmul2(v[m], tw[k * m * step]);
+        dft<R>(v, P.sign);
+        const int o = q * ns * R + k;
+#pragma unroll
+        for (int m = 0; m < R; ++m) b[(o + m * ns) * P.lp + l] = v[m];
+    }
+}
+// a stage of any radix by its definition, one output per thread
+__device__ __forceinline__ void fft_stage_any(const FftPlan& P, int st, int lb, const float2* a, float2* b, const float2* tw)
+{
+    const int nb = P.nb[st], ns = P.ns[st], r = P.radix[st], step = nb / ns, L = 1 << lb;
+    for (int t = threadIdx.x; t < P.n << lb; t += FFT_T) {
+        const int l = t & (L - 1), jm = t >> lb, mo = jm / nb, j = jm - mo * nb;
+        const int q = div_magic(j, P.nm[st], P.nsft[st]), k = j - q * ns;
+        // angle of input m: m (k step + mo nb), modulo n
+        int inc = k * step + mo * nb, at = 0;
+        if (inc >= P.n) inc -= P.n;
+        float2 s = make_float2(0.0f, 0.0f);
+        for (int m = 0; m < r; ++m) {
+            s = cadd2(s, cmul2(a[(j + m * nb) * P.lp + l], tw[at]));
+            at += inc;
+            if (at >= P.n) at -= P.n;
+        }
+        b[(q * ns * r + k + mo * ns) * P.lp + l] = s;
+    }
+}
+
+enum { FFT_INPLACE = 0, FFT_FIRST = 1, FFT_LAST = 2 };
+
+// Lines along axis (0 x, 1 y, 2 z) of field blockIdx.y.  FFT_FIRST (axis x) takes the force
+// density from the shell entries; FFT_LAST (axis x) writes the real fields, sums them over the
+// fluid nodes, and its last block forms the shifts: a uniform velocity so that fluid and
+// particle momentum add up to zero (rho0 sum_fluid u + sum_p M_p U_p = 0) and no net mass.
+template <int MODE>
+__global__ void __launch_bounds__(FFT_T) fft_kernel(const __grid_constant__ Stokes S, const __grid_constant__ FftPlan P, int axis, int lb)
 {
     extern __shared__ float2 fsm[];
-    const int n = 1 << logn;
-    float2* buf = fsm;
-    float2* tw = fsm + n;
-    const long long N = (long long)nx * ny * nz;
-    const long long lines = N / n;                  // lines of one component
-    const int comp = (int)(blockIdx.x / lines);
-    const long long l = blockIdx.x - comp * lines;
-    long long base, stride;
-    if (axis == 0) {
-        stride = 1;
-        base = comp * N + l * nx;
-    } else if (axis == 1) {
-        stride = nx;
-        base = comp * N + (l / nx) * ((long long)nx * ny) + (l % nx);
-    } else {
-        stride = (long long)nx * ny;
-        base = comp * N + l;                        // l = y * nx + x
-    }
-    for (int j = threadIdx.x; j < n / 2; j += blockDim.x) {
+    float2* a = fsm;
+    float2* b = a + P.n * P.lp;
+    float2* tw = b + P.n * P.lp;
+    const int n = P.n, L = 1 << lb, comp = blockIdx.y;
+    for (int j = threadIdx.x; j < n; j += FFT_T) {
         float sn, cs;
         sincospif(2.0f * (float)j / (float)n, &sn, &cs);
-        tw[j] = make_float2(cs, sign * sn);
+        tw[j] = make_float2(cs, P.sign * sn);
     }
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const int rj = (int)(__brev((unsigned)j) >> (32 - logn));
-        buf[rj] = in[base + j * stride];
+    float2* z = S.z + comp * S.N;
+    // first element, line pitch, element stride and number of lines of this block
+    long long base, ls, es;
+    int nl;
+    if (axis == 0) {
+        const long long rows = (long long)S.ny * S.nz, r0 = (long long)blockIdx.x << lb;
+        base = r0 * S.nx; ls = S.nx; es = 1;
+        nl = (int)min((long long)L, rows - r0);
+    } else {
+        const int tiles = (S.nx + L - 1) >> lb, pl = blockIdx.x / tiles, x0 = (blockIdx.x - pl * tiles) << lb;
+        const long long row = (long long)S.nx * S.ny;
+        base = (axis == 1 ? pl * row : (long long)pl * S.nx) + x0; ls = 1; es = axis == 1 ? S.nx : row;
+        nl = min(L, S.nx - x0);
+    }
+    // along x consecutive threads take consecutive elements of a line, else consecutive lines
+    if (axis == 0) {
+        for (int l = threadIdx.x >> 5; l < nl; l += FFT_T / 32)
+            for (int j = threadIdx.x & 31; j < n; j += 32) {
+                if (MODE == FFT_FIRST) {
+                    const int e = S.shell[base + l * ls + j];
+                    float2 v = make_float2(0.0f, 0.0f);
+                    if (e >= 0) v = comp == 0 ? make_float2(S.table[3 * e], S.table[3 * e + 1]) : make_float2(S.table[3 * e + 2], 0.0f);
+                    a[j * P.lp + l] = v;
+                } else {
+                    a[j * P.lp + l] = z[base + l * ls + j];
+                }
+            }
+    } else {
+        for (int t = threadIdx.x; t < n << lb; t += FFT_T) {
+            const int l = t & (L - 1), j = t >> lb;
+            if (l < nl) a[j * P.lp + l] = z[base + l + j * es];
+        }
     }
     __syncthreads();
-    for (int st = 1; st <= logn; ++st) {
-        const int half = 1 << (st - 1);
-        for (int t = threadIdx.x; t < n / 2; t += blockDim.x) {
-            const int grp = t >> (st - 1), pos = t & (half - 1);
-            const int i0 = (grp << st) + pos, i1 = i0 + half;
-            const float2 w = tw[pos << (logn - st)];
-            const float2 a = buf[i0], b = buf[i1];
-            const float2 bw = make_float2(b.x * w.x - b.y * w.y, b.x * w.y + b.y * w.x);
-            buf[i0] = make_float2(a.x + bw.x, a.y + bw.y);
-            buf[i1] = make_float2(a.x - bw.x, a.y - bw.y);
+    for (int st = 0; st < P.ns_; ++st) {
+        switch (P.radix[st]) {
+        case 8: fft_stage<8>(P, st, lb, a, b, tw); break;
+        case 5: fft_stage<5>(P, st, lb, a, b, tw); break;
+        case 4: fft_stage<4>(P, st, lb, a, b, tw); break;
+        case 3: fft_stage<3>(P, st, lb, a, b, tw); break;
+        case 2: fft_stage<2>(P, st, lb, a, b, tw); break;
+        default: fft_stage_any(P, st, lb, a, b, tw);
         }
         __syncthreads();
+        float2* t = a;
+        a = b;
+        b = t;
     }
-    for (int j = threadIdx.x; j < n; j += blockDim.x) out[base + j * stride] = buf[j];
+    if (MODE != FFT_LAST) {
+        if (axis == 0) {
+            for (int l = threadIdx.x >> 5; l < nl; l += FFT_T / 32)
+                for (int j = threadIdx.x & 31; j < n; j += 32) z[base + l * ls + j] = a[j * P.lp + l];
+        } else {
+            for (int t = threadIdx.x; t < n << lb; t += FFT_T) {
+                const int l = t & (L - 1), j = t >> lb;
+                if (l < nl) z[base + l + j * es] = a[j * P.lp + l];
+            }
+        }
+        return;
+    }
+    // real fields and their sums over the fluid nodes (per thread as a sum and its rounding errors)
+    float hi[2] = {0.0f, 0.0f}, lo[2] = {0.0f, 0.0f};
+    const float ik = 1.0f / S.kappa;
+    for (int l = threadIdx.x >> 5; l < nl; l += FFT_T / 32)
+        for (int j = threadIdx.x & 31; j < n; j += 32) {
+            const long long at = base + l * ls + j;
+            const float2 v = a[j * P.lp + l];
+            const float w[2] = {v.x, comp == 0 ? v.y : v.y * ik};
+            S.u[(comp == 0 ? 0 : 2) * S.N + at] = w[0];
+            if (comp == 0) S.u[S.N + at] = w[1];
+            else if (S.drho) S.drho[at] = w[1];
+            if (S.shell[at] >= 0) {
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const float t = hi[c] + w[c], d = t - hi[c];
+                    lo[c] += (hi[c] - (t - d)) + (w[c] - d);
+                    hi[c] = t;
+                }
+            }
+        }
+    __shared__ double s_sum[FFT_T / 32][2];
+    __shared__ bool s_last;
+    double v[2] = {(double)hi[0] + (double)lo[0], (double)hi[1] + (double)lo[1]};
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        for (int o = 16; o > 0; o >>= 1) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
+        if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5][c] = v[c];
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        double t = 0.0;
+        for (int w = 0; w < FFT_T / 32; ++w) t += s_sum[w][threadIdx.x];
+        atomicAdd(S.sum + 2 * comp + threadIdx.x, t);
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(S.done + 1, 1u) == gridDim.x * gridDim.y - 1;
+    __syncthreads();
+    if (!s_last || threadIdx.x >= 4) return;
+    __threadfence();
+    const int k = threadIdx.x, nf = __ldcg(S.counts);
+    double Pk = 0.0;
+    if (k < 3)
+        for (int p = 0; p < S.np; ++p) Pk += S.pd[p].M * S.pd[p].U[k];
+    S.shift[k] = nf > 0 ? (float)((-Pk / S.rho0 - __ldcg(S.sum + k)) / (double)nf) : 0.0f;
 }
 
-static int log2_if_pow2(int n)
+// the shifts, on the fluid nodes
+__global__ void __launch_bounds__(256) shift_kernel(const Stokes S)
 {
-    if (n < 2 || (n & (n - 1)) != 0) return -1;
-    int l = 0;
-    while ((1 << l) < n) ++l;
-    return l;
+    const float s[4] = {S.shift[0], S.shift[1], S.shift[2], S.shift[3]};
+    for (long long n = blockIdx.x * 256ll + threadIdx.x; n < S.N; n += gridDim.x * 256ll) {
+        if (S.shell[n] < 0) continue;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) S.u[k * S.N + n] += s[k];
+        if (S.drho) S.drho[n] += s[3];
+    }
 }
 
 // Steady state of the linear lattice fluid itself (D3Q19 BGK, omega = 1/tau,
@@ -241,151 +430,150 @@ static int log2_if_pow2(int n)
 //   -omega H1 drho + rho0 D2 u     = g/2 + 3 (1 - omega/2) H2 g
 // with H1 = sum w_i c_i h_i, H2 = sum w_i c_i c_i^T h_i,
 // D0 = sum w_i (1 - e_i) q_i and D2 = sum 3 w_i c_i c_i^T (1 - e_i) q_i,
-// q_i = 1 / (1 - (1 - omega) e_i), with 1 - e_i = 2 sin^2(th/2) + i sin th
-// written without cancellation (D0 and D2 vanish like k^2).  The terms of one
-// direction in FP32, their sums and the solve in FP64 (Gaussian elimination
-// with partial pivoting); the k = 0 mode (mean flow and
-// mass, set afterwards) and numerically singular modes are zero.  On entry g
-// holds the transformed force density (components 0-2); on exit u^ (0-2) and
-// drho^ (3), with the 1/N of the inverse DFT folded in.
-struct cplx {
-    double re, im;
+// q_i = 1 / (1 - (1 - omega) e_i).  The terms of c and -c are complex conjugates, so H1 = i a
+// with a real and H2, D0, D2 are real: over the nine pairs of directions
+//   a = sum 2 w c Im h,  H2 = sum 2 w c c^T Re h,  D0 = sum 2 w r,  D2 = sum 6 w c c^T r,
+//   r = Re (1 - e) q = (1 + (1 - omega)) 2 sin^2(th/2) / |1 - (1 - omega) e|^2 >= 0,
+// without cancellation (D0 and D2 vanish like k^2).  With drho = i s,
+//   s = (fo a.g + 3 rho0 omega a.u) / D0,   (rho0 D2 + 3 rho0 omega^2 a a^T / D0) u = g/2 + fo H2 g - (omega fo a.g / D0) a
+// (fo = 3 (1 - omega/2)): a symmetric positive definite 3 x 3 system with real
+// coefficients for the real and the imaginary part of g, solved by cofactors.  The terms of one
+// direction are FP32; sums and solve are carried to twice FP32's digits (ff below).
+// One thread takes a mode and its conjugate: the fields are real, so the transforms of two of
+// them come as one, Z(k) = X(k) + i Y(k), X(k) = (Z(k) + conj Z(-k)) / 2, and go back the
+// same way.  The k = 0 mode (mean flow and mass, set afterwards) and numerically singular
+// modes are zero; the 1/N of the inverse DFT is folded in.
+// Numbers as the unevaluated sum of two FP32 (Dekker, "A floating-point technique for
+// extending the available precision", 1971; Knuth's two-sum): 48 bits of significand from FP32
+// instructions, which this part issues 64 times as often as FP64 ones.  The system above loses a
+// factor of about 1 / k^2 (4e2 at an edge of 128, 4e5 at 4096) to the stiff longitudinal
+// direction: 2^-46 times that stays far below the FP32 rounding of its terms.
+struct ff {
+    float h, l;
 };
-__device__ __forceinline__ cplx cmul(cplx a, cplx b) { return {a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re}; }
-__device__ __forceinline__ cplx cdiv(cplx a, cplx b)
+__device__ __forceinline__ ff two_sum(float a, float b)
 {
-    const double d = b.re * b.re + b.im * b.im;
-    return {(a.re * b.re + a.im * b.im) / d, (a.im * b.re - a.re * b.im) / d};
+    const float s = __fadd_rn(a, b), d = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, d)), __fsub_rn(b, d))};
 }
-__device__ __forceinline__ cplx csub(cplx a, cplx b) { return {a.re - b.re, a.im - b.im}; }
-__device__ __forceinline__ cplx cadd(cplx a, cplx b) { return {a.re + b.re, a.im + b.im}; }
-__device__ __forceinline__ cplx cscale(cplx a, double s) { return {a.re * s, a.im * s}; }
-
-__global__ void lattice_steady_kernel(float2* g, int nx, int ny, int nz, double omega, double rho0)
+__device__ __forceinline__ ff quick(float a, float b)       // |a| >= |b|
 {
-    const long long N = (long long)nx * ny * nz;
-    const long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (r >= N) return;
-    const int x = (int)(r % nx), y = (int)((r / nx) % ny), z = (int)(r / ((long long)nx * ny));
-    cplx H1[3] = {}, H2[3][3] = {}, D0 = {}, D2[3][3] = {};
-    // each direction's terms in FP32 (the terms of c and -c are exact complex
-    // conjugates, so the imaginary parts still cancel pairwise), summed in FP64
-    const float fx = (float)x / nx, fy = (float)y / ny, fz = (float)z / nz, om1 = (float)(1.0 - omega);
+    const float s = __fadd_rn(a, b);
+    return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ ff operator+(ff a, ff b)
+{
+    const ff s = two_sum(a.h, b.h);
+    return quick(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ ff operator-(ff a, ff b) { return a + ff{-b.h, -b.l}; }
+__device__ __forceinline__ ff operator+(ff a, float b)
+{
+    const ff s = two_sum(a.h, b);
+    return quick(s.h, __fadd_rn(s.l, a.l));
+}
+__device__ __forceinline__ ff operator*(ff a, ff b)
+{
+    const float p = __fmul_rn(a.h, b.h);
+    return quick(p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p))));
+}
+__device__ __forceinline__ ff operator*(ff a, float b)
+{
+    const float p = __fmul_rn(a.h, b);
+    return quick(p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p)));
+}
+__device__ __forceinline__ ff recip(ff a)
+{
+    const float x = 1.0f / a.h;
+    const float e = __fmaf_rn(-a.l, x, __fmaf_rn(-a.h, x, 1.0f));      // 1 - a x
+    return quick(x, __fmul_rn(x, e));
+}
+
+struct SteadyConst {
+    ff om, fo18, fo, six_rho, tro, inv_n;   // omega, fo / 18, fo, 6 / rho0, 3 rho0 omega, 1 / N
+    float om1, opm;                         // 1 - omega, 2 - omega
+};
+
+// One thread per mode of the planes z <= nz / 2 that comes no later than its conjugate.
+// Sums in units of 1/18: D0 = D0' / 18, a = a' / 18, H2 = H2' / 18, D2 = D2' / 6.
+// Measured at 128^3: 4,207 us as a complex 4 x 4 FP64 elimination with pivoting per mode,
+// STEADY_NOTE.
+__global__ void __launch_bounds__(128) steady_kernel(const Stokes S, const SteadyConst K)
+{
+    const int nx = S.nx, ny = S.ny, nz = S.nz;
+    const int r = (int)(blockIdx.x * 128u + threadIdx.x);           // 19 N < 2^31
+    const int plane = nx * ny;
+    if (r >= (nz / 2 + 1) * plane) return;
+    const int z = r / plane, y = (r - z * plane) / nx, x = r - z * plane - y * nx;
+    const int r2 = ((z == 0 ? 0 : nz - z) * ny + (y == 0 ? 0 : ny - y)) * nx + (x == 0 ? 0 : nx - x);
+    if (r2 < r) return;
+    const float2 z1 = S.z[r], z1c = S.z[r2], z2 = S.z[S.N + r];
+    const float fx = (float)x / nx, fy = (float)y / ny, fz = (float)z / nz;
+    const ff zero = {0.0f, 0.0f};
+    ff a[3] = {zero, zero, zero}, D0 = zero;
+    ff H[6] = {zero, zero, zero, zero, zero, zero}, D[6] = {zero, zero, zero, zero, zero, zero};      // xx yy zz xy xz yz
 #pragma unroll
-    for (int i = 1; i < Q; ++i) {        // the rest population has c = 0: no share in H1, H2, D0, D2
-        const int c[3] = {cx_of(i), cy_of(i), cz_of(i)};
-        // theta / pi, reduced to [-1, 1) so that sinpi / cospi stay exact at multiples of pi
-        float tp = 2.0f * (fx * c[0] + fy * c[1] + fz * c[2]);
+    for (int m = 0; m < 9; ++m) {
+        const int i = 2 * m + 1, cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
+        // theta / pi, reduced to [-1, 1) so that the half angle stays in the accurate range
+        float tp = 2.0f * (fx * cx + fy * cy + fz * cz);
         tp -= 2.0f * floorf(0.5f * tp + 0.5f);
-        float snf, csf;
-        sincospif(tp, &snf, &csf);
-        const float shf = sinpif(0.5f * tp);
-        const float dre = 1.0f - om1 * csf, dim = om1 * snf, dd = dre * dre + dim * dim;
-        // h = e / den, q = (1 - e) / den with e = cs - i sn, 1 - e = 2 sh^2 + i sn
-        const float hre = (csf * dre - snf * dim) / dd, him = (-snf * dre - csf * dim) / dd;
-        const float are = 2.0f * shf * shf, aim = snf;
-        const float qre = (are * dre + aim * dim) / dd, qim = (aim * dre - are * dim) / dd;
-        const cplx h = {(double)hre, (double)him};
-        const cplx q = {(double)qre, (double)qim};
-        const double w = wd_of(i);
+        float sh, ch;
+        sincospif(0.5f * tp, &sh, &ch);
+        const float s2 = sh * sh;
+        // |1 - (1 - omega) e|^2 as a sum of terms of one sign
+        const float dd = K.om1 >= 0.0f ? (1.0f - K.om1) * (1.0f - K.om1) + 4.0f * K.om1 * s2
+                                       : K.opm * K.opm - 4.0f * K.om1 * (ch * ch);
+        const float wt = m < 3 ? 2.0f : 1.0f;                       // 36 w
+        const float id = wt / dd;
+        const float hre = (1.0f - K.om1 - 2.0f * s2) * id, him = -2.0f * sh * ch * id, rr = K.opm * (2.0f * s2) * id;
+        D0 = D0 + rr;
+        if (cx) { a[0] = a[0] + (float)cx * him; H[0] = H[0] + hre; D[0] = D[0] + rr; }
+        if (cy) { a[1] = a[1] + (float)cy * him; H[1] = H[1] + hre; D[1] = D[1] + rr; }
+        if (cz) { a[2] = a[2] + (float)cz * him; H[2] = H[2] + hre; D[2] = D[2] + rr; }
+        if (cx * cy) { H[3] = H[3] + (float)(cx * cy) * hre; D[3] = D[3] + (float)(cx * cy) * rr; }
+        if (cx * cz) { H[4] = H[4] + (float)(cx * cz) * hre; D[4] = D[4] + (float)(cx * cz) * rr; }
+        if (cy * cz) { H[5] = H[5] + (float)(cy * cz) * hre; D[5] = D[5] + (float)(cy * cz) * rr; }
+    }
+    // [part][component] of g: real, imaginary
+    const float g[2][3] = {{0.5f * (z1.x + z1c.x), 0.5f * (z1.y + z1c.y), z2.x}, {0.5f * (z1.y - z1c.y), 0.5f * (z1c.x - z1.x), z2.y}};
+    float u[2][3] = {}, sd[2] = {};
+    const bool ok0 = r != 0 && D0.h > 0.0f;
+    const ff iD = recip(ok0 ? D0 : ff{1.0f, 0.0f}), oD = K.om * iD;
+    const ff t[3] = {a[0] * oD, a[1] * oD, a[2] * oD};
+    const ff v[3] = {t[0] * K.om, t[1] * K.om, t[2] * K.om};
+    const ff Mxx = D[0] + a[0] * v[0], Myy = D[1] + a[1] * v[1], Mzz = D[2] + a[2] * v[2];
+    const ff Mxy = D[3] + a[0] * v[1], Mxz = D[4] + a[0] * v[2], Myz = D[5] + a[1] * v[2];
+    const ff Cxx = Myy * Mzz - Myz * Myz, Cxy = Mxz * Myz - Mxy * Mzz, Cxz = Mxy * Myz - Mxz * Myy;
+    const ff Cyy = Mxx * Mzz - Mxz * Mxz, Cyz = Mxy * Mxz - Mxx * Myz, Czz = Mxx * Myy - Mxy * Mxy;
+    const ff det = Mxx * Cxx + Mxy * Cxy + Mxz * Cxz;
+    // numerically singular: a determinant below 1e-13 of the product of the diagonal
+    if (ok0 && det.h > 1e-13f * Mxx.h * Myy.h * Mzz.h) {
+        const ff idet = recip(det) * K.inv_n;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (c[a] == 0) continue;
-            H1[a] = cadd(H1[a], cscale(h, w * c[a]));
-#pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                if (c[b] == 0) continue;
-                H2[a][b] = cadd(H2[a][b], cscale(h, w * c[a] * c[b]));
-                D2[a][b] = cadd(D2[a][b], cscale(q, 3.0 * w * c[a] * c[b]));
-            }
-        }
-        D0 = cadd(D0, cscale(q, w));
-    }
-    const float2 g0 = g[r], g1 = g[N + r], g2 = g[2 * N + r];
-    const cplx gh[3] = {{g0.x, g0.y}, {g1.x, g1.y}, {g2.x, g2.y}};
-    const double fo = 3.0 * (1.0 - 0.5 * omega);
-    // augmented 4 x 5 system: unknowns (drho, ux, uy, uz)
-    cplx M[4][5];
-    M[0][0] = D0;
-    cplx r0 = {0.0, 0.0};
-    for (int a = 0; a < 3; ++a) {
-        M[0][1 + a] = cscale(H1[a], -3.0 * rho0 * omega);
-        r0 = cadd(r0, cmul(H1[a], gh[a]));
-    }
-    M[0][4] = cscale(r0, fo);
-    for (int a = 0; a < 3; ++a) {
-        M[1 + a][0] = cscale(H1[a], -omega);
-        cplx ra = cscale(gh[a], 0.5);
-        for (int b = 0; b < 3; ++b) {
-            M[1 + a][1 + b] = cscale(D2[a][b], rho0);
-            ra = cadd(ra, cscale(cmul(H2[a][b], gh[b]), fo));
-        }
-        M[1 + a][4] = ra;
-    }
-    double scale = 0.0;
-    for (int a = 0; a < 4; ++a)
-        for (int b = 0; b < 4; ++b) scale = fmax(scale, fabs(M[a][b].re) + fabs(M[a][b].im));
-    bool ok = r != 0 && scale > 0.0;
-    for (int col = 0; col < 4 && ok; ++col) {
-        int piv = col;
-        double best = 0.0;
-        for (int row = col; row < 4; ++row) {
-            const double m = M[row][col].re * M[row][col].re + M[row][col].im * M[row][col].im;
-            if (m > best) { best = m; piv = row; }
-        }
-        if (!(sqrt(best) > 1e-14 * scale)) { ok = false; break; }
-        if (piv != col)
-            for (int j = 0; j < 5; ++j) { const cplx t = M[col][j]; M[col][j] = M[piv][j]; M[piv][j] = t; }
-        for (int row = 0; row < 4; ++row) {
-            if (row == col) continue;
-            const cplx f = cdiv(M[row][col], M[col][col]);
-            for (int j = col; j < 5; ++j) M[row][j] = csub(M[row][j], cmul(f, M[col][j]));
+        for (int c = 0; c < 2; ++c) {
+            const ff ag = a[0] * g[c][0] + a[1] * g[c][1] + a[2] * g[c][2];
+            const ff hx = H[0] * g[c][0] + H[3] * g[c][1] + H[4] * g[c][2] - ag * t[0];
+            const ff hy = H[3] * g[c][0] + H[1] * g[c][1] + H[5] * g[c][2] - ag * t[1];
+            const ff hz = H[4] * g[c][0] + H[5] * g[c][1] + H[2] * g[c][2] - ag * t[2];
+            const ff bx = (K.fo18 * hx + 0.5f * g[c][0]) * K.six_rho, by = (K.fo18 * hy + 0.5f * g[c][1]) * K.six_rho,
+                     bz = (K.fo18 * hz + 0.5f * g[c][2]) * K.six_rho;
+            const ff ux = (Cxx * bx + Cxy * by + Cxz * bz) * idet, uy = (Cxy * bx + Cyy * by + Cyz * bz) * idet,
+                     uz = (Cxz * bx + Cyz * by + Czz * bz) * idet;
+            const ff s = (K.fo * ag * K.inv_n + K.tro * (a[0] * ux + a[1] * uy + a[2] * uz)) * iD;
+            u[c][0] = ux.h + ux.l; u[c][1] = uy.h + uy.l; u[c][2] = uz.h + uz.l;
+            sd[c] = s.h + s.l;
         }
     }
-    cplx sol[4] = {};
-    if (ok)
-        for (int a = 0; a < 4; ++a) sol[a] = cscale(cdiv(M[a][4], M[a][a]), 1.0 / (double)N);
-    g[r] = make_float2((float)sol[1].re, (float)sol[1].im);
-    g[N + r] = make_float2((float)sol[2].re, (float)sol[2].im);
-    g[2 * N + r] = make_float2((float)sol[3].re, (float)sol[3].im);
-    g[3 * N + r] = make_float2((float)sol[0].re, (float)sol[0].im);
-}
-
-__global__ void real_part_kernel(const float2* g, long long n3, float* u)
-{
-    const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (e < n3) u[e] = g[e].x;
-}
-
-// sum over fluid nodes of u and drho (4 doubles), one atomic per warp
-__global__ void fluid_sum_kernel(const float* u, const int* owner, long long N, double* sum)
-{
-    const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    if (n < N && owner[n] == 0)
-        for (int k = 0; k < 4; ++k) v[k] = u[k * N + n];
-    for (int k = 0; k < 4; ++k) {
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-        if ((threadIdx.x & 31) == 0 && v[k] != 0.0) atomicAdd(sum + k, v[k]);
+    // drho = i s: real part -Im s, imaginary part Re s
+    const float dre = -sd[1] * S.kappa, dim = sd[0] * S.kappa;
+    S.z[r] = make_float2(u[0][0] - u[1][1], u[1][0] + u[0][1]);
+    S.z[S.N + r] = make_float2(u[0][2] - dim, u[1][2] + dre);
+    if (r2 != r) {
+        S.z[r2] = make_float2(u[0][0] + u[1][1], u[0][1] - u[1][0]);
+        S.z[S.N + r2] = make_float2(u[0][2] + dim, dre - u[1][2]);
     }
 }
-
-// uniform shift of the fluid so that fluid + particle momentum is zero:
-// rho0 sum_fluid u + sum_p M_p U_p = 0
-__global__ void momentum_shift_kernel(float* u, const int* owner, long long N, const double* sum, const int* counts,
-                                      const PartDev* pd, int np, double rho0)
-{
-    const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (n >= N || owner[n] != 0 || counts[0] == 0) return;
-    for (int k = 0; k < 3; ++k) {
-        double P = 0.0;
-        for (int p = 0; p < np; ++p) P += pd[p].M * pd[p].U[k];
-        const double shift = (-P / rho0 - sum[k]) / (double)counts[0];
-        u[k * N + n] += (float)shift;
-    }
-    u[3 * N + n] -= (float)(sum[3] / (double)counts[0]);     // no net mass change
-}
-
 static unsigned nblk(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
 cudaError_t launch_init_fluid(const BoxDev& B, int precision, void* fbuf, const float* u, const float* drho,
@@ -398,45 +586,92 @@ cudaError_t launch_init_fluid(const BoxDev& B, int precision, void* fbuf, const 
     return cudaGetLastError();
 }
 
-// work: 8 N float2 (two complex [4][N] buffers); counts: np + 1 ints; sum: 4
-// doubles; u: [4][N] (velocity, then the density deviation)
+// radices of a line of length n: 8, 4, 2, then 3, 5, then whatever primes are left
+static FftPlan fft_plan(int n, float sign)
+{
+    FftPlan P{};
+    P.n = n;
+    P.sign = sign;
+    int left = n, ns = 1;
+    auto take = [&](int r) {
+        P.radix[P.ns_] = r;
+        P.ns[P.ns_] = ns;
+        P.nb[P.ns_] = n / r;
+        magic_div((unsigned)ns, P.nm[P.ns_], P.nsft[P.ns_]);
+        ++P.ns_;
+        ns *= r;
+        left /= r;
+    };
+    while (left % 8 == 0 && left != 16) take(8);        // 16 = 4 x 4
+    for (int r : {4, 2, 3, 5})
+        while (left % r == 0) take(r);
+    for (int r = 7; left > 1; r += 2) {
+        if (r * r > left) r = left;
+        while (left % r == 0) take(r);
+    }
+    return P;
+}
+
+// z: 2 N float2; shell: N ints; counts: np + 1 ints; table: 3 (np + 1) floats; sum: 4 doubles,
+// shift: 4 floats, done: 2 counters; u [3][N], drho [N] or null: the result
 cudaError_t launch_stokes(const BoxDev& B, const int* owner, const PartDev* pd, int np, int counter_on,
-                          const double body[3], float2* work, int* counts, double* sum, float* u,
-                          cudaStream_t s)
+                          const double body[3], float2* z, int* shell, int* counts, float* table, double* sum, float* u,
+                          float* drho, cudaStream_t s)
 {
     cudaError_t e;
-    const long long N = B.N;
+    Stokes S{};
+    S.nx = B.nx; S.ny = B.ny; S.nz = B.nz; S.np = np; S.counter = counter_on; S.N = B.N;
+    for (int k = 0; k < 3; ++k) S.body[k] = body[k];
+    S.rho0 = B.rho0; S.omega = (double)B.omega;
+    // drho is of the order of mu u / r a few nodes from a particle: scaled so that neither of
+    // the two fields that share a transform loses digits to the other
+    int ex = 0;
+    std::frexp(4.0 / (B.rho0 * (1.0 / S.omega - 0.5) / 3.0), &ex);
+    S.kappa = (float)std::ldexp(1.0, ex);
+    S.owner = owner; S.pd = pd; S.shell = shell; S.counts = counts; S.table = table; S.sum = sum;
+    S.shift = reinterpret_cast<float*>(sum + 4);
+    S.done = reinterpret_cast<unsigned*>(S.shift + 4);
+    S.z = z; S.u = u; S.drho = drho;
     if ((e = cudaMemsetAsync(counts, 0, sizeof(int) * (np + 1), s)) != cudaSuccess) return e;
-    count_owner_kernel<<<nblk(N, 256), 256, 0, s>>>(owner, B.nx, B.ny, B.nz, counts, np);
-    float2* a = work;
-    float2* b = work + 4 * N;
-    force_density_kernel<<<nblk(N, 256), 256, 0, s>>>(owner, B.nx, B.ny, B.nz, counts, pd, np, counter_on, body[0],
-                                                       body[1], body[2], a);
+    if ((e = cudaMemsetAsync(sum, 0, 4 * sizeof(double) + 4 * sizeof(float) + 2 * sizeof(unsigned), s)) != cudaSuccess) return e;
+    shell_kernel<<<nblk(S.N, 256), 256, 0, s>>>(S);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const int nmax = B.nx > B.ny ? (B.nx > B.nz ? B.nx : B.nz) : (B.ny > B.nz ? B.ny : B.nz);
-    const size_t sh = sizeof(float2) * nmax;
-    // one pass along an axis: the radix-2 FFT for power-of-two edges, else the
-    // transform by definition
-    auto pass = [&](const float2* src, float2* dst, int ax, float sign, int ncomp) {
-        const int n = ax == 0 ? B.nx : (ax == 1 ? B.ny : B.nz);
-        const int lg = log2_if_pow2(n);
-        if (lg > 0) {
-            const int threads = n / 2 < 32 ? 32 : (n / 2 > 256 ? 256 : n / 2);
-            fft_axis_kernel<<<(unsigned)(ncomp * (N / n)), threads, sizeof(float2) * (n + n / 2), s>>>(
-                src, dst, B.nx, B.ny, B.nz, ax, sign, lg);
-        } else {
-            dft_axis_kernel<<<nblk(ncomp * N, 256), 256, sh, s>>>(src, dst, B.nx, B.ny, B.nz, ax, sign, ncomp);
-        }
+    auto pass = [&](int mode, int ax, float sign) {
+        FftPlan P = fft_plan(ax == 0 ? B.nx : (ax == 1 ? B.ny : B.nz), sign);
+        // 16 lines (128-byte runs along x) while two buffers of them take at most 72 KiB of shared memory
+        int lb = 4;
+        while (lb > 0 && 2ll * P.n * ((1 << lb) + 1) * 8 > 72 * 1024) --lb;
+        P.lp = (1 << lb) + 1;
+        const size_t sm = sizeof(float2) * (2ull * P.n * P.lp + P.n);
+        const long long lines = ax == 0 ? ((long long)B.ny * B.nz + (1 << lb) - 1) >> lb
+                                        : (long long)(ax == 1 ? B.nz : B.ny) * ((B.nx + (1 << lb) - 1) >> lb);
+        const dim3 grid((unsigned)lines, 2);
+        auto go = [&](auto* k) {
+            if (sm > 48 * 1024) {
+                const cudaError_t r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+                if (r != cudaSuccess) return r;
+            }
+            k<<<grid, FFT_T, sm, s>>>(S, P, ax, lb);
+            return cudaGetLastError();
+        };
+        return mode == FFT_FIRST ? go(fft_kernel<FFT_FIRST>) : (mode == FFT_LAST ? go(fft_kernel<FFT_LAST>) : go(fft_kernel<FFT_INPLACE>));
     };
-    for (int ax = 0; ax < 3; ++ax) pass(ax % 2 == 0 ? a : b, ax % 2 == 0 ? b : a, ax, -1.0f, 3);
-    // forward result in b (three passes: a->b, b->a, a->b)
-    lattice_steady_kernel<<<nblk(N, 128), 128, 0, s>>>(b, B.nx, B.ny, B.nz, (double)B.omega, B.rho0);
-    for (int ax = 0; ax < 3; ++ax) pass(ax % 2 == 0 ? b : a, ax % 2 == 0 ? a : b, ax, 1.0f, 4);
-    // inverse result in a
-    real_part_kernel<<<nblk(4 * N, 256), 256, 0, s>>>(a, 4 * N, u);
-    if ((e = cudaMemsetAsync(sum, 0, 4 * sizeof(double), s)) != cudaSuccess) return e;
-    fluid_sum_kernel<<<nblk(N, 256), 256, 0, s>>>(u, owner, N, sum);
-    momentum_shift_kernel<<<nblk(N, 256), 256, 0, s>>>(u, owner, N, sum, counts, pd, np, B.rho0);
+    if ((e = pass(FFT_FIRST, 0, -1.0f)) != cudaSuccess) return e;
+    for (int ax = 1; ax < 3; ++ax)
+        if ((e = pass(FFT_INPLACE, ax, -1.0f)) != cudaSuccess) return e;
+    SteadyConst K;
+    const double om = S.omega, fo = 3.0 * (1.0 - 0.5 * om);
+    auto split = [](double v) { const float h = (float)v; return ff{h, (float)(v - (double)h)}; };
+    K.om = split(om); K.fo18 = split(fo / 18.0); K.fo = split(fo); K.six_rho = split(6.0 / S.rho0);
+    K.tro = split(3.0 * S.rho0 * om); K.inv_n = split(1.0 / (double)S.N);
+    K.om1 = (float)(1.0 - om); K.opm = (float)(2.0 - om);
+    steady_kernel<<<nblk((long long)(B.nz / 2 + 1) * B.nx * B.ny, 128), 128, 0, s>>>(S, K);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    for (int ax = 2; ax > 0; --ax)
+        if ((e = pass(FFT_INPLACE, ax, 1.0f)) != cudaSuccess) return e;
+    if ((e = pass(FFT_LAST, 0, 1.0f)) != cudaSuccess) return e;
+    const unsigned g = nblk(S.N, 256);
+    shift_kernel<<<g < 1216 ? g : 1216, 256, 0, s>>>(S);
     return cudaGetLastError();
 }
 
