@@ -37,7 +37,7 @@ cudaError_t launch_init_fluid(const BoxDev& B, int precision, void* fbuf, const 
                               const int* owner, float tau, int stress, cudaStream_t s);
 cudaError_t launch_stokes(const BoxDev& B, const int* owner, const PartDev* pd, int np, int counter_on,
                           const double body[3], float2* z, int* shell, int* counts, float* table, double* sum,
-                          float* u, float* drho, cudaStream_t s);
+                          float* u, float* drho, double tau, cudaStream_t s);
 }  // namespace lbsph
 
 using namespace lbsph;
@@ -1336,7 +1336,7 @@ extern "C" lb_status lb_stokes_field(lb_ctx* ctx, int32_t box, float* u_dev, flo
     CK(launch_stokes(B, reinterpret_cast<int*>(ctx->d_tmp), ctx->d_pd + B.pbeg, B.pcnt, d.counter_force, d.body_force,
                      ctx->d_stokes, reinterpret_cast<int*>(ctx->d_stokes + 2 * B.N), counts,
                      reinterpret_cast<float*>(counts + ctx->maxp + 1), ctx->d_sums, direct ? u_dev : out,
-                     direct ? drho_dev : out + 3 * B.N, s));
+                     direct ? drho_dev : out + 3 * B.N, d.tau, s));
     if (!direct) {
         CK(cudaMemcpyAsync(u_dev, out, 3ull * B.N * sizeof(float), cudaMemcpyDeviceToDevice, s));
         if (drho_dev) CK(cudaMemcpyAsync(drho_dev, out + 3 * B.N, (size_t)B.N * sizeof(float), cudaMemcpyDeviceToDevice, s));

@@ -43,16 +43,11 @@ __global__ void init_fluid_kernel(const BoxDev B, void* fbuf, const float* u, co
     const float rho = B.rho0f + dr;
     float du[3][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};   // du[a][b] = d_a u_b
     if (stress && fluid) {
-        const int nx = B.nx, ny = B.ny, nz = B.nz;
-        const int x = (int)(n % nx), y = (int)((n / nx) % ny), z = (int)(n / ((long long)nx * ny));
-        const long long row = (long long)nx * ny;
-        const long long yz = (long long)z * row + (long long)y * nx;
-        const long long nb[3][2] = {
-            {yz + (x == nx - 1 ? 0 : x + 1), yz + (x == 0 ? nx - 1 : x - 1)},
-            {(long long)z * row + (long long)(y == ny - 1 ? 0 : y + 1) * nx + x,
-             (long long)z * row + (long long)(y == 0 ? ny - 1 : y - 1) * nx + x},
-            {(long long)(z == nz - 1 ? 0 : z + 1) * row + (long long)y * nx + x,
-             (long long)(z == 0 ? nz - 1 : z - 1) * row + (long long)y * nx + x}};
+        const int nx = B.nx, ny = B.ny, nz = B.nz, m = (int)n, row = nx * ny;           // 19 N < 2^31
+        const int r = (int)((unsigned)m / (unsigned)nx), x = m - r * nx, z = div_magic(r, B.dy_m, B.dy_s), y = r - z * ny;
+        const int nb[3][2] = {{x == nx - 1 ? m + 1 - nx : m + 1, x == 0 ? m + nx - 1 : m - 1},
+                              {y == ny - 1 ? m + nx - row : m + nx, y == 0 ? m + row - nx : m - nx},
+                              {z == nz - 1 ? m - (nz - 1) * row : m + row, z == 0 ? m + (nz - 1) * row : m - row}};
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
@@ -80,22 +75,16 @@ __global__ void init_fluid_kernel(const BoxDev B, void* fbuf, const float* u, co
 
 // shell owner of a fluid node: the particle (p + 1) owning one of its six face
 // neighbours, 0 if none (periodic; the first one found if several)
-__device__ __forceinline__ int shell_owner(const int* owner, int nx, int ny, int nz, long long n)
+__device__ __forceinline__ int shell_owner(const int* owner, unsigned nx, unsigned ny, unsigned nz, unsigned n)
 {
-    const int x = (int)(n % nx), y = (int)((n / nx) % ny), z = (int)(n / ((long long)nx * ny));
-    const int xs[2] = {x == 0 ? nx - 1 : x - 1, x == nx - 1 ? 0 : x + 1};
-    const int ys[2] = {y == 0 ? ny - 1 : y - 1, y == ny - 1 ? 0 : y + 1};
-    const int zs[2] = {z == 0 ? nz - 1 : z - 1, z == nz - 1 ? 0 : z + 1};
-    const long long row = (long long)nx * ny;
+    const unsigned r = n / nx, x = n - r * nx, z = r / ny, y = r - z * ny, row = nx * ny;       // 19 N < 2^31
+    const int v[6] = {owner[n - x + (x == 0 ? nx - 1 : x - 1)], owner[(y == 0 ? n + row - nx : n - nx)],
+                      owner[(z == 0 ? n + (nz - 1) * row : n - row)], owner[n - x + (x == nx - 1 ? 0 : x + 1)],
+                      owner[(y == ny - 1 ? n + nx - row : n + nx)], owner[(z == nz - 1 ? n - (nz - 1) * row : n + row)]};
     int o = 0;
-    for (int k = 0; k < 2; ++k) {
-        const int a = owner[z * row + (long long)y * nx + xs[k]];
-        const int b = owner[z * row + (long long)ys[k] * nx + x];
-        const int c = owner[zs[k] * row + (long long)y * nx + x];
-        if (o == 0 && a > 0) o = a;
-        if (o == 0 && b > 0) o = b;
-        if (o == 0 && c > 0) o = c;
-    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        if (o == 0 && v[k] > 0) o = v[k];
     return o;
 }
 
@@ -128,18 +117,22 @@ __global__ void __launch_bounds__(256) shell_kernel(const Stokes S)
 {
     __shared__ int s_n;
     __shared__ bool s_last;
-    const long long n = blockIdx.x * 256ll + threadIdx.x;
     if (threadIdx.x == 0) s_n = 0;
     __syncthreads();
-    int e = -1;
-    if (n < S.N && S.owner[n] == 0) {
-        const int o = shell_owner(S.owner, S.nx, S.ny, S.nz, n);
-        e = o > 0 && o <= S.np ? o : 0;
+    int fluid = 0;
+    // a fixed number of blocks: with one per 256 nodes their counter atomics took 30 us at 128^3
+    for (long long n = blockIdx.x * 256ll + threadIdx.x; n < S.N; n += gridDim.x * 256ll) {
+        int e = -1;
+        if (S.owner[n] == 0) {
+            const int o = shell_owner(S.owner, S.nx, S.ny, S.nz, (unsigned)n);
+            e = o > 0 && o <= S.np ? o : 0;
+            ++fluid;
+        }
+        S.shell[n] = e;
+        if (e > 0) atomicAdd(S.counts + e, 1);
     }
-    if (n < S.N) S.shell[n] = e;
-    if (e > 0) atomicAdd(S.counts + e, 1);
-    const unsigned m = __ballot_sync(0xffffffffu, e >= 0);
-    if ((threadIdx.x & 31) == 0) atomicAdd(&s_n, __popc(m));
+    fluid = __reduce_add_sync(0xffffffffu, fluid);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&s_n, fluid);
     __syncthreads();
     if (threadIdx.x == 0) {
         atomicAdd(S.counts, s_n);
@@ -169,7 +162,8 @@ __global__ void __launch_bounds__(256) shell_kernel(const Stokes S)
 // sector), in place; the two fields of real data travel as real and imaginary part of one
 // complex field.  Traffic (16 bytes in, 16 out per node and pass, within L2 up to 128^3) and
 // the stages' shared-memory accesses bound a pass.  Measured at 128^3: seven passes of one
-// line per block over 3 + 4 complex fields took 1,270 us, the six passes here FFT_NOTE.
+// line per block over 3 + 4 complex fields took 1,270 us, the six passes here 158
+// (fft_kernel: 21 forward and 23 us each, 45 for the last with its sums).
 constexpr int FFT_T = 256, FFT_ST = 12;
 struct FftPlan {
     int n, ns_, L, lp;                  // stages, lines per block, padded pitch of a row of lines
@@ -434,20 +428,22 @@ __global__ void __launch_bounds__(256) shift_kernel(const Stokes S)
 // with a real and H2, D0, D2 are real: over the nine pairs of directions
 //   a = sum 2 w c Im h,  H2 = sum 2 w c c^T Re h,  D0 = sum 2 w r,  D2 = sum 6 w c c^T r,
 //   r = Re (1 - e) q = (1 + (1 - omega)) 2 sin^2(th/2) / |1 - (1 - omega) e|^2 >= 0,
-// without cancellation (D0 and D2 vanish like k^2).  With drho = i s,
-//   s = (fo a.g + 3 rho0 omega a.u) / D0,   (rho0 D2 + 3 rho0 omega^2 a a^T / D0) u = g/2 + fo H2 g - (omega fo a.g / D0) a
-// (fo = 3 (1 - omega/2)): a symmetric positive definite 3 x 3 system with real
-// coefficients for the real and the imaginary part of g, solved by cofactors.  The terms of one
-// direction are FP32; sums and solve are carried to twice FP32's digits (ff below).
+// without cancellation (D0 and D2 vanish like k^2).  With drho = i s and b = g/2 + fo H2 g
+// (fo = 3 (1 - omega/2)) the equations are real, for the real and the imaginary part of g alike:
+//   rho0 D2 u = b - omega a s,   (D0 + 3 omega^2 a.D2^-1 a) s = fo a.g + 3 omega a.D2^-1 b,
+// D2 symmetric positive definite, inverted by cofactors, and a scalar equation whose terms on
+// the left have one sign.  (One 3 x 3 system with the pressure eliminated is stiff along a by 1 / (nu k^2),
+// and its determinant loses the square of that.)  The terms of one direction are FP32; sums and
+// solve are carried to twice FP32's digits (ff below).
 // One thread takes a mode and its conjugate: the fields are real, so the transforms of two of
 // them come as one, Z(k) = X(k) + i Y(k), X(k) = (Z(k) + conj Z(-k)) / 2, and go back the
 // same way.  The k = 0 mode (mean flow and mass, set afterwards) and numerically singular
 // modes are zero; the 1/N of the inverse DFT is folded in.
 // Numbers as the unevaluated sum of two FP32 (Dekker, "A floating-point technique for
 // extending the available precision", 1971; Knuth's two-sum): 48 bits of significand from FP32
-// instructions, which this part issues 64 times as often as FP64 ones.  The system above loses a
-// factor of about 1 / k^2 (4e2 at an edge of 128, 4e5 at 4096) to the stiff longitudinal
-// direction: 2^-46 times that stays far below the FP32 rounding of its terms.
+// instructions, which this part issues 64 times as often as FP64 ones.  In u = D2^-1 (b - omega a s)
+// the longitudinal part cancels down to about nu k^2 of its terms (1e-4 at an edge of 64 and
+// tau = 0.52): 2^-46 over that stays far below the FP32 rounding of the directions' terms.
 struct ff {
     float h, l;
 };
@@ -490,14 +486,15 @@ __device__ __forceinline__ ff recip(ff a)
 }
 
 struct SteadyConst {
-    ff om, fo18, fo, six_rho, tro, inv_n;   // omega, fo / 18, fo, 6 / rho0, 3 rho0 omega, 1 / N
-    float om1, opm;                         // 1 - omega, 2 - omega
+    ff fo, fo18, om2, om18, om_18;          // fo, fo / 18, omega^2, 18 omega, omega / 18
+    ff six_rho_n, inv_n;                    // 6 / (rho0 N), 1 / N
+    float om, om1, opm;                     // omega, 1 - omega, 2 - omega
 };
 
 // One thread per mode of the planes z <= nz / 2 that comes no later than its conjugate.
 // Sums in units of 1/18: D0 = D0' / 18, a = a' / 18, H2 = H2' / 18, D2 = D2' / 6.
 // Measured at 128^3: 4,207 us as a complex 4 x 4 FP64 elimination with pivoting per mode,
-// STEADY_NOTE.
+// 102 us like this.
 __global__ void __launch_bounds__(128) steady_kernel(const Stokes S, const SteadyConst K)
 {
     const int nx = S.nx, ny = S.ny, nz = S.nz;
@@ -508,7 +505,8 @@ __global__ void __launch_bounds__(128) steady_kernel(const Stokes S, const Stead
     const int r2 = ((z == 0 ? 0 : nz - z) * ny + (y == 0 ? 0 : ny - y)) * nx + (x == 0 ? 0 : nx - x);
     if (r2 < r) return;
     const float2 z1 = S.z[r], z1c = S.z[r2], z2 = S.z[S.N + r];
-    const float fx = (float)x / nx, fy = (float)y / ny, fz = (float)z / nz;
+    // from the index nearer to zero, so that the small angles of both ends keep their digits
+    const float fx = (float)(2 * x > nx ? x - nx : x) / nx, fy = (float)(2 * y > ny ? y - ny : y) / ny, fz = (float)z / nz;
     const ff zero = {0.0f, 0.0f};
     ff a[3] = {zero, zero, zero}, D0 = zero;
     ff H[6] = {zero, zero, zero, zero, zero, zero}, D[6] = {zero, zero, zero, zero, zero, zero};      // xx yy zz xy xz yz
@@ -520,13 +518,14 @@ __global__ void __launch_bounds__(128) steady_kernel(const Stokes S, const Stead
         tp -= 2.0f * floorf(0.5f * tp + 0.5f);
         float sh, ch;
         sincospif(0.5f * tp, &sh, &ch);
-        const float s2 = sh * sh;
-        // |1 - (1 - omega) e|^2 as a sum of terms of one sign
-        const float dd = K.om1 >= 0.0f ? (1.0f - K.om1) * (1.0f - K.om1) + 4.0f * K.om1 * s2
-                                       : K.opm * K.opm - 4.0f * K.om1 * (ch * ch);
+        const float s2 = sh * sh, c2 = ch * ch;
+        // |1 - (1 - omega) e|^2 as a sum of terms of one sign, cos th - (1 - omega) from the half angle that is
+        // small where it cancels
+        const float dd = K.om1 >= 0.0f ? K.om * K.om + 4.0f * K.om1 * s2 : K.opm * K.opm - 4.0f * K.om1 * c2;
+        const float hn = K.om1 >= 0.0f ? K.om - 2.0f * s2 : 2.0f * c2 - K.opm;
         const float wt = m < 3 ? 2.0f : 1.0f;                       // 36 w
         const float id = wt / dd;
-        const float hre = (1.0f - K.om1 - 2.0f * s2) * id, him = -2.0f * sh * ch * id, rr = K.opm * (2.0f * s2) * id;
+        const float hre = hn * id, him = -2.0f * sh * ch * id, rr = K.opm * (2.0f * s2) * id;
         D0 = D0 + rr;
         if (cx) { a[0] = a[0] + (float)cx * him; H[0] = H[0] + hre; D[0] = D[0] + rr; }
         if (cy) { a[1] = a[1] + (float)cy * him; H[1] = H[1] + hre; D[1] = D[1] + rr; }
@@ -538,31 +537,30 @@ __global__ void __launch_bounds__(128) steady_kernel(const Stokes S, const Stead
     // [part][component] of g: real, imaginary
     const float g[2][3] = {{0.5f * (z1.x + z1c.x), 0.5f * (z1.y + z1c.y), z2.x}, {0.5f * (z1.y - z1c.y), 0.5f * (z1c.x - z1.x), z2.y}};
     float u[2][3] = {}, sd[2] = {};
-    const bool ok0 = r != 0 && D0.h > 0.0f;
-    const ff iD = recip(ok0 ? D0 : ff{1.0f, 0.0f}), oD = K.om * iD;
-    const ff t[3] = {a[0] * oD, a[1] * oD, a[2] * oD};
-    const ff v[3] = {t[0] * K.om, t[1] * K.om, t[2] * K.om};
-    const ff Mxx = D[0] + a[0] * v[0], Myy = D[1] + a[1] * v[1], Mzz = D[2] + a[2] * v[2];
-    const ff Mxy = D[3] + a[0] * v[1], Mxz = D[4] + a[0] * v[2], Myz = D[5] + a[1] * v[2];
-    const ff Cxx = Myy * Mzz - Myz * Myz, Cxy = Mxz * Myz - Mxy * Mzz, Cxz = Mxy * Myz - Mxz * Myy;
-    const ff Cyy = Mxx * Mzz - Mxz * Mxz, Cyz = Mxy * Mxz - Mxx * Myz, Czz = Mxx * Myy - Mxy * Mxy;
-    const ff det = Mxx * Cxx + Mxy * Cxy + Mxz * Cxz;
+    // E = D2'^-1 by cofactors (its eigenvalues lie close together), E a, and the pressure's factor
+    const ff Cxx = D[1] * D[2] - D[5] * D[5], Cxy = D[4] * D[5] - D[3] * D[2], Cxz = D[3] * D[5] - D[4] * D[1];
+    const ff Cyy = D[0] * D[2] - D[4] * D[4], Cyz = D[3] * D[4] - D[0] * D[5], Czz = D[0] * D[1] - D[3] * D[3];
+    const ff det = D[0] * Cxx + D[3] * Cxy + D[4] * Cxz;
     // numerically singular: a determinant below 1e-13 of the product of the diagonal
-    if (ok0 && det.h > 1e-13f * Mxx.h * Myy.h * Mzz.h) {
-        const ff idet = recip(det) * K.inv_n;
+    if (r != 0 && D0.h > 0.0f && det.h > 1e-13f * D[0].h * D[1].h * D[2].h) {
+        const ff idet = recip(det);
+        const ff ea[3] = {(Cxx * a[0] + Cxy * a[1] + Cxz * a[2]) * idet, (Cxy * a[0] + Cyy * a[1] + Cyz * a[2]) * idet,
+                          (Cxz * a[0] + Cyz * a[1] + Czz * a[2]) * idet};
+        const ff is = recip(D0 + K.om2 * (a[0] * ea[0] + a[1] * ea[1] + a[2] * ea[2]));
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
             const ff ag = a[0] * g[c][0] + a[1] * g[c][1] + a[2] * g[c][2];
-            const ff hx = H[0] * g[c][0] + H[3] * g[c][1] + H[4] * g[c][2] - ag * t[0];
-            const ff hy = H[3] * g[c][0] + H[1] * g[c][1] + H[5] * g[c][2] - ag * t[1];
-            const ff hz = H[4] * g[c][0] + H[5] * g[c][1] + H[2] * g[c][2] - ag * t[2];
-            const ff bx = (K.fo18 * hx + 0.5f * g[c][0]) * K.six_rho, by = (K.fo18 * hy + 0.5f * g[c][1]) * K.six_rho,
-                     bz = (K.fo18 * hz + 0.5f * g[c][2]) * K.six_rho;
-            const ff ux = (Cxx * bx + Cxy * by + Cxz * bz) * idet, uy = (Cxy * bx + Cyy * by + Cyz * bz) * idet,
-                     uz = (Cxz * bx + Cyz * by + Czz * bz) * idet;
-            const ff s = (K.fo * ag * K.inv_n + K.tro * (a[0] * ux + a[1] * uy + a[2] * uz)) * iD;
+            const ff bx = K.fo18 * (H[0] * g[c][0] + H[3] * g[c][1] + H[4] * g[c][2]) + 0.5f * g[c][0];
+            const ff by = K.fo18 * (H[3] * g[c][0] + H[1] * g[c][1] + H[5] * g[c][2]) + 0.5f * g[c][1];
+            const ff bz = K.fo18 * (H[4] * g[c][0] + H[5] * g[c][1] + H[2] * g[c][2]) + 0.5f * g[c][2];
+            const ff x0 = (Cxx * bx + Cxy * by + Cxz * bz) * idet, x1 = (Cxy * bx + Cyy * by + Cyz * bz) * idet,
+                     x2 = (Cxz * bx + Cyz * by + Czz * bz) * idet;
+            const ff s = (K.fo * ag + K.om18 * (a[0] * x0 + a[1] * x1 + a[2] * x2)) * is;
+            const ff q = K.om_18 * s;
+            const ff ux = (x0 - q * ea[0]) * K.six_rho_n, uy = (x1 - q * ea[1]) * K.six_rho_n, uz = (x2 - q * ea[2]) * K.six_rho_n;
+            const ff sn = s * K.inv_n;
             u[c][0] = ux.h + ux.l; u[c][1] = uy.h + uy.l; u[c][2] = uz.h + uz.l;
-            sd[c] = s.h + s.l;
+            sd[c] = sn.h + sn.l;
         }
     }
     // drho = i s: real part -Im s, imaginary part Re s
@@ -616,17 +614,17 @@ static FftPlan fft_plan(int n, float sign)
 // shift: 4 floats, done: 2 counters; u [3][N], drho [N] or null: the result
 cudaError_t launch_stokes(const BoxDev& B, const int* owner, const PartDev* pd, int np, int counter_on,
                           const double body[3], float2* z, int* shell, int* counts, float* table, double* sum, float* u,
-                          float* drho, cudaStream_t s)
+                          float* drho, double tau, cudaStream_t s)
 {
     cudaError_t e;
     Stokes S{};
     S.nx = B.nx; S.ny = B.ny; S.nz = B.nz; S.np = np; S.counter = counter_on; S.N = B.N;
     for (int k = 0; k < 3; ++k) S.body[k] = body[k];
-    S.rho0 = B.rho0; S.omega = (double)B.omega;
+    S.rho0 = B.rho0; S.omega = 1.0 / tau;        // in FP64: at tau = 0.52 an FP32 omega is worth 1e-6 of the viscosity
     // drho is of the order of mu u / r a few nodes from a particle: scaled so that neither of
     // the two fields that share a transform loses digits to the other
     int ex = 0;
-    std::frexp(4.0 / (B.rho0 * (1.0 / S.omega - 0.5) / 3.0), &ex);
+    std::frexp(0.5 / (B.rho0 * (1.0 / S.omega - 0.5) / 3.0), &ex);
     S.kappa = (float)std::ldexp(1.0, ex);
     S.owner = owner; S.pd = pd; S.shell = shell; S.counts = counts; S.table = table; S.sum = sum;
     S.shift = reinterpret_cast<float*>(sum + 4);
@@ -634,7 +632,8 @@ cudaError_t launch_stokes(const BoxDev& B, const int* owner, const PartDev* pd, 
     S.z = z; S.u = u; S.drho = drho;
     if ((e = cudaMemsetAsync(counts, 0, sizeof(int) * (np + 1), s)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(sum, 0, 4 * sizeof(double) + 4 * sizeof(float) + 2 * sizeof(unsigned), s)) != cudaSuccess) return e;
-    shell_kernel<<<nblk(S.N, 256), 256, 0, s>>>(S);
+    const unsigned g = nblk(S.N, 256) < 1216 ? nblk(S.N, 256) : 1216;
+    shell_kernel<<<g, 256, 0, s>>>(S);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     auto pass = [&](int mode, int ax, float sign) {
         FftPlan P = fft_plan(ax == 0 ? B.nx : (ax == 1 ? B.ny : B.nz), sign);
@@ -662,16 +661,15 @@ cudaError_t launch_stokes(const BoxDev& B, const int* owner, const PartDev* pd, 
     SteadyConst K;
     const double om = S.omega, fo = 3.0 * (1.0 - 0.5 * om);
     auto split = [](double v) { const float h = (float)v; return ff{h, (float)(v - (double)h)}; };
-    K.om = split(om); K.fo18 = split(fo / 18.0); K.fo = split(fo); K.six_rho = split(6.0 / S.rho0);
-    K.tro = split(3.0 * S.rho0 * om); K.inv_n = split(1.0 / (double)S.N);
-    K.om1 = (float)(1.0 - om); K.opm = (float)(2.0 - om);
+    K.fo = split(fo); K.fo18 = split(fo / 18.0); K.om2 = split(om * om); K.om18 = split(18.0 * om); K.om_18 = split(om / 18.0);
+    K.six_rho_n = split(6.0 / (S.rho0 * (double)S.N)); K.inv_n = split(1.0 / (double)S.N);
+    K.om = (float)om; K.om1 = (float)(1.0 - om); K.opm = (float)(2.0 - om);
     steady_kernel<<<nblk((long long)(B.nz / 2 + 1) * B.nx * B.ny, 128), 128, 0, s>>>(S, K);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     for (int ax = 2; ax > 0; --ax)
         if ((e = pass(FFT_INPLACE, ax, 1.0f)) != cudaSuccess) return e;
     if ((e = pass(FFT_LAST, 0, 1.0f)) != cudaSuccess) return e;
-    const unsigned g = nblk(S.N, 256);
-    shift_kernel<<<g < 1216 ? g : 1216, 256, 0, s>>>(S);
+    shift_kernel<<<g, 256, 0, s>>>(S);
     return cudaGetLastError();
 }
 
