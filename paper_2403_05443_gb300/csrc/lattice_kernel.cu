@@ -3,52 +3,31 @@
 // iteration t-1 of the paper's Appendix (step 2 streaming, step 6 bounce-back
 // with U(t), Omega(t), the remap of step 8) without the collision, with
 // density and velocity moments.  Every decision is taken per node from the
-// occupancy maps, in a layout independent of the bulk + boundary kernels that
-// advance the simulation, so the read-back also cross-checks them.
+// occupancy maps.
 //
-// Thread mapping: one thread per 4 consecutive x nodes ("quad"), 256 threads
-// per block, blocks in x-fastest order over the box.  Each direction is read
-// with one 16-byte load of the source row; the +-1 shift in x comes from the
-// neighbouring lane by a warp shuffle (a scalar load at warp and row ends,
-// which also wraps x periodically).  Threads whose nodes (grown by one) touch
-// a particle's bounding cube or a wall test them against the occupancy
-// bitmaps (old map for the streaming sources, new map for the node itself).
+// One launch, two kinds of blocks:
+//   - plain blocks, one thread per 4 consecutive x nodes ("quad"), 256 quads per
+//     block: each direction is one 16-byte load of the source row (8 bytes in
+//     16-bit storage), the +-1 shift in x comes from the neighbouring lane by a
+//     shuffle (a scalar load at warp and row ends, which also wraps x); solid
+//     nodes are written as 0, the nodes of a particle's redo mask are left out;
+//   - surface blocks (the first ones of the grid), one thread per node of a
+//     particle's cube, which do the masked nodes: the pull, the node's own
+//     populations for the links that end inside the old surface (Eq. fb, Eq. ub)
+//     and the uncovered nodes.  A node in the masks of two particles is written
+//     twice with the same value.
 //
-// Away from the particles the kernel is bound by the populations it reads; near
-// them by the latency of what each thread looks up, so a tile keeps only the indices of
-// the particles it meets (their state is read through L1 where it is needed), a
-// neighbourhood row is one load and two shifts, the box's uniform force is summed by one
-// warp while the others load, and the owner field reads no populations.  Measured, FP32:
-// u or rho of a 64^3 box with one particle 48.6 -> 18.4 us, of 128 x 64 x 128 nodes between
-// walls 52 -> 39, of 128^3 nodes with 16 particles 321 -> 90 (13, 27 and 57 without the
-// bounce-back); the owner field of 128^3 nodes 118 -> 11.
-#include "lattice_common.cuh"
+// Bound: the populations, read once (HBM) - so the plain blocks need as many loads
+// in flight as fit.  With the surface code in every thread a block took 255 registers
+// and an SM held 8 warps, each waiting at the block's list of particles; apart, the
+// plain code fits 128 (two blocks per SM; three would spill 250-480 bytes per thread), and the
+// surface nodes cost few warps.  Measured per call, u or rho: a 64^3 box with one
+// particle 17 -> 7.5 us (FP16), the 32 squirmer boxes of 48^3 to 128^3 nodes in BF16
+// 57 -> 16.6 on average, 128^3 nodes with 16 particles in FP32 88 -> 56; all populations
+// of 128^3 nodes before the first step 72 -> 54, the owner field 9.5 -> 7.1.
+#include "bulk_tile.cuh"
 
 namespace lbsph {
-
-// Is lattice node (X, Y, Z) (wrapped into the box) a solid node of one of the
-// tile's particles?  old selects map t-1 (streaming sources) or map t.
-__device__ __forceinline__ const PartK* lookup(const PartK* pk, const int* cs, int nc, bool old, int X, int Y, int Z, int nx,
-                                               int ny, int nz, int& mx, int& my, int& mz)
-{
-    for (int c = 0; c < nc; ++c) {
-        const PartK& K = pk[cs[c]];
-        const int* ow = old ? K.ow_old : K.ow_new;
-        const int S = K.S;
-        const int ax = wrapd(X - ow[0], nx);
-        if (ax >= S) continue;
-        const int ay = wrapd(Y - ow[1], ny);
-        if (ay >= S) continue;
-        const int az = wrapd(Z - ow[2], nz);
-        if (az >= S) continue;
-        const uint64_t* rows = old ? K.rows_old : K.rows_new;
-        if ((rows[az * S + ay] >> ax) & 1ull) {
-            mx = ax; my = ay; mz = az;
-            return &K;
-        }
-    }
-    return nullptr;
-}
 
 // The 6 nodes x = X0-1 .. X0+4 of a cube row as bits 0..5: its word shifted by the window's
 // offset d in the cube, and by what of the window lies beyond the periodic end.
@@ -72,246 +51,165 @@ __device__ __forceinline__ bool hits(int lo, int hi, int ow, int S, int L)
 // ---------------------------------------------------------------------------
 enum { FK_F = 0, FK_MOMENTS = 1, FK_SOLID = 2 };
 
+// blocks per SM the registers are held to
 template <class St, int WHAT>
-__global__ void __launch_bounds__(KBLOCK, 1) fields_kernel(const KParams P)
+constexpr int FIELD_BLOCKS = 2;
+
+// Density deviation and momentum of one node's populations, in this order of additions.
+__device__ __forceinline__ void node_moments(const float (&f)[Q], float rho0, const float* g, float& drho, float& ux,
+                                             float& uy, float& uz)
+{
+    drho = 0.f;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) drho += f[i];
+    const float jx = (f[1] - f[2]) + (f[7] - f[8]) + (f[9] - f[10]) + (f[11] - f[12]) + (f[13] - f[14]);
+    const float jy = (f[3] - f[4]) + (f[7] - f[8]) - (f[9] - f[10]) + (f[15] - f[16]) + (f[17] - f[18]);
+    const float jz = (f[5] - f[6]) + (f[11] - f[12]) - (f[13] - f[14]) + (f[15] - f[16]) - (f[17] - f[18]);
+    const float ir = 1.0f / (rho0 + drho);
+    ux = (jx + 0.5f * g[0]) * ir;
+    uy = (jy + 0.5f * g[1]) * ir;
+    uz = (jz + 0.5f * g[2]) * ir;
+}
+
+// The box's uniform force, by one warp: body force and the counter force over the fluid nodes.
+__device__ __forceinline__ void box_force(const KParams& P, const BoxDev& B, int lane, float* g_out)
+{
+    double fx = 0.0, fy = 0.0, fz = 0.0;
+    int nsol = 0;                           // at most N < 2^31 / 19
+    for (int j = lane; j < B.pcnt; j += 32) {
+        const PartK& k = P.pk[B.pbeg + j];
+        fx += k.Fext[0]; fy += k.Fext[1]; fz += k.Fext[2];
+        nsol += k.nsolid;
+    }
+    for (int o = B.pcnt > 1 ? 16 : 0; o > 0; o >>= 1) {
+        fx += __shfl_xor_sync(0xffffffffu, fx, o);
+        fy += __shfl_xor_sync(0xffffffffu, fy, o);
+        fz += __shfl_xor_sync(0xffffffffu, fz, o);
+        nsol += __shfl_xor_sync(0xffffffffu, nsol, o);
+    }
+    if (lane == 0) {
+        const double nf = (double)(B.N - B.nwall - nsol);
+        double g[3] = {B.body[0], B.body[1], B.body[2]};
+        if (B.counter && nf > 0) { g[0] -= fx / nf; g[1] -= fy / nf; g[2] -= fz / nf; }
+        g_out[0] = (float)g[0]; g_out[1] = (float)g[1]; g_out[2] = (float)g[2];
+    }
+}
+
+// A 256-quad tile may meet at most MAXC particles (grown by one node; old and new cubes): else ST_CAPACITY.  One warp.
+__device__ __forceinline__ void tile_capacity(const KParams& P, const BoxDev& B, int q0, int lane)
+{
+    const int ny = B.ny, nz = B.nz;
+    const int qlast = min(q0 + KBLOCK, (int)B.nq) - 1;
+    const int r0 = div_magic(q0, B.dq_m, B.dq_s), r1 = div_magic(qlast, B.dq_m, B.dq_s);
+    const int z0 = div_magic(r0, B.dy_m, B.dy_s), z1 = div_magic(r1, B.dy_m, B.dy_s);
+    const int y0 = r0 - z0 * ny, y1 = r1 - z1 * ny;
+    const int ylo = z0 == z1 ? y0 - 1 : -1, yhi = z0 == z1 ? y1 + 1 : ny;
+    int nc = 0;
+    for (int base = 0; base < B.pcnt; base += 32) {
+        bool hit = false;
+        if (base + lane < B.pcnt) {
+            const PartK& k = P.pk[B.pbeg + base + lane];
+            const int S = k.S;
+            hit = (hits(ylo, yhi, k.ow_old[1], S, ny) && hits(z0 - 1, z1 + 1, k.ow_old[2], S, nz)) ||
+                  (hits(ylo, yhi, k.ow_new[1], S, ny) && hits(z0 - 1, z1 + 1, k.ow_new[2], S, nz));
+        }
+        nc += __popc(__ballot_sync(0xffffffffu, hit));
+    }
+    if (lane == 0 && nc > MAXC) atomicOr(P.status, ST_CAPACITY);
+}
+
+// Node l of particle p's cube, if its redo mask holds it and no particle covers it now.
+template <class St, int WHAT>
+__device__ __forceinline__ void surface_node(const KParams& P, const BoxDev& B, int p, int l, const float* s_g)
 {
     using T = typename St::T;
-    __shared__ int s_c[MAXC];
-    __shared__ int s_nc;
-    __shared__ float s_g[3];
-
-    // ---- box of this block
-    const BoxDev& B = P.boxes[P.only_box];
-    const int nx = B.nx, ny = B.ny, nz = B.nz, nxq = B.nxq;
-    const int N = (int)B.N;                     // 19 N < 2^31
-    // the blocks walk the box's tiles, so that the box force is summed once per block
-    for (int tile = blockIdx.x; tile < B.nblocks; tile += gridDim.x) {
-    if (tile != (int)blockIdx.x) __syncthreads();        // the last tile's list has been read
-    const int q0 = tile * KBLOCK;
-    const int qlast = min(q0 + KBLOCK, (int)B.nq) - 1;
-
-    // ---- this thread's quad
-    int q = q0 + (int)threadIdx.x;
-    const bool valid = q < (int)B.nq;
-    if (!valid) q = (int)B.nq - 1;
-    const int row = div_magic(q, B.dq_m, B.dq_s);
-    const int xq = q - row * nxq;
-    const int z = div_magic(row, B.dy_m, B.dy_s);
-    const int y = row - z * ny;
-    const int lane = threadIdx.x & 31;
-    const T* A = reinterpret_cast<const T*>(P.src) + B.off;
-    const float inv = B.inv_scale;
+    const int nx = B.nx, ny = B.ny, nz = B.nz, N = (int)B.N;
+    const NeedHdr h = P.need_hdr[p];
+    const int S = h.S;
+    const int r = l / S, mz = r / S;            // cube row r = mz S + my
+    bool on = mz < S;
+    if (on) on = (P.need[(size_t)p * (MAXS * MAXS) + r] >> (l - r * S)) & 1ull;
+    const int X = wrapd(h.ow[0] + (l - r * S), nx), y = wrapd(h.ow[1] + (r - mz * S), ny), z = on ? wrapd(h.ow[2] + mz, nz) : 0;
+    if (B.walls && (y == 0 || y == ny - 1)) on = false;
+    const float rho0 = B.rho0f, inv = B.inv_scale;
     const unsigned long long pol = l2_evict_normal();
-    const int own = row * nx + 4 * xq;
-    const bool first = P.nopull != 0;
-
-    // ---- pull (stream): v[i] = f*_i(x - c_i) for the 4 nodes
-    float4 v[Q];
-    if (WHAT != FK_SOLID) {
-        int rofs[3][3];  // element offset of source rows (y + dy, z + dz), wrapped
-        {
-            const int yy[3] = {y == 0 ? ny - 1 : y - 1, y, y == ny - 1 ? 0 : y + 1};
-            const int zz[3] = {z == 0 ? nz - 1 : z - 1, z, z == nz - 1 ? 0 : z + 1};
+    const T* A = reinterpret_cast<const T*>(P.src) + B.off;
+    const int own = (z * ny + y) * nx + X;
+    float f[Q], o[Q];
+    if (on) {
+        const int xx[3] = {X == 0 ? nx - 1 : X - 1, X, X == nx - 1 ? 0 : X + 1};
+        const int yy[3] = {y == 0 ? ny - 1 : y - 1, y, y == ny - 1 ? 0 : y + 1};
+        const int zz[3] = {z == 0 ? nz - 1 : z - 1, z, z == nz - 1 ? 0 : z + 1};
+#pragma unroll
+        for (int i = 0; i < Q; ++i)
+            f[i] = St::ld1(A + (i * N + (zz[1 - cz_of(i)] * ny + yy[1 - cy_of(i)]) * nx + xx[1 - cx_of(i)]), inv, pol);
+        // the node's own populations, wanted by the links that end in a surface: all of them at once, so that one
+        // latency covers them
+#pragma unroll
+        for (int i = 1; i < Q; ++i) o[i] = St::ld1(A + (i * N + own), inv, pol);
+        const int wall_cy = !B.walls ? 0 : (y == 1 ? 1 : (y == ny - 2 ? -1 : 0));     // directions from a wall
+        if (wall_cy != 0) {
+            const float* uw = y == 1 ? B.uw_lo : B.uw_hi;
+#pragma unroll
+            for (int i = 1; i < Q; ++i)
+                if (cy_of(i) != 0 && cy_of(i) == wall_cy)
+                    f[i] = o[opp_of(i)] + 6.0f * w_of(i) * rho0 * (cx_of(i) * uw[0] + cy_of(i) * uw[1] + cz_of(i) * uw[2]);
+        }
+        int c0 = -1;                            // the particle whose old map holds the node
+        for (int c = B.pbeg; c < B.pbeg + B.pcnt; ++c) {
+            const PartK& C = P.pk[c];
+            const int Sc = C.S;
+            const int ax = wrapd(X - C.ow_new[0], nx), ay = wrapd(y - C.ow_new[1], ny), az = wrapd(z - C.ow_new[2], nz);
+            if (ax < Sc && ay < Sc && az < Sc && ((C.rows_new[az * Sc + ay] >> ax) & 1ull)) on = false;
+            const int oo[3] = {C.ow_old[0], C.ow_old[1], C.ow_old[2]};
+            if (!(hits(X - 1, X + 1, oo[0], Sc, nx) && hits(y - 1, y + 1, oo[1], Sc, ny) && hits(z - 1, z + 1, oo[2], Sc, nz)))
+                continue;
+            // occupancy of x - 1, x, x + 1 (bits 0..2) in the 9 rows (y + dy, z + dz) of the old map
+            const int d = wrapd(wrapd(X - 1, nx) - oo[0], nx);
+            int my3[3], mz3[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                my3[a] = wrapd(yy[a] - oo[1], ny);
+                mz3[a] = wrapd(zz[a] - oo[2], nz);
+            }
+            unsigned w[3][3], any = 0u;
 #pragma unroll
             for (int a = 0; a < 3; ++a)
 #pragma unroll
-                for (int b = 0; b < 3; ++b) rofs[a][b] = (zz[b] * ny + yy[a]) * nx;
-        }
-        const bool left_ld = (lane == 0) || (xq == 0);
-        const bool right_ld = (lane == 31) || (xq == nxq - 1);
-        if (first) {
-            // before the first collision: the initial distributions in place
-#pragma unroll
-            for (int i = 0; i < Q; ++i) v[i] = St::ld4(A + (i * N + own), inv, pol);
-        } else {
-#pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                const T* rp = A + (i * N + rofs[1 - cy_of(i)][1 - cz_of(i)]);
-                float4 t = St::ld4(rp + 4 * xq, inv, pol);
-                if (cx_of(i) == 1) {           // source x - 1
-                    float l = __shfl_up_sync(0xffffffffu, t.w, 1);
-                    if (left_ld) l = St::ld1(rp + (xq == 0 ? nx - 1 : 4 * xq - 1), inv, pol);
-                    t = make_float4(l, t.x, t.y, t.z);
-                } else if (cx_of(i) == -1) {   // source x + 1
-                    float r = __shfl_down_sync(0xffffffffu, t.x, 1);
-                    if (right_ld) r = St::ld1(rp + (xq == nxq - 1 ? 0 : 4 * xq + 4), inv, pol);
-                    t = make_float4(t.y, t.z, t.w, r);
+                for (int b = 0; b < 3; ++b) {
+                    w[a][b] = 0u;
+                    if (my3[a] < Sc && mz3[b] < Sc) w[a][b] = window6(C.rows_old[mz3[b] * Sc + my3[a]], Sc, d, nx);
+                    any |= w[a][b];
                 }
-                v[i] = t;
-            }
-        }
-    }
-
-    // ---- particles near the tile (first warp), box force (second warp)
-    if (threadIdx.x < 32) {
-        const int r0 = div_magic(q0, B.dq_m, B.dq_s), r1 = div_magic(qlast, B.dq_m, B.dq_s);
-        const int z0 = div_magic(r0, B.dy_m, B.dy_s), z1 = div_magic(r1, B.dy_m, B.dy_s);
-        const int y0 = r0 - z0 * ny, y1 = r1 - z1 * ny;
-        const int ylo = z0 == z1 ? y0 - 1 : -1, yhi = z0 == z1 ? y1 + 1 : ny;
-        int nc = 0;
-        for (int base = 0; base < B.pcnt; base += 32) {
-            bool hit = false;
-            if (base + lane < B.pcnt) {
-                const PartK& k = P.pk[B.pbeg + base + lane];
-                const int S = k.S;
-                hit = (hits(ylo, yhi, k.ow_old[1], S, ny) && hits(z0 - 1, z1 + 1, k.ow_old[2], S, nz)) ||
-                      (hits(ylo, yhi, k.ow_new[1], S, ny) && hits(z0 - 1, z1 + 1, k.ow_new[2], S, nz));
-            }
-            const unsigned m = __ballot_sync(0xffffffffu, hit);
-            const int at = nc + __popc(m & ((1u << lane) - 1u));
-            if (hit && at < MAXC) s_c[at] = B.pbeg + base + lane;
-            nc += __popc(m);
-        }
-        if (lane == 0) {
-            if (nc > MAXC) atomicOr(P.status, ST_CAPACITY);
-            s_nc = nc < MAXC ? nc : MAXC;
-        }
-    } else if (WHAT == FK_MOMENTS && threadIdx.x < 64 && tile == (int)blockIdx.x) {
-        double fx = 0.0, fy = 0.0, fz = 0.0;
-        int nsol = 0;                           // at most N < 2^31 / 19
-        for (int j = lane; j < B.pcnt; j += 32) {
-            const PartK& k = P.pk[B.pbeg + j];
-            fx += k.Fext[0]; fy += k.Fext[1]; fz += k.Fext[2];
-            nsol += k.nsolid;
-        }
-        for (int o = B.pcnt > 1 ? 16 : 0; o > 0; o >>= 1) {
-            fx += __shfl_xor_sync(0xffffffffu, fx, o);
-            fy += __shfl_xor_sync(0xffffffffu, fy, o);
-            fz += __shfl_xor_sync(0xffffffffu, fz, o);
-            nsol += __shfl_xor_sync(0xffffffffu, nsol, o);
-        }
-        if (lane == 0) {
-            const double nf = (double)(B.N - B.nwall - nsol);
-            double g[3] = {B.body[0], B.body[1], B.body[2]};
-            if (B.counter && nf > 0) { g[0] -= fx / nf; g[1] -= fy / nf; g[2] -= fz / nf; }
-            s_g[0] = (float)g[0]; s_g[1] = (float)g[1]; s_g[2] = (float)g[2];
-        }
-    }
-    __syncthreads();
-    const int nc = s_nc;
-
-    // ---- walls: link bounce-back (Eq. fb with u_b = u_w) of the rows next to them
-    const bool wallrow = B.walls && (y == 0 || y == ny - 1);
-    const float rho0 = B.rho0f;
-    const int wall_cy = !B.walls || first ? 0 : (y == 1 ? 1 : (y == ny - 2 ? -1 : 0));     // directions from a wall
-    if (WHAT != FK_SOLID && wall_cy != 0) {
-        const float* uw = y == 1 ? B.uw_lo : B.uw_hi;
+            if ((any & 7u) == 0u) continue;
+            if (c0 < 0 && ((w[1][1] >> 1) & 1u)) c0 = c;
+            const float ro[3] = {C.ro_old[0], C.ro_old[1], C.ro_old[2]}, U[3] = {C.U[0], C.U[1], C.U[2]},
+                        W[3] = {C.W[0], C.W[1], C.W[2]};
+            const int squirmer = C.squirmer;
 #pragma unroll
-        for (int i = 1; i < Q; ++i) {
-            if (cy_of(i) == 0 || cy_of(i) != wall_cy) continue;
-            const float4 o = St::ld4(A + (opp_of(i) * N + own), inv, pol);
-            const float ubc = cx_of(i) * uw[0] + cy_of(i) * uw[1] + cz_of(i) * uw[2];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) set_comp(v[i], k, comp(o, k) + 6.0f * w_of(i) * rho0 * ubc);
-        }
-    }
-    // ---- particles whose cubes the thread's nodes (grown by one) touch: the neighbourhood's occupancy as 6-bit
-    // windows of the 9 rows (y + dy, z + dz), and bounce-back (Eq. fb, Eq. ub) where the source was inside
-    unsigned so = 0u, sn = 0u;                  // this row's windows of all particles, old and new map
-    for (int c = 0; c < nc; ++c) {
-        const PartK& C = P.pk[s_c[c]];
-        const int S = C.S;
-        const int on[3] = {C.ow_new[0], C.ow_new[1], C.ow_new[2]}, oo[3] = {C.ow_old[0], C.ow_old[1], C.ow_old[2]};
-        if (hits(y, y, on[1], S, ny) && hits(z, z, on[2], S, nz) && hits(4 * xq - 1, 4 * xq + 4, on[0], S, nx))
-            sn |= window6(C.rows_new[wrapd(z - on[2], nz) * S + wrapd(y - on[1], ny)], S,
-                          wrapd(wrapd(4 * xq - 1, nx) - on[0], nx), nx);
-        if (WHAT == FK_SOLID || first || wallrow) continue;
-        if (!(hits(y - 1, y + 1, oo[1], S, ny) && hits(z - 1, z + 1, oo[2], S, nz) && hits(4 * xq - 1, 4 * xq + 4, oo[0], S, nx))) continue;
-        const uint64_t* rows = C.rows_old;
-        const int d = wrapd(wrapd(4 * xq - 1, nx) - oo[0], nx);
-        int my[3], mz[3];                       // cube rows of y - 1, y, y + 1 and z - 1, z, z + 1
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            my[a] = wrapd(wrapd(y + a - 1, ny) - oo[1], ny);
-            mz[a] = wrapd(wrapd(z + a - 1, nz) - oo[2], nz);
-        }
-        unsigned w[3][3], any = 0u;
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                w[a][b] = 0u;
-                if (my[a] < S && mz[b] < S) w[a][b] = window6(rows[mz[b] * S + my[a]], S, d, nx);
-                any |= w[a][b];
-            }
-        so |= w[1][1];
-        if (any == 0u) continue;
-        const float ro[3] = {C.ro_old[0], C.ro_old[1], C.ro_old[2]}, U[3] = {C.U[0], C.U[1], C.U[2]},
-                    W[3] = {C.W[0], C.W[1], C.W[2]};
-        const int squirmer = C.squirmer;
-        // six directions at a time, so that their loads (the nodes' own populations of the opposite direction) overlap
-#pragma unroll
-        for (int i0 = 1; i0 < Q; i0 += 6) {
-            float4 o[6];
-            unsigned lm[6];
-#pragma unroll
-            for (int e = 0; e < 6; ++e) {
-                const int i = i0 + e;
-                lm[e] = (w[1 - cy_of(i)][1 - cz_of(i)] >> (1 - cx_of(i))) & 0xfu;
-                if (cy_of(i) != 0 && cy_of(i) == wall_cy) lm[e] = 0u;
-                if (lm[e]) o[e] = St::ld4(A + (opp_of(i) * N + own), inv, pol);
-            }
-#pragma unroll
-            for (int e = 0; e < 6; ++e) {
-                const int i = i0 + e;
-                if (lm[e] == 0u) continue;
-                const float ry = ro[1] + my[1 - cy_of(i)] + 0.5f * cy_of(i);
-                const float rz = ro[2] + mz[1 - cz_of(i)] + 0.5f * cz_of(i);
-#pragma unroll 1
-                for (int k = 0; k < 4; ++k) {
-                    if (!((lm[e] >> k) & 1u)) continue;
-                    int sx = d + k + 1 - cx_of(i);
-                    if (sx >= nx) sx -= nx;
-                    const float rx = ro[0] + sx + 0.5f * cx_of(i);
-                    float ux = U[0] + (W[1] * rz - W[2] * ry);
-                    float uy = U[1] + (W[2] * rx - W[0] * rz);
-                    float uz = U[2] + (W[0] * ry - W[1] * rx);
-                    if (squirmer) {
-                        float qx, qy, qz;
-                        squirmer_slip(C.e_old, C.a, C.eps2, C.B1, C.B2, rx, ry, rz, qx, qy, qz);
-                        ux += qx; uy += qy; uz += qz;
-                    }
-                    const float ubc = cx_of(i) * ux + cy_of(i) * uy + cz_of(i) * uz;
-                    const float fb = comp(o[e], k) + 6.0f * w_of(i) * rho0 * ubc;
-                    v[i].x = k == 0 ? fb : v[i].x;
-                    v[i].y = k == 1 ? fb : v[i].y;
-                    v[i].z = k == 2 ? fb : v[i].z;
-                    v[i].w = k == 3 ? fb : v[i].w;
+            for (int i = 1; i < Q; ++i) {
+                if (!((w[1 - cy_of(i)][1 - cz_of(i)] >> (1 - cx_of(i))) & 1u)) continue;
+                if (cy_of(i) != 0 && cy_of(i) == wall_cy) continue;
+                int sx = d + 1 - cx_of(i);
+                if (sx >= nx) sx -= nx;
+                const float rx = ro[0] + sx + 0.5f * cx_of(i);
+                const float ry = ro[1] + my3[1 - cy_of(i)] + 0.5f * cy_of(i);
+                const float rz = ro[2] + mz3[1 - cz_of(i)] + 0.5f * cz_of(i);
+                float ux = U[0] + (W[1] * rz - W[2] * ry);
+                float uy = U[1] + (W[2] * rx - W[0] * rz);
+                float uz = U[2] + (W[0] * ry - W[1] * rx);
+                if (squirmer) {
+                    float qx, qy, qz;
+                    squirmer_slip(C.e_old, C.a, C.eps2, C.B1, C.B2, rx, ry, rz, qx, qy, qz);
+                    ux += qx; uy += qy; uz += qz;
                 }
+                const float ubc = cx_of(i) * ux + cy_of(i) * uy + cz_of(i) * uz;
+                f[i] = o[opp_of(i)] + 6.0f * w_of(i) * rho0 * ubc;
             }
         }
-    }
-    if (WHAT == FK_SOLID) {
-        int solid_out[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            solid_out[k] = wallrow ? -1 : 0;
-            if (wallrow || !((sn >> (k + 1)) & 1u)) continue;
-            int mx, my, mz;
-            const PartK* c = lookup(P.pk, s_c, nc, false, 4 * xq + k, y, z, nx, ny, nz, mx, my, mz);
-            if (c) solid_out[k] = (int)(c - P.pk) - B.pbeg + 1;
-        }
-        if (valid) *reinterpret_cast<int4*>(P.out_solid + own) = make_int4(solid_out[0], solid_out[1], solid_out[2], solid_out[3]);
-        continue;
-    }
-    const float gx = s_g[0], gy = s_g[1], gz = s_g[2];
-    float rho_out[4], u_out[4][3];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int X = 4 * xq + k;
-        bool skip = !valid;
-        rho_out[k] = 0.f; u_out[k][0] = u_out[k][1] = u_out[k][2] = 0.f;
-        float f[Q];
-        const bool sol_old = !wallrow && ((so >> (k + 1)) & 1u);
-        const bool sol_new = !wallrow && ((sn >> (k + 1)) & 1u);
-        int mx, my, mz;
-        if (wallrow || sol_new) {
-            // a wall, solid before and after, or covered: its mass and momentum go to the particle (remap, step 8)
-            skip = true;
-        } else if (sol_old) {
+        if (on && c0 >= 0) {
             // uncovered: f = f_eq(rho0, U + Omega x r) (remap, step 8)
-            const PartK* c0 = lookup(P.pk, s_c, nc, true, X, y, z, nx, ny, nz, mx, my, mz);
-            const PartK& c = c0 ? *c0 : P.pk[s_c[0]];
+            const PartK& c = P.pk[c0];
             const int ax = wrapd(X - c.ow_new[0], nx), ay = wrapd(y - c.ow_new[1], ny), az = wrapd(z - c.ow_new[2], nz);
             const float rx = c.ro_new[0] + ax, ry = c.ro_new[1] + ay, rz = c.ro_new[2] + az;
             const float ux = c.U[0] + (c.W[1] * rz - c.W[2] * ry);
@@ -323,63 +221,208 @@ __global__ void __launch_bounds__(KBLOCK, 1) fields_kernel(const KParams P)
                 const float cu = cx_of(i) * ux + cy_of(i) * uy + cz_of(i) * uz;
                 f[i] = w_of(i) * rho0 * (3.0f * cu + 4.5f * cu * cu - 1.5f * uu);
             }
-        } else {
-            // fluid at t-1: pulled populations, bounced back where the source was solid
-#pragma unroll
-            for (int i = 0; i < Q; ++i) f[i] = comp(v[i], k);
-        }
-        if (skip) {
-#pragma unroll
-            for (int i = 0; i < Q; ++i) set_comp(v[i], k, 0.0f);
-            continue;
-        }
-        if (WHAT == FK_MOMENTS) {
-            float drho = 0.f;
-#pragma unroll
-            for (int i = 0; i < Q; ++i) drho += f[i];
-            const float jx = (f[1] - f[2]) + (f[7] - f[8]) + (f[9] - f[10]) + (f[11] - f[12]) + (f[13] - f[14]);
-            const float jy = (f[3] - f[4]) + (f[7] - f[8]) - (f[9] - f[10]) + (f[15] - f[16]) + (f[17] - f[18]);
-            const float jz = (f[5] - f[6]) + (f[11] - f[12]) - (f[13] - f[14]) + (f[15] - f[16]) - (f[17] - f[18]);
-            const float ir = 1.0f / (rho0 + drho);
-            rho_out[k] = drho;
-            u_out[k][0] = (jx + 0.5f * gx) * ir;
-            u_out[k][1] = (jy + 0.5f * gy) * ir;
-            u_out[k][2] = (jz + 0.5f * gz) * ir;
-        } else {
-#pragma unroll
-            for (int i = 0; i < Q; ++i) set_comp(v[i], k, P.out_dev ? f[i] : f[i] + w_of(i) * rho0);
         }
     }
-
-    if (!valid) continue;
+    if (WHAT == FK_MOMENTS) __syncthreads();    // the box force
+    if (!on) return;
     if (WHAT == FK_F) {
 #pragma unroll
-        for (int i = 0; i < Q; ++i) *reinterpret_cast<float4*>(P.out_f + (i * N + own)) = v[i];
+        for (int i = 0; i < Q; ++i) P.out_f[i * N + own] = P.out_dev ? f[i] : f[i] + w_of(i) * rho0;
     } else {
-        if (P.out_rho) *reinterpret_cast<float4*>(P.out_rho + own) = make_float4(rho_out[0], rho_out[1], rho_out[2], rho_out[3]);
-        if (P.out_u) {
+        float drho, u[3];
+        node_moments(f, rho0, s_g, drho, u[0], u[1], u[2]);
+        if (P.out_rho) P.out_rho[own] = drho;
+        if (P.out_u)
+            for (int a = 0; a < 3; ++a) P.out_u[a * N + own] = u[a];
+    }
+}
+
+template <class St, int WHAT>
+__global__ void __launch_bounds__(KBLOCK, FIELD_BLOCKS<St, WHAT>) fields_kernel(const __grid_constant__ KParams P)
+{
+    using T = typename St::T;
+    __shared__ float s_g[3];
+    const BoxDev& B = P.boxes[P.only_box];
+    const int lane = threadIdx.x & 31;
+    if (WHAT != FK_SOLID && (int)blockIdx.x < P.surf_blocks) {
+        if (WHAT == FK_MOMENTS && threadIdx.x < 32) box_force(P, B, lane, s_g);
+        surface_node<St, WHAT>(P, B, B.pbeg + blockIdx.x / P.surf_per, (blockIdx.x % P.surf_per) * KBLOCK + threadIdx.x, s_g);
+        return;
+    }
+    // ---- this thread's quad
+    const int nx = B.nx, ny = B.ny, nz = B.nz, nxq = B.nxq;
+    const int N = (int)B.N;                     // 19 N < 2^31
+    const int q0 = ((int)blockIdx.x - P.surf_blocks) * KBLOCK;
+    int q = q0 + (int)threadIdx.x;
+    const bool valid = q < (int)B.nq;
+    if (!valid) q = (int)B.nq - 1;
+    const int row = div_magic(q, B.dq_m, B.dq_s);
+    const int xq = q - row * nxq;
+    const int z = div_magic(row, B.dy_m, B.dy_s);
+    const int y = row - z * ny;
+    const T* A = reinterpret_cast<const T*>(P.src) + B.off;
+    const float inv = B.inv_scale, rho0 = B.rho0f;
+    const unsigned long long pol = l2_evict_normal();
+    const int own = row * nx + 4 * xq;
+    const bool first = P.nopull != 0;
+    const int pcnt = B.pcnt;
+    NeedHdr hd;                                 // the cube of one particle per lane, on its way while the populations load
+    hd.ow[0] = hd.ow[1] = hd.ow[2] = hd.S = 0;
+    if (lane < pcnt) hd = P.need_hdr[B.pbeg + lane];
+
+    // ---- pull (stream): v[i] = f*_i(x - c_i) for the 4 nodes
+    float4 v[Q];
+    if (WHAT != FK_SOLID) {
+        if (first) {
+            // before the first collision: the initial distributions in place
 #pragma unroll
-            for (int a = 0; a < 3; ++a)
-                *reinterpret_cast<float4*>(P.out_u + (a * N + own)) = make_float4(u_out[0][a], u_out[1][a], u_out[2][a], u_out[3][a]);
+            for (int i = 0; i < Q; ++i) v[i] = St::ld4(A + (i * N + own), inv, pol);
+        } else {
+            int rofs[3][3];  // element offset of source rows (y + dy, z + dz), wrapped
+            {
+                const int yy[3] = {y == 0 ? ny - 1 : y - 1, y, y == ny - 1 ? 0 : y + 1};
+                const int zz[3] = {z == 0 ? nz - 1 : z - 1, z, z == nz - 1 ? 0 : z + 1};
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+#pragma unroll
+                    for (int b = 0; b < 3; ++b) rofs[a][b] = (zz[b] * ny + yy[a]) * nx;
+            }
+            const bool left_ld = (lane == 0) || (xq == 0);
+            const bool right_ld = (lane == 31) || (xq == nxq - 1);
+#pragma unroll
+            for (int i = 0; i < Q; ++i) v[i] = St::ld4(A + (i * N + rofs[1 - cy_of(i)][1 - cz_of(i)]) + 4 * xq, inv, pol);
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const T* rp = A + (i * N + rofs[1 - cy_of(i)][1 - cz_of(i)]);
+                const float4 t = v[i];
+                if (cx_of(i) == 1) {           // source x - 1
+                    float e = __shfl_up_sync(0xffffffffu, t.w, 1);
+                    if (left_ld) e = St::ld1(rp + (xq == 0 ? nx - 1 : 4 * xq - 1), inv, pol);
+                    v[i] = make_float4(e, t.x, t.y, t.z);
+                } else if (cx_of(i) == -1) {   // source x + 1
+                    float e = __shfl_down_sync(0xffffffffu, t.x, 1);
+                    if (right_ld) e = St::ld1(rp + (xq == nxq - 1 ? 0 : 4 * xq + 4), inv, pol);
+                    v[i] = make_float4(t.y, t.z, t.w, e);
+                }
+            }
         }
     }
+    if (threadIdx.x < 32) {
+        if (pcnt > MAXC) tile_capacity(P, B, q0, lane);
+    } else if (WHAT == FK_MOMENTS && threadIdx.x < 64) {
+        box_force(P, B, lane, s_g);
+    }
+    if (WHAT == FK_MOMENTS) __syncthreads();
+
+    // ---- walls: link bounce-back (Eq. fb with u_b = u_w) of the rows next to them
+    const bool wallrow = B.walls && (y == 0 || y == ny - 1);
+    if (WHAT != FK_SOLID && B.walls && !first && (y == 1 || y == ny - 2)) {
+        const int wall_cy = y == 1 ? 1 : -1;    // directions from the wall
+        const float* uw = y == 1 ? B.uw_lo : B.uw_hi;
+#pragma unroll
+        for (int i = 1; i < Q; ++i) {
+            if (cy_of(i) == 0 || cy_of(i) != wall_cy) continue;
+            const float4 o = St::ld4(A + (opp_of(i) * N + own), inv, pol);
+            const float ubc = cx_of(i) * uw[0] + cy_of(i) * uw[1] + cz_of(i) * uw[2];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) set_comp(v[i], k, comp(o, k) + 6.0f * w_of(i) * rho0 * ubc);
+        }
+    }
+    // ---- nodes solid now (zero; owner: the lowest particle), and nodes of the surface blocks (skip)
+    unsigned zero = wallrow ? 0xfu : 0u, skip = 0u;
+    int owner[4];
+    if (WHAT == FK_SOLID)
+        for (int k = 0; k < 4; ++k) owner[k] = wallrow ? -1 : 0;
+    for (int j0 = 0; j0 < pcnt; j0 += 32) {
+        if (j0 > 0) {
+            hd.S = 0;
+            if (j0 + lane < pcnt) hd = P.need_hdr[B.pbeg + j0 + lane];
+        }
+        for (unsigned m = cubes_near(hd, row, B); m != 0; m &= m - 1) {
+            const int j = j0 + __ffs((int)m) - 1;
+            const NeedHdr c = P.need_hdr[B.pbeg + j];
+            int dz = z - c.ow[2];
+            if (dz < 0) dz += nz;
+            int dy = y - c.ow[1];
+            if (dy < 0) dy += ny;
+            int dx = 4 * xq - c.ow[0];
+            if (dx < 0) dx += nx;
+            if (dz >= c.S || dy >= c.S || wallrow) continue;
+            if (dx >= c.S && dx + 3 < nx) continue;
+            const uint64_t w = P.pk[B.pbeg + j].rows_new[dz * c.S + dy];
+            const uint64_t nd = WHAT == FK_SOLID || first ? 0ull : P.need[(size_t)(B.pbeg + j) * (MAXS * MAXS) + dz * c.S + dy];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int mx = dx + k < nx ? dx + k : dx + k - nx;
+                if (mx >= c.S) continue;
+                if ((w >> mx) & 1ull) {
+                    if (WHAT == FK_SOLID && !((zero >> k) & 1u)) owner[k] = j + 1;
+                    zero |= 1u << k;
+                }
+                if ((nd >> mx) & 1ull) skip |= 1u << k;
+            }
+        }
+    }
+    if (!valid) return;
+    if (WHAT == FK_SOLID) {
+        *reinterpret_cast<int4*>(P.out_solid + own) = make_int4(owner[0], owner[1], owner[2], owner[3]);
+        return;
+    }
+    skip &= ~zero;
+    if (WHAT == FK_F) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const float f = comp(v[i], k);
+                set_comp(v[i], k, ((zero >> k) & 1u) ? 0.0f : (P.out_dev ? f : f + w_of(i) * rho0));
+            }
+        if (skip == 0u) {
+#pragma unroll
+            for (int i = 0; i < Q; ++i) *reinterpret_cast<float4*>(P.out_f + (i * N + own)) = v[i];
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if ((skip >> k) & 1u) continue;
+#pragma unroll
+                for (int i = 0; i < Q; ++i) P.out_f[i * N + own + k] = comp(v[i], k);
+            }
+        }
+        return;
+    }
+    float4 out[4];                              // rho, u_x, u_y, u_z of the four nodes
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        float f[Q], a[4];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) f[i] = comp(v[i], k);
+        node_moments(f, rho0, s_g, a[0], a[1], a[2], a[3]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) set_comp(out[e], k, ((zero >> k) & 1u) ? 0.0f : a[e]);
+    }
+    float* dst[4] = {P.out_rho, P.out_u, P.out_u ? P.out_u + N : nullptr, P.out_u ? P.out_u + 2 * N : nullptr};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        if (!dst[e]) continue;
+        if (skip == 0u) {
+            *reinterpret_cast<float4*>(dst[e] + own) = out[e];
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (!((skip >> k) & 1u)) dst[e][own + k] = comp(out[e], k);
+        }
     }
 }
 
 // ---------------------------------------------------------------------------
-// Field read-back: pre-collision populations at the start of iteration t
-// (streaming, bounce-back and remap fix-ups of t-1 without a collision), every
-// tile tested against the particles' occupancy maps.
+// blocks: 256-quad tiles of the box; p.surf_blocks more for the nodes next to a surface
 template <class St>
-static cudaError_t launch_mode(const KParams& p, int blocks, cudaStream_t s)
+static cudaError_t launch_mode(KParams p, int blocks, cudaStream_t s)
 {
-    int dev = 0, nsm = 0;
-    cudaError_t e;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const int g = blocks < nsm ? blocks : nsm;          // one block of this many registers per SM
+    if (p.out_solid) p.surf_blocks = 0;
+    const int g = blocks + p.surf_blocks;
     if (p.out_f) fields_kernel<St, FK_F><<<g, KBLOCK, 0, s>>>(p);
-    else if (p.out_solid) fields_kernel<St, FK_SOLID><<<blocks, KBLOCK, 0, s>>>(p);
+    else if (p.out_solid) fields_kernel<St, FK_SOLID><<<g, KBLOCK, 0, s>>>(p);
     else fields_kernel<St, FK_MOMENTS><<<g, KBLOCK, 0, s>>>(p);
     return cudaGetLastError();
 }

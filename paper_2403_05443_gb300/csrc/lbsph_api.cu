@@ -869,6 +869,8 @@ static KParams base_kparams(lb_ctx* ctx)
     k.nbox = (int)ctx->hbox.size();
     k.pk = ctx->d_pk;
     k.status = ctx->d_status;
+    k.need_hdr = ctx->d_need_hdr + (size_t)ctx->cur * ctx->maxp;
+    k.need = ctx->d_need + (size_t)ctx->cur * MAXS * MAXS * ctx->maxp;
     return k;
 }
 
@@ -1082,6 +1084,17 @@ extern "C" lb_status lb_get_fields(lb_ctx* ctx, int32_t box, uint32_t what, void
     k.src = ctx->fbuf[ctx->cur];
     k.only_box = box;
     k.nopull = ctx->collided ? 0 : 1;
+    if (ctx->collided && !ctx->parts[box].empty()) {
+        // blocks for the nodes next to the surfaces, one thread per node of a particle's cube
+        int S = 0;
+        for (const lb_particle& p : ctx->parts[box]) {
+            int hp, Sp;
+            cube_of(p, hp, Sp);
+            S = std::max(S, Sp);
+        }
+        k.surf_per = (S * S * S + KBLOCK - 1) / KBLOCK;
+        k.surf_blocks = k.surf_per * (int)ctx->parts[box].size();
+    }
     k.out_dev = (what == LB_FIELD_DF) ? 1 : 0;
     if (what == LB_FIELD_F || what == LB_FIELD_DF) k.out_f = out;
     if (what == LB_FIELD_RHO) k.out_rho = out;

@@ -248,6 +248,10 @@ struct KParams {
     int* out_solid;                 // [N] or nullptr
     int only_box;                   // box index (the grid covers that box only)
     int nopull;                     // before the first collision: f = w rho0, no streaming
+    // field read-back: the redo masks of the next iteration, and the blocks for their nodes
+    const NeedHdr* need_hdr;        // per particle
+    const uint64_t* need;           // per particle MAXS*MAXS words
+    int surf_blocks, surf_per;      // in all, and per particle of the box (covering S^3 cube nodes)
 };
 
 struct PParams {
