@@ -108,7 +108,8 @@ struct lb_ctx {
     int dpar27 = 0;                    // slot of d_dyn27 ([2][nbox]) the next lattice pass reads
     int nbpp27 = 1;                    // near-pass blocks per particle
     cudaStream_t s27 = nullptr;        // near pass and particle kernel, beside the bulk pass
-    cudaEvent_t ev27a = nullptr, ev27b = nullptr;
+    cudaStream_t s27x = nullptr;       // auxiliary kernel, beside the bulk pass and the next near pass
+    cudaEvent_t ev27a = nullptr, ev27b = nullptr, ev27c = nullptr;
 };
 
 static lb_status fail(lb_ctx* c, lb_status s, const std::string& msg)
@@ -288,6 +289,8 @@ static lb_status q27_create(lb_ctx* ctx, const lb_box_desc* boxes, int nbox)
     CK(cudaStreamCreateWithPriority(&ctx->s27, cudaStreamNonBlocking, prio_hi));
     CK(cudaEventCreateWithFlags(&ctx->ev27a, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ctx->ev27b, cudaEventDisableTiming));
+    CK(cudaStreamCreateWithPriority(&ctx->s27x, cudaStreamNonBlocking, prio_hi));
+    CK(cudaEventCreateWithFlags(&ctx->ev27c, cudaEventDisableTiming));
     CK(cudaStreamSynchronize(ctx->stream));
     return LB_OK;
 }
@@ -370,6 +373,7 @@ static lb_status q27_set_particles(lb_ctx* ctx, int box, const lb_particle* p, i
     q27::PartParams27 pp{ctx->d_part27, ctx->d_dyn27 + (size_t)ctx->dpar27 * nbox, ctx->d_box27, ctx->d_rows,
                          ctx->d_acc, ctx->d_status, 1, ctx->opt.didt_mode};
     CK(q27::launch_particles27(pp, np, s));
+    CK(q27::launch_particles27_aux(pp, np, s));
     CK(cudaStreamSynchronize(s));
     return read_status(ctx);
 }
@@ -385,6 +389,7 @@ static cudaError_t q27_enqueue(lb_ctx* ctx, int nsteps, cudaStream_t s)
 {
     cudaError_t e = cudaSuccess;
     const size_t nbox = ctx->desc.size();
+    bool aux = false;                   // an auxiliary kernel of this call may still run on s27x
     for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
         const q27::Dyn27* dcur = ctx->d_dyn27 + (size_t)ctx->dpar27 * nbox;
         q27::Dyn27* dnext = ctx->d_dyn27 + (size_t)(ctx->dpar27 ^ 1) * nbox;
@@ -401,23 +406,30 @@ static cudaError_t q27_enqueue(lb_ctx* ctx, int nsteps, cudaStream_t s)
         } else if (!ctx->collided) {
             if ((e = q27::launch_lattice27(lp, ctx->blocks27, s)) != cudaSuccess) break;
             if ((e = q27::launch_particles27(pp, ctx->np, s)) != cudaSuccess) break;
+            if ((e = q27::launch_particles27_aux(pp, ctx->np, s)) != cudaSuccess) break;
         } else {
             if ((e = cudaEventRecord(ctx->ev27a, s)) != cudaSuccess) break;
             if ((e = cudaStreamWaitEvent(ctx->s27, ctx->ev27a, 0)) != cudaSuccess) break;
             q27::LatParams27 near = lp;
             near.mode = q27::LAT_NEAR;
             if ((e = q27::launch_lattice27(near, ctx->np * ctx->nbpp27, ctx->s27)) != cudaSuccess) break;
+            if (aux && (e = cudaStreamWaitEvent(ctx->s27, ctx->ev27c, 0)) != cudaSuccess) break;
             if ((e = q27::launch_particles27(pp, ctx->np, ctx->s27)) != cudaSuccess) break;
             q27::LatParams27 bulk = lp;
             bulk.mode = q27::LAT_BULK;
             if ((e = q27::launch_bulk27(bulk, ctx->blocks27, s)) != cudaSuccess) break;
             if ((e = cudaEventRecord(ctx->ev27b, ctx->s27)) != cudaSuccess) break;
             if ((e = cudaStreamWaitEvent(s, ctx->ev27b, 0)) != cudaSuccess) break;
+            if ((e = cudaStreamWaitEvent(ctx->s27x, ctx->ev27b, 0)) != cudaSuccess) break;
+            if ((e = q27::launch_particles27_aux(pp, ctx->np, ctx->s27x)) != cudaSuccess) break;
+            if ((e = cudaEventRecord(ctx->ev27c, ctx->s27x)) != cudaSuccess) break;
+            aux = true;
         }
         ctx->cur ^= 1;
         ctx->dpar27 ^= 1;
         ctx->collided = true;
     }
+    if (aux && e == cudaSuccess) e = cudaStreamWaitEvent(s, ctx->ev27c, 0);
     return e;
 }
 
@@ -499,8 +511,10 @@ extern "C" lb_status lb_create(const lb_box_desc* boxes, int32_t nbox, const lb_
             cudaStreamSynchronize(ctx->stream);
             free_all(ctx);
             if (ctx->s27) cudaStreamDestroy(ctx->s27);
+            if (ctx->s27x) cudaStreamDestroy(ctx->s27x);
             if (ctx->ev27a) cudaEventDestroy(ctx->ev27a);
             if (ctx->ev27b) cudaEventDestroy(ctx->ev27b);
+            if (ctx->ev27c) cudaEventDestroy(ctx->ev27c);
             cudaStreamDestroy(ctx->stream);
             cudaEventDestroy(ctx->ev_done);
             delete ctx;
@@ -634,8 +648,10 @@ extern "C" lb_status lb_destroy(lb_ctx* ctx)
     cudaDeviceSynchronize();
     free_all(ctx);
     if (ctx->s27) cudaStreamDestroy(ctx->s27);
+    if (ctx->s27x) cudaStreamDestroy(ctx->s27x);
     if (ctx->ev27a) cudaEventDestroy(ctx->ev27a);
     if (ctx->ev27b) cudaEventDestroy(ctx->ev27b);
+    if (ctx->ev27c) cudaEventDestroy(ctx->ev27c);
     cudaStreamDestroy(ctx->stream);
     cudaEventDestroy(ctx->ev_done);
     delete ctx;

@@ -496,20 +496,11 @@ __device__ __forceinline__ void cross27(const double a[3], const double b[3], do
     o[2] = a[0] * b[1] - a[1] * b[0];
 }
 
-// The parts of the solve of Eq. Fdiscrete / Eq. Tdiscrete for particle D,
-// spread over the block: q27_sums (one thread) turns the integer sums of the
-// last lattice pass into F0, T0 and the remap terms; the inertia and its rate
-// come from another warp at the same time; a warp solves the 6 x 6 system
-// (q27_solve6); six threads form F and T; three threads move the centre and
-// another the orientation, and a warp writes the record.
-__device__ void q27_sums(const PartParams27& P, Part27* D, const Box27& B, int p, double F0[3], double T0[3])
+// The integer sums of the last lattice pass (acc) into F0, T0 and the remap terms.  One thread.
+__device__ void q27_sums(const long long* acc, Part27* D, const Box27& B, double F0[3], double T0[3])
 {
-    long long* acc = P.acc + (size_t)p * NACC;
     double a[NACC];
-    for (int e = 0; e < NACC; ++e) {
-        a[e] = (double)acc[e];
-        acc[e] = 0;
-    }
+    for (int e = 0; e < NACC; ++e) a[e] = (double)acc[e];
     const double rho0 = B.rho0;
     double Fd[3], Tm[3], J[3], MJ[3], Sm[3], phi[3];
     for (int k = 0; k < 3; ++k) {
@@ -597,13 +588,11 @@ __device__ __forceinline__ bool gj_inv6_warp_f32(float (&col)[6], int lane)
 // with the residual in FP64.  Each step multiplies the error by about cond(A)
 // times the FP32 rounding; three steps bring it to FP64 rounding for these
 // systems (mass, inertia and drag matrices: cond(A) of order 10-10^3).  Only
-// the residuals are FP64, so the chain of dependent FP64 operations is short;
-// measured beside the bulk pass the solve still takes about as long as a
-// Gauss-Jordan elimination in FP64 (about 15 us; with the pivot loop rolled up,
-// a fifth of the code, 17.5 us), so its time is the latency of its dependent
-// chain, not arithmetic or instruction fetch.  s_Ai: 36 floats of scratch.
-// Writes x6 (lanes 0..5); false if a pivot vanishes.
-__device__ bool q27_solve6(const double* A6, const double* rhs, double* x6, float* s_Ai, int lane)
+// the residuals are FP64.  The inverse (a dependent chain of about 10 us beside
+// the bulk pass) needs no force, so the auxiliary kernel forms it while the
+// lattice passes run, and the critical kernel only refines.
+// Ai: the 36 floats of the inverse; false if a pivot vanishes.
+__device__ bool q27_inverse6(const double* A6, float* Ai, int lane)
 {
     float col[6];
 #pragma unroll
@@ -612,15 +601,21 @@ __device__ bool q27_solve6(const double* A6, const double* rhs, double* x6, floa
     const bool ok = gj_inv6_warp_f32(col, lane);
     if (lane >= 6 && lane < 12)
 #pragma unroll
-        for (int i = 0; i < 6; ++i) s_Ai[i * 6 + lane - 6] = col[i];
+        for (int i = 0; i < 6; ++i) Ai[i * 6 + lane - 6] = col[i];
     __syncwarp();
+    return ok;
+}
+
+// writes x6 (lanes 0..5)
+__device__ void q27_refine6(const double* A6, const float* Ai, const double* rhs, double* x6, int lane)
+{
     const int i = lane < 6 ? lane : 0;
     double a[6];
     float ai[6];
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
         a[j] = A6[i * 6 + j];
-        ai[j] = s_Ai[i * 6 + j];
+        ai[j] = Ai[i * 6 + j];
     }
     const double b = rhs[i];
     float xf = 0.0f;
@@ -642,41 +637,40 @@ __device__ bool q27_solve6(const double* A6, const double* rhs, double* x6, floa
     }
     if (lane < 6) x6[lane] = x;
     __syncwarp();
-    return ok;
 }
 
 // ---------------------------------------------------------------------------
-// Particle kernel: one block of 512 threads per particle, the particle's state
-// staged in shared memory and written back at the end.  Step mode: the solve
-// and pose update of the last lattice pass's iteration, then for the new pose
-// the occupancy map (Eq. ellipsoidsurface), built in shared memory one cube row
-// per thread: along a row the inside value is the quadratic a x^2 + b x + c,
-// evaluated in FP32 and decided there outside a band around 1 (its FP32 error
-// stays far below the band inside the cube); the nodes inside the band are
-// collected and then tested by the exact FP64 test in the oracle's operation
-// order, one node per thread, so the map is bit-identical to the oracle's.
-// The links (x fluid, x + c_b solid) of each row and direction are a bit mask;
-// their drag matrix and the geometric parts of F0 / T0 (Eq. drag1-4, Eq. F0,
-// Eq. T0) come from exact integer sums per direction (link count, sum of m,
-// sum of m m^T over the cube coordinates m of the fluid ends), combined once
-// in FP64 with p = phi + m, r_b x c_b = p x c_b.  Init mode: the map and its
-// terms for the current pose.
+// Critical particle kernel: one block of 512 threads per particle, the
+// particle's state staged in shared memory and written back at the end.  It is
+// what the next near pass waits for, so it holds no more than that pass needs:
+// the solve and pose update of the last lattice pass's iteration (one warp, with
+// the matrix and its FP32 inverse from the auxiliary kernel), then for the new
+// pose the occupancy map (Eq. ellipsoidsurface) and the box's uniform terms.  The
+// map is built in shared memory one cube row per thread: along a row the inside
+// value is the quadratic a x^2 + b x + c, and where its FP32 rounding is far below
+// a only the nodes within 1.5 of its roots are evaluated (the others are decided
+// by more than that rounding).  An evaluated node is decided in FP32 outside a
+// band around 1; the nodes inside the band are collected and then tested by the
+// exact FP64 test in the oracle's operation order, one node per thread, so the
+// map is bit-identical to the oracle's.  Init mode: the map of the current pose.
+// Measured, a step with its share of the read-back, before (the link sums, the drag
+// matrix and the solve's elimination in this kernel, 54 us of the chain near pass ->
+// particle kernel -> near pass) and after: one 64^3 box 59.7 -> 50.1 us, four 87.5 ->
+// 69.4, one of 128^3 nodes 103 -> 92; eight 64^3 boxes 105.9 -> 105.3, where the bulk
+// pass beside the near pass sets the pace.
 constexpr int NCAND = 512;                       // nodes of the FP32 band tested exactly after the row pass
 __global__ void __launch_bounds__(PBLK, 1) particle27_kernel(const __grid_constant__ PartParams27 P)
 {
-    constexpr int NSUM = 10;                     // per direction: n, sum m (3), sum m m^T (6)
-    constexpr int NG = PBLK / (Q27 - 1);         // row groups of the link sums (one direction per thread)
     const int p = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     Part27* G = P.pd + p;
     __shared__ Part27 sD;
     __shared__ Box27 sB;
     __shared__ uint64_t s_map[MAXS * MAXS];
-    __shared__ int s_sum[Q27][NSUM];
-    __shared__ double s_con[Q27][42];            // per direction: drag matrix (36), F0g (3), T0g (3)
+    __shared__ long long s_acc[NACC];
     __shared__ double s_A[9], s_E[9], s_x[3], s_phi[3];
+    __shared__ double s_F0[3], s_T0[3], s_rhs[6], s_x6[6];
     __shared__ float s_A32[9], s_d0[3];
-    __shared__ int s_o[3], s_ow[3], s_S, s_slot, s_ok, s_nsol, s_ncand;
-    __shared__ float s_band;
+    __shared__ int s_o[3], s_ow[3], s_ok, s_nsol, s_ncand;
     __shared__ int s_cand[NCAND];
     static_assert(sizeof(Part27) % 8 == 0 && sizeof(Box27) % 4 == 0, "staged as words");
     {
@@ -685,145 +679,116 @@ __global__ void __launch_bounds__(PBLK, 1) particle27_kernel(const __grid_consta
             reinterpret_cast<unsigned long long*>(&sD)[k] = reinterpret_cast<const unsigned long long*>(G)[k];
         if (tid >= 256 && tid < 256 + (int)(sizeof(Box27) / 4))
             reinterpret_cast<int*>(&sB)[tid - 256] = __ldg(reinterpret_cast<const int*>(P.boxes + bi) + (tid - 256));
+        else if (!P.init && tid >= 384 && tid < 384 + NACC) {
+            long long* acc = P.acc + (size_t)p * NACC + (tid - 384);
+            s_acc[tid - 384] = *acc;
+            *acc = 0;
+        }
+        if (tid == 0) s_nsol = s_ncand = 0;
     }
     __syncthreads();
     Part27* D = &sD;
     const Box27& B = sB;
-    if (!P.init) {
-        __shared__ double s_F0[3], s_T0[3], s_In[9], s_dI[9], s_A6[36], s_rhs[6], s_x6[6], s_FT[6], s_xn[3], s_qn[4];
-        __shared__ float s_Ai[36];
-        __shared__ int s_solved;
-        if (tid == 0) {
-            q27_sums(P, D, B, p, s_F0, s_T0);
-        } else if (tid == 32) {
-            inertia27(D->q, D->Ib, s_In);
-            if (P.didt_mode == 1) {
-                for (int k = 0; k < 9; ++k) s_dI[k] = s_In[k] - D->Iprev[k];
-            } else {
-                inertia_rate27(s_In, D->W, s_dI);
-            }
-        }
-        __syncthreads();
-        if (tid < 36) {
-            // A = zeta + diag(M) + (I + dI) in the rotational block
-            const int i = tid / 6, j = tid % 6;
-            double a = D->zeta[tid];
-            if (i == j && i < 3) a += D->M;
-            if (i >= 3 && j >= 3) a += s_In[(i - 3) * 3 + j - 3] + s_dI[(i - 3) * 3 + j - 3];
-            s_A6[tid] = a;
-        } else if (tid >= 64 && tid < 70) {
-            // rhs = (M U + F0 + F_ext + dP, I W + T0 + T_ext + dL)
-            const int k = tid - 64;
-            if (k < 3) {
-                s_rhs[k] = D->M * D->U[k] + s_F0[k] + D->Fext[k] + D->dP[k];
-            } else {
-                const int m = k - 3;
-                s_rhs[k] = s_In[m * 3] * D->W[0] + s_In[m * 3 + 1] * D->W[1] + s_In[m * 3 + 2] * D->W[2] + s_T0[m] +
-                           D->Text[m] + D->dL[m];
-            }
-        }
-        __syncthreads();
-        if (tid < 32) {
-            const bool ok = q27_solve6(s_A6, s_rhs, s_x6, s_Ai, tid);
-            if (tid == 0) s_solved = ok;
-        }
-        __syncthreads();
-        if (P.didt_mode == 2 && s_solved) {
-            // corrector: I(t+1) of the orientation the first solution predicts
-            if (tid == 0) {
-                double Wm[3], qp[4], Ip[9];
-                for (int k = 0; k < 3; ++k) Wm[k] = 0.5 * (D->W[k] + s_x6[k + 3]);
-                qstep27(D->q, Wm, qp);
-                inertia27(qp, D->Ib, Ip);
-                for (int i = 0; i < 3; ++i)
-                    for (int j = 0; j < 3; ++j) s_A6[(i + 3) * 6 + j + 3] = D->zeta[(i + 3) * 6 + j + 3] + Ip[i * 3 + j];
-            }
-            __syncthreads();
-            if (tid < 32) {
-                const bool ok = q27_solve6(s_A6, s_rhs, s_x6, s_Ai, tid);
-                if (tid == 0) s_solved = ok;
-            }
-            __syncthreads();
-        }
-        // F = F0 - zeta_F (U', W'), T = T0 - zeta_T (U', W'), one component per
-        // thread; the new centre (Eq. posupdate) on three threads and the new
-        // orientation (Eq. qnplus0-1, mean angular velocity of the step) on another
-        if (tid < 6) {
-            double z = 0.0;
-            for (int j = 0; j < 6; ++j) z += D->zeta[tid * 6 + j] * s_x6[j];
-            s_FT[tid] = (tid < 3 ? s_F0[tid] : s_T0[tid - 3]) - z;
-        } else if (tid >= 32 && tid < 35) {
-            const int k = tid - 32;
-            s_xn[k] = D->x[k] + 0.5 * (D->U[k] + s_x6[k]);
-        } else if (tid == 64) {
-            double Wm[3];
-            for (int k = 0; k < 3; ++k) Wm[k] = 0.5 * (D->W[k] + s_x6[k + 3]);
-            qstep27(D->q, Wm, s_qn);
-        }
-        __syncthreads();
-        if (s_solved) {
-            // the new state, and the record F0, T0, F, T, U, W, x, q (finite or ST_NAN)
-            if (tid < 9) {
-                D->Iprev[tid] = s_In[tid];
-                if (tid < 3) {
-                    D->x[tid] = s_xn[tid];
-                    D->U[tid] = s_x6[tid];
-                    D->W[tid] = s_x6[tid + 3];
+    if (warp == 0) {
+        bool solved = true;
+        if (!P.init) {
+            if (lane == 0) q27_sums(s_acc, D, B, s_F0, s_T0);
+            __syncwarp();
+            if (lane < 6) {
+                // rhs = (M U + F0 + F_ext + dP, I W + T0 + T_ext + dL)
+                const int k = lane;
+                if (k < 3) {
+                    s_rhs[k] = D->M * D->U[k] + s_F0[k] + D->Fext[k] + D->dP[k];
+                } else {
+                    const int m = k - 3;
+                    s_rhs[k] = D->In[m * 3] * D->W[0] + D->In[m * 3 + 1] * D->W[1] + D->In[m * 3 + 2] * D->W[2] + s_T0[m] +
+                               D->Text[m] + D->dL[m];
                 }
-                if (tid < 4) D->q[tid] = s_qn[tid];
-            } else if (warp == 1) {
-                double v = 0.0;
-                if (lane < 3) v = s_F0[lane];
-                else if (lane < 6) v = s_T0[lane - 3];
-                else if (lane < 12) v = s_FT[lane - 6];
-                else if (lane < 18) v = s_x6[lane - 12];
-                else if (lane < 21) v = s_xn[lane - 18];
-                else if (lane < 25) v = s_qn[lane - 21];
-                if (lane < 25) D->rec[lane] = v;
-                if (!__all_sync(0xffffffffu, lane >= 25 || isfinite(v)) && lane == 0) atomicOr(P.status, ST_NAN);
             }
-        } else if (tid == 0) {
-            atomicOr(P.status, ST_NAN);
-        }
-        __syncthreads();
-    }
-    // the cube of the new pose (origin floor(x) - h, side S = 2h + 2), one axis
-    // per thread; the exact inside-test matrix of the new orientation on another
-    // warp (lanes 0..8)
-    if (tid < 3) {
-        const int k = tid;
-        const int L = k == 0 ? B.nx : (k == 1 ? B.ny : B.nz);
-        const int o = (int)floor(D->x[k]) - D->h;
-        s_o[k] = o;
-        s_ow[k] = ((o % L) + L) % L;
-        s_phi[k] = (double)o - D->x[k];
-        s_d0[k] = (float)s_phi[k];                 // d = X - x_c at cube coordinate 0
-        s_x[k] = D->x[k];
-        if (k == 0) {
-            s_ok = 1;
-            if (!P.init) {
-                if (__ldcg(P.status) & ST_NAN) s_ok = 0;
+            __syncwarp();
+            solved = D->inv_ok != 0;
+            q27_refine6(D->A6, D->Ai, s_rhs, s_x6, lane);
+            if (P.didt_mode == 2 && solved) {
+                // corrector: I(t+1) of the orientation the first solution predicts
+                if (lane == 0) {
+                    double Wm[3], qp[4], Ip[9];
+                    for (int k = 0; k < 3; ++k) Wm[k] = 0.5 * (D->W[k] + s_x6[k + 3]);
+                    qstep27(D->q, Wm, qp);
+                    inertia27(qp, D->Ib, Ip);
+                    for (int i = 0; i < 3; ++i)
+                        for (int j = 0; j < 3; ++j) D->A6[(i + 3) * 6 + j + 3] = D->zeta[(i + 3) * 6 + j + 3] + Ip[i * 3 + j];
+                }
+                __syncwarp();
+                solved = q27_inverse6(D->A6, D->Ai, lane);
+                q27_refine6(D->A6, D->Ai, s_rhs, s_x6, lane);
             }
-            s_S = D->S;
-            s_slot = P.init ? 0 : 1 - D->slot;
-            s_nsol = 0;
-            s_ncand = 0;
-            s_band = D->band;                      // the FP32 decision band of the map (set on the host)
+            if (solved) {
+                // the new centre (Eq. posupdate) and orientation (Eq. qnplus0-1, mean angular velocity of the step)
+                double Wm[3], qn[4];
+                for (int k = 0; k < 3; ++k) Wm[k] = 0.5 * (D->W[k] + s_x6[k + 3]);
+                qstep27(D->q, Wm, qn);
+                const int k = lane % 3;
+                const double xn = D->x[k] + 0.5 * (D->U[k] + s_x6[k]);
+                __syncwarp();
+                if (lane < 3) {
+                    D->x[lane] = xn;
+                    D->U[lane] = s_x6[lane];
+                    D->W[lane] = s_x6[lane + 3];
+                }
+                if (lane < 4) D->q[lane] = lane == 0 ? qn[0] : (lane == 1 ? qn[1] : (lane == 2 ? qn[2] : qn[3]));
+                if (lane < 9) D->Iprev[lane] = D->In[lane];
+            }
+            __syncwarp();
+        } else if (lane == 0) {
+            inertia27(D->q, D->Ib, D->Iprev);      // I(t - 1) = I(t) before the first step
         }
-    } else if (warp == 1) {
+        // the cube of the new pose (origin floor(x) - h, side S = 2h + 2), one axis
+        // per lane, and the exact inside-test matrix of the new orientation (lanes 0..8)
+        if (lane < 3) {
+            const int k = lane;
+            const int L = k == 0 ? B.nx : (k == 1 ? B.ny : B.nz);
+            const int o = (int)floor(D->x[k]) - D->h;
+            s_o[k] = o;
+            s_ow[k] = ((o % L) + L) % L;
+            s_phi[k] = (double)o - D->x[k];
+            s_d0[k] = (float)s_phi[k];             // d = X - x_c at cube coordinate 0
+            s_x[k] = D->x[k];
+        }
+        __syncwarp();
         canon_shape_warp(D->inv2, D->q, s_E, s_A, lane);
+        __syncwarp();
         if (lane < 9) s_A32[lane] = (float)s_A[lane];
-    } else if (P.init && tid == 64) {
-        inertia27(D->q, D->Ib, D->Iprev);          // I(t - 1) = I(t) before the first step
+        if (lane == 0) {
+            if (!solved) atomicOr(P.status, ST_NAN);
+            s_ok = P.init || (solved && !(__ldcg(P.status) & ST_NAN));
+        }
     }
-    for (int k = tid; k < Q27 * NSUM; k += PBLK) (&s_sum[0][0])[k] = 0;
     __syncthreads();
+    if (!P.init && warp == PBLK / 32 - 1 && D->inv_ok) {
+        // the record F0, T0, F = F0 - zeta_F (U', W'), T likewise, U, W, x, q (finite or ST_NAN), on a warp with few rows
+        double v = 0.0;
+        if (lane < 12) {
+            const int k = lane < 6 ? lane : lane - 6;
+            v = k < 3 ? s_F0[k] : s_T0[k - 3];
+            if (lane >= 6) {
+                double z = 0.0;
+                for (int j = 0; j < 6; ++j) z += D->zeta[k * 6 + j] * s_x6[j];
+                v -= z;
+            }
+        } else if (lane < 18) v = s_x6[lane - 12];
+        else if (lane < 21) v = D->x[lane - 18];
+        else if (lane < 25) v = D->q[lane - 21];
+        if (lane < 25) D->rec[lane] = v;
+        if (!__all_sync(0xffffffffu, lane >= 25 || isfinite(v)) && lane == 0) atomicOr(P.status, ST_NAN);
+    }
     if (!s_ok) {
+        __syncthreads();
         for (int k = tid; k < (int)(sizeof(Part27) / 8); k += PBLK)
             reinterpret_cast<unsigned long long*>(G)[k] = reinterpret_cast<const unsigned long long*>(&sD)[k];
         return;
     }
-    const int S = s_S;
+    const int S = D->S;
+    const int slot = P.init ? 0 : 1 - D->slot;
     const uint64_t full = S == 64 ? ~0ull : ((1ull << S) - 1ull);
     // ---- occupancy of the new pose: FP32 outside the band, band nodes listed
     for (int r = tid; r < S * S; r += PBLK) {
@@ -831,9 +796,34 @@ __global__ void __launch_bounds__(PBLK, 1) particle27_kernel(const __grid_consta
         const float dy = s_d0[1] + (float)my, dz = s_d0[2] + (float)mz;
         const float qa = s_A32[0], qb = 2.0f * (s_A32[1] * dy + s_A32[2] * dz);
         const float qc = s_A32[4] * dy * dy + 2.0f * s_A32[5] * dy * dz + s_A32[8] * dz * dz;
-        const float band = s_band;
-        uint64_t w = 0;
-        for (int mx = 0; mx < S; ++mx) {
+        const float band = D->band;
+        // nodes to evaluate: all, or where the rounding of v and of its minimum (a few 1e-7 of the terms that cancel)
+        // is below a tenth of a, the nodes within 1.5 of a root (there |v - 1| >= 2 a and more beyond); none if the
+        // minimum lies above the band
+        uint64_t w = 0, todo = full;
+        const float terms = fabsf(qc) + qb * qb / (4.0f * qa);
+        const float vmin = qc - qb * qb / (4.0f * qa);
+        if (5e-6f * terms < fminf(qa, 0.1f)) {
+            if (vmin > 1.0f + 2.0f * band + 5e-6f * terms) {
+                todo = 0;
+            } else {
+                const float xv = -qb / (2.0f * qa) - s_d0[0];
+                const float hw = sqrtf(fmaxf(1.0f - vmin, 0.0f) / qa);
+                // the band's width in x: within it of a root |v - 1| may stay below the band
+                const float wd = 1.5f + sqrtf((band + 5e-6f * terms) / qa);
+                auto range = [&](float lo, float hi) -> uint64_t {       // nodes lo <= m <= hi of the row
+                    const int m0 = max(0, (int)ceilf(fmaxf(lo, -2.0f))), m1 = min(S - 1, (int)floorf(fminf(hi, 100.0f)));
+                    if (m1 < m0) return 0ull;
+                    return ((m1 >= 63 ? ~0ull : ((1ull << (m1 + 1)) - 1ull)) & ~((1ull << m0) - 1ull)) & full;
+                };
+                const uint64_t inner = hw > wd ? range(xv - hw + wd, xv + hw - wd) : 0ull;
+                todo = range(xv - hw - wd, xv + hw + wd) & ~inner;
+                w = inner;
+            }
+        }
+        while (todo) {
+            const int mx = __ffsll((long long)todo) - 1;
+            todo &= todo - 1;
             const float dx = s_d0[0] + (float)mx;
             const float v = (qa * dx + qb) * dx + qc;
             if (fabsf(v - 1.0f) > band) {
@@ -863,13 +853,9 @@ __global__ void __launch_bounds__(PBLK, 1) particle27_kernel(const __grid_consta
         }
     }
     __syncthreads();
-    // ---- solid nodes; the map into its global slot (the lattice kernel and the
-    // read-back use it); links of the new map summed per direction in integers:
-    // thread t takes direction 1 + t % 26 over the rows g, g + NG, ... (g = t / 26);
-    // the sums of x and x^2 over a row's link bits come from popcounts of the
-    // masks of bit positions whose bit p is set (x = sum_p 2^p [bit p of x])
+    // ---- solid nodes; the map into its global slot (the lattice kernels, the auxiliary kernel and the read-back use it)
     {
-        uint64_t* map = P.rows + ((size_t)p * 2 + s_slot) * RW;
+        uint64_t* map = P.rows + ((size_t)p * 2 + slot) * RW;
         int ns = 0;
         for (int r = tid; r < S * S; r += PBLK) {
             const uint64_t w = s_map[r];
@@ -879,6 +865,94 @@ __global__ void __launch_bounds__(PBLK, 1) particle27_kernel(const __grid_consta
         ns = __reduce_add_sync(0xffffffffu, ns);
         if (lane == 0 && ns) atomicAdd(&s_nsol, ns);
     }
+    __syncthreads();
+    // the new state, one thread per axis (thread 0 also the scalars)
+    if (tid < 3) {
+        const int i = tid;
+        const int ns = s_nsol;
+        Dyn27& Y = P.dyn[D->box];
+        // the map the next pass bounces back from is the current one
+        const int Lk = i == 0 ? B.nx : (i == 1 ? B.ny : B.nz);
+        Y.phi_old[i] = P.init ? (float)s_phi[i] : (float)D->phi[i];
+        Y.o_old[i] = P.init ? s_ow[i] : ((D->o[i] % Lk) + Lk) % Lk;
+        // the box that holds both cubes (the near pass covers its nodes)
+        const int lo = P.init ? s_o[i] : min(D->o[i], s_o[i]);
+        const int hi = (P.init ? s_o[i] : max(D->o[i], s_o[i])) + S;
+        Y.E[i] = min(hi - lo, Lk);
+        Y.uo[i] = ((lo % Lk) + Lk) % Lk;
+        if (!P.init && abs(s_o[i] - D->o[i]) > 1) atomicOr(P.status, ST_CAPACITY);
+        Y.phi_new[i] = (float)s_phi[i];
+        Y.o_new[i] = s_ow[i];
+        Y.U[i] = (float)D->U[i];
+        Y.W[i] = (float)D->W[i];
+        // uniform terms of the next collision: body force (with the counter
+        // force on the fluid nodes of the new map) and the mass of this remap,
+        // returned over every fluid node
+        const double inf = 1.0 / (double)(B.N - ns);
+        Y.g[i] = (float)(B.body[i] - (B.counter ? D->Fext[i] * inf : 0.0));
+        if (i == 0) {
+            Y.slot_old = P.init ? slot : D->slot;
+            Y.slot_new = slot;
+            Y.S = S;
+            Y.active = 1;
+            Y.eps = P.init ? 0.0f : (float)(D->dm * inf);
+        }
+    }
+    __syncthreads();
+    if (tid < 3) {
+        D->phi[tid] = s_phi[tid];
+        D->o[tid] = s_o[tid];
+        if (tid == 0) {
+            D->slot = slot;
+            D->nsolid = s_nsol;
+        }
+    }
+    __syncthreads();
+    for (int k = tid; k < (int)(sizeof(Part27) / 8); k += PBLK)
+        reinterpret_cast<unsigned long long*>(G)[k] = reinterpret_cast<const unsigned long long*>(&sD)[k];
+}
+
+// Auxiliary particle kernel: one block of 512 threads per particle, beside the
+// bulk pass of its step and the near pass of the next one.  What the solve of the
+// next iteration needs besides the forces: the links (x fluid, x + c_b solid) of the
+// current map, of each row and direction a bit mask; their drag matrix and the
+// geometric parts of F0 / T0 (Eq. drag1-4, Eq. F0, Eq. T0) from exact integer sums
+// per direction (link count, sum of m, sum of m m^T over the cube coordinates m of
+// the fluid ends), combined once in FP64 with p = phi + m, r_b x c_b = p x c_b; the
+// inertia and its rate, the matrix of Eq. Fdiscrete / Eq. Tdiscrete and its FP32
+// inverse.  Only the critical kernel of the next step waits for it.
+__global__ void __launch_bounds__(PBLK, 1) particle27_aux_kernel(const __grid_constant__ PartParams27 P)
+{
+    constexpr int NSUM = 10;                     // per direction: n, sum m (3), sum m m^T (6)
+    constexpr int NG = PBLK / (Q27 - 1);         // row groups of the link sums (one direction per thread)
+    const int p = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    Part27* G = P.pd + p;
+    __shared__ Part27 sD;
+    __shared__ Box27 sB;
+    __shared__ uint64_t s_map[MAXS * MAXS];
+    __shared__ int s_sum[Q27][NSUM];
+    __shared__ double s_con[Q27][42];            // per direction: drag matrix (36), F0g (3), T0g (3)
+    __shared__ double s_dI[9];
+    const int S = __ldg(&G->S);
+    {
+        const int bi = __ldg(&G->box);
+        const uint64_t* map = P.rows + ((size_t)p * 2 + G->slot) * RW;
+        for (int r = tid; r < S * S; r += PBLK) s_map[r] = map[r];
+        for (int k = tid; k < (int)(sizeof(Part27) / 8); k += PBLK)
+            reinterpret_cast<unsigned long long*>(&sD)[k] = reinterpret_cast<const unsigned long long*>(G)[k];
+        if (tid >= 256 && tid < 256 + (int)(sizeof(Box27) / 4))
+            reinterpret_cast<int*>(&sB)[tid - 256] = __ldg(reinterpret_cast<const int*>(P.boxes + bi) + (tid - 256));
+        for (int k = tid; k < Q27 * NSUM; k += PBLK) (&s_sum[0][0])[k] = 0;
+    }
+    __syncthreads();
+    Part27* D = &sD;
+    const Box27& B = sB;
+    const double* s_phi = D->phi;
+    const uint64_t full = S == 64 ? ~0ull : ((1ull << S) - 1ull);
+    // ---- links of the map summed per direction in integers: thread t takes
+    // direction 1 + t % 26 over the rows g, g + NG, ... (g = t / 26); the sums of x
+    // and x^2 over a row's link bits come from popcounts of the masks of bit
+    // positions whose bit p is set (x = sum_p 2^p [bit p of x])
     {
         const int b = 1 + tid % (Q27 - 1), g = tid / (Q27 - 1);
         if (g < NG) {
@@ -992,50 +1066,39 @@ __global__ void __launch_bounds__(PBLK, 1) particle27_kernel(const __grid_consta
         }
     }
     __syncthreads();
-    // the new state, one thread per axis (thread 0 also the scalars)
-    if (tid < 3) {
-        const int i = tid;
-        const int ns = s_nsol;
-        Dyn27& Y = P.dyn[D->box];
-        // the map the next pass bounces back from is the current one
-        const int Lk = i == 0 ? B.nx : (i == 1 ? B.ny : B.nz);
-        Y.phi_old[i] = P.init ? (float)s_phi[i] : (float)D->phi[i];
-        Y.o_old[i] = P.init ? s_ow[i] : ((D->o[i] % Lk) + Lk) % Lk;
-        // the box that holds both cubes (the near pass covers its nodes)
-        const int lo = P.init ? s_o[i] : min(D->o[i], s_o[i]);
-        const int hi = (P.init ? s_o[i] : max(D->o[i], s_o[i])) + S;
-        Y.E[i] = min(hi - lo, Lk);
-        Y.uo[i] = ((lo % Lk) + Lk) % Lk;
-        if (!P.init && abs(s_o[i] - D->o[i]) > 1) atomicOr(P.status, ST_CAPACITY);
-        Y.phi_new[i] = (float)s_phi[i];
-        Y.o_new[i] = s_ow[i];
-        Y.U[i] = (float)D->U[i];
-        Y.W[i] = (float)D->W[i];
-        // uniform terms of the next collision: body force (with the counter
-        // force on the fluid nodes of the new map) and the mass of this remap,
-        // returned over every fluid node
-        const double inf = 1.0 / (double)(B.N - ns);
-        Y.g[i] = (float)(B.body[i] - (B.counter ? D->Fext[i] * inf : 0.0));
-        if (i == 0) {
-            Y.slot_old = P.init ? s_slot : D->slot;
-            Y.slot_new = s_slot;
-            Y.S = S;
-            Y.active = 1;
-            Y.eps = P.init ? 0.0f : (float)(D->dm * inf);
+    // the next solve: inertia and its rate, the matrix and its inverse
+    if (warp == 0) {
+        if (lane == 0) {
+            inertia27(D->q, D->Ib, D->In);
+            if (P.didt_mode == 1) {
+                for (int k = 0; k < 9; ++k) s_dI[k] = D->In[k] - D->Iprev[k];
+            } else {
+                inertia_rate27(D->In, D->W, s_dI);
+            }
+        }
+        __syncwarp();
+        for (int e = lane; e < 36; e += 32) {
+            // A = zeta + diag(M) + (I + dI) in the rotational block
+            const int i = e / 6, j = e % 6;
+            double a = D->zeta[e];
+            if (i == j && i < 3) a += D->M;
+            if (i >= 3 && j >= 3) a += D->In[(i - 3) * 3 + j - 3] + s_dI[(i - 3) * 3 + j - 3];
+            D->A6[e] = a;
+        }
+        __syncwarp();
+        const bool ok = q27_inverse6(D->A6, D->Ai, lane);
+        if (lane == 0) G->inv_ok = ok;
+        for (int e = lane; e < 36; e += 32) {
+            G->zeta[e] = D->zeta[e];
+            G->A6[e] = D->A6[e];
+            G->Ai[e] = D->Ai[e];
+        }
+        if (lane < 9) G->In[lane] = D->In[lane];
+        if (lane < 3) {
+            G->F0g[lane] = D->F0g[lane];
+            G->T0g[lane] = D->T0g[lane];
         }
     }
-    __syncthreads();
-    if (tid < 3) {
-        D->phi[tid] = s_phi[tid];
-        D->o[tid] = s_o[tid];
-        if (tid == 0) {
-            D->slot = s_slot;
-            D->nsolid = s_nsol;
-        }
-    }
-    __syncthreads();
-    for (int k = tid; k < (int)(sizeof(Part27) / 8); k += PBLK)
-        reinterpret_cast<unsigned long long*>(G)[k] = reinterpret_cast<const unsigned long long*>(&sD)[k];
 }
 
 // ---------------------------------------------------------------------------
@@ -1146,6 +1209,13 @@ cudaError_t launch_particles27(const PartParams27& p, int np, cudaStream_t s)
 {
     if (np <= 0) return cudaSuccess;
     particle27_kernel<<<np, PBLK, 0, s>>>(p);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_particles27_aux(const PartParams27& p, int np, cudaStream_t s)
+{
+    if (np <= 0) return cudaSuccess;
+    particle27_aux_kernel<<<np, PBLK, 0, s>>>(p);
     return cudaGetLastError();
 }
 

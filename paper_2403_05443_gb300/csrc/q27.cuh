@@ -12,14 +12,17 @@
 //   particle  one block per particle: F0, T0 and the remap terms, the
 //             implicit solve (Eq. Fdiscrete, Tdiscrete), the pose update
 //             (Eq. posupdate, qnplus0-1), the new occupancy map (Eq.
-//             ellipsoidsurface, exact FP64 test near the surface) and the drag
-//             matrix of its links (Eq. drag1-4), and the box's uniform terms of
-//             the next collision.
+//             ellipsoidsurface, exact FP64 test near the surface) and the box's
+//             uniform terms of the next collision;
+//   auxiliary one block per particle: the drag matrix of the new map's links
+//             (Eq. drag1-4), the inertia, and the matrix of the next solve
+//             with its inverse.
 // The iteration is the oracle's Appendix order turned by half a step: a
 // lattice pass does the streaming, bounce-back and remap of iteration t-1 and
 // the collision of iteration t, so the particle solve sits between two lattice
 // passes and every population is read and written once per step.  The near
-// pass and the particle kernel run on their own stream beside the bulk pass.
+// pass and the particle kernel run on their own stream beside the bulk pass, the
+// auxiliary kernel on another, beside the bulk pass and the next near pass.
 #pragma once
 
 #include <cstdint>
@@ -100,6 +103,11 @@ struct Part27 {
     double phi[3];                  // cube origin - x of the current map
     double dP[3], dL[3], dm;        // terms of the last remap (dm: its mass, returned at the next collision)
     double rec[25];                 // F0, T0, F, T, U, Omega, x, q of the last iteration
+    // for the next solve, from the auxiliary kernel
+    double In[9];                   // lab inertia I(t)
+    double A6[36];                  // matrix of Eq. Fdiscrete / Eq. Tdiscrete
+    float Ai[36];                   // its inverse, FP32
+    int inv_ok;                     // 1: no pivot vanished
     int o[3];                       // unwrapped cube origin of the current map
     int S, h, slot, nsolid, box;
     int pad;
@@ -151,6 +159,7 @@ struct FieldParams27 {
 cudaError_t launch_lattice27(const LatParams27& p, int blocks, cudaStream_t s);
 cudaError_t launch_bulk27(const LatParams27& p, int blocks, cudaStream_t s);   // LAT_BULK only
 cudaError_t launch_particles27(const PartParams27& p, int np, cudaStream_t s);
+cudaError_t launch_particles27_aux(const PartParams27& p, int np, cudaStream_t s);
 cudaError_t launch_fields27(const FieldParams27& p, int blocks, cudaStream_t s);
 cudaError_t launch_refresh27(const Part27* pd, const Box27* boxes, Dyn27* dyn, int np, cudaStream_t s);
 cudaError_t launch_links27(const Part27* pd, const Box27* boxes, const uint64_t* rows, int p, int* out, int cap,
