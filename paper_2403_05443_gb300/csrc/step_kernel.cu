@@ -16,14 +16,21 @@
 //   - bulk work (bulk_tile.cuh), every other node of every box, taken by
 //     every warp from a counter in units of 32 quads (128 nodes), so that the
 //     warps of a block load and compute out of step with each other; the next
-//     unit is fetched while one runs.
+//     unit is fetched while one runs.  Even and odd warps take even and odd
+//     units, each from a counter on a line of its own: one counter for all 2,432
+//     warps served an addition every 2-3.6 ns (its L2 slice has the populations to
+//     serve too), which held back every batch with many units.  Two counters, us
+//     per step: 8 boxes of 128^3 nodes in FP32 482 -> 384, the 32 squirmer boxes in
+//     BF16 407 -> 387, 8 of 64^3 in FP16 40.3 -> 39.3 and in FP32 56.7 -> 56.9.
+//     Four are no faster, and with eight a class whose warps fall behind leaves a
+//     tail (16 particles in 128^3 nodes: 6 % slower).
 // A grid barrier ends the iteration: after it the lattice of step t, the box
 // terms and the redo masks of step t+1 are complete.  The auxiliary block of
 // the last iteration runs first in the next launch: a launch ends at its last
 // barrier, with the arrival and item counters at zero, so launches follow each
 // other with no reset in between.  The iterations take their bulk units from
-// two counters in turn (by barrier generation), each cleared by block 0 while
-// the other one is in use.
+// two sets of counters in turn (by barrier generation), each cleared by block 0
+// while the other one is in use.
 //
 // Cross-block data are read through L2 (ld.global.cg, see lattice_common.cuh).
 // Every wait is bounded: a barrier that waits longer than SPIN_LIMIT polls
@@ -35,10 +42,15 @@
 
 namespace lbsph {
 
-constexpr int SYNC_BAR = 0;          // barrier arrivals (zero between barriers)
+constexpr int SYNC_BAR = 544;        // barrier arrivals (zero between barriers), on a line of their own
 constexpr int SYNC_GEN = 2;          // barrier generation (counts up, wraps), 8-byte aligned with
 constexpr int SYNC_ABORT = 3;        //   the abort flag: nonzero once a wait ran out
-constexpr int SYNC_WORK = 4;         // + (generation & 1): bulk units taken in the iteration of that generation
+// counters the bulk units are taken from, by the parity of the warp: warp w of a block takes the units u = w (mod NCLASS)
+constexpr int NCLASS = 2;
+// + ((generation & 1) * NCLASS + class) * 32: units of the class taken in the iteration of that generation
+constexpr int SYNC_WORK = 32;
+static_assert(SYNC_WORK + 2 * NCLASS * 32 <= SYNC_BAR && SYNC_BAR < SYNC_HDR, "the work counters precede the item counters");
+static_assert((KBLOCK / 32) % NCLASS == 0, "as many units and as many warps in every class");
 constexpr int SYNC_PART = SYNC_HDR;  // + p: items of particle p done in this iteration
 constexpr int MAX_GRID = 4096;
 constexpr long long SPIN_LIMIT = 1ll << 22;   // polls (an L2 read, then a 64 ns sleep): a few seconds
@@ -156,9 +168,10 @@ __global__ void __launch_bounds__(KBLOCK, 2) step_kernel(const __grid_constant__
         // the generation before this launch's first barrier (no block can pass
         // that barrier before every block has read it)
         s_gen = *reinterpret_cast<volatile unsigned*>(SP.sync + SYNC_GEN);
-        // the work counter of the first iteration was the last launch's last
-        // one: clear it (the launches on a stream do not overlap)
-        if (blockIdx.x == 0) SP.sync[SYNC_WORK + ((s_gen + 1) & 1)] = 0;
+        // the work counters of the first iteration were the last launch's last
+        // ones: clear them (the launches on a stream do not overlap)
+        if (blockIdx.x == 0)
+            for (int w = 0; w < NCLASS; ++w) SP.sync[SYNC_WORK + (((s_gen + 1) & 1) * NCLASS + w) * 32] = 0;
     }
     if (!grid_barrier(SP, s_gen)) return;
     {
@@ -172,16 +185,15 @@ __global__ void __launch_bounds__(KBLOCK, 2) step_kernel(const __grid_constant__
     }
     __syncthreads();
     const int prank = s_rank;
-    const int nwarps = (int)gridDim.x * (KBLOCK / 32);
     for (int it = 0; it < SP.iters; ++it) {
         const int cur = (SP.cur0 + it) & 1;
         const BulkParams& BP = SP.bulk[cur];
         const BndParams& NP = SP.bnd[cur];
         const PParams& PP = SP.part[cur];
         const unsigned gen = s_gen;
-        unsigned* work = SP.sync + SYNC_WORK + (gen & 1);
-        // the other work counter (the last iteration's) for the next iteration
-        if (blockIdx.x == 0 && tid == 0) SP.sync[SYNC_WORK + ((gen + 1) & 1)] = 0;
+        unsigned* work = SP.sync + SYNC_WORK + ((gen & 1) * NCLASS + (tid >> 5) % NCLASS) * 32;
+        // the other work counters (the last iteration's) for the next iteration
+        if (blockIdx.x == 0 && tid < NCLASS) SP.sync[SYNC_WORK + (((gen + 1) & 1) * NCLASS + tid) * 32] = 0;
         // ---- particle items
         for (int item = prank; item < npart; item += gridDim.x) {
             const int p = item / (gx + 1), c = item % (gx + 1);
@@ -221,16 +233,15 @@ __global__ void __launch_bounds__(KBLOCK, 2) step_kernel(const __grid_constant__
             __syncthreads();
         }
         // ---- bulk work in warp-sized units (32 quads of a tile): SP.fetch
-        // consecutive units per fetch from the counter while more than two
-        // rounds of such fetches remain, then single units, so that the last
-        // units to finish are short; no block barrier, each warp moves on as
-        // soon as its stores are issued; the next fetch is issued before the
+        // consecutive units of the warp's class per fetch from its counter while
+        // more than two rounds of such fetches remain, then single units, so that
+        // the last units to finish are short; no block barrier, each warp moves on
+        // as soon as its stores are issued; the next fetch is issued before the
         // current units run
         {
-            const int lane = tid & 31;
-            const int units = SP.tiles * (KBLOCK / 32);
-            const int fetch = SP.fetch;
-            const int coarse_end = units - 2 * nwarps * fetch;
+            const int lane = tid & 31, cls = (tid >> 5) % NCLASS;
+            const int units = SP.tiles * (KBLOCK / 32 / NCLASS), fetch = SP.fetch;     // of this warp's class
+            const int coarse_end = units - 2 * (int)gridDim.x * (KBLOCK / 32 / NCLASS) * fetch;
             int u = 0, nf = fetch;
             if (lane == 0) u = (int)atomicAdd(work, (unsigned)fetch);
             u = __shfl_sync(0xffffffffu, u, 0);
@@ -239,7 +250,10 @@ __global__ void __launch_bounds__(KBLOCK, 2) step_kernel(const __grid_constant__
                 nf = u + nf < coarse_end ? fetch : 1;
                 int nu = 0;
                 if (lane == 0) nu = (int)atomicAdd(work, (unsigned)nf);
-                for (int v = u; v < end; ++v) bulk_tile<St, false>(BP, v >> 3, ((v & 7) << 5) + lane);
+                for (int v = u; v < end; ++v) {
+                    const int w = v * NCLASS + cls;
+                    bulk_tile<St, false>(BP, w >> 3, ((w & 7) << 5) + lane);
+                }
                 u = __shfl_sync(0xffffffffu, nu, 0);
             }
         }
