@@ -31,10 +31,16 @@ __device__ __forceinline__ long long warp_sum(long long v)
     return v;
 }
 
-// block c (of P.gx) of particle p; BBLOCK threads
+// block c (of P.gx) of particle p; BBLOCK threads.  A function of its own, as the
+// critical and the auxiliary block are: inlined into the step kernel they cost the bulk
+// loop registers (spilled ones, in some builds; us per step, with and without inlining:
+// 8 boxes of 64^3 in FP32 56.3 / 55.0 and in FP16 39.1 / 37.0, the 32 squirmer boxes in
+// BF16 404 / 380).  The parameters are copied once at its start: read through the
+// reference each is a load on the particle's chain (channel 33.6 / 32.1 us).
 template <class St, bool FIRST>
-__device__ __forceinline__ void boundary_block(const BndParams& P, int p, int c)
+__device__ __noinline__ void boundary_block(const BndParams& kernel_params, int p, int c)
 {
+    const BndParams P = kernel_params;
     using T = typename St::T;
     constexpr int NW = BBLOCK / 32;
     const int gx = P.gx;
@@ -99,6 +105,12 @@ __device__ __forceinline__ void boundary_block(const BndParams& P, int p, int c)
         if (ax < 0 || ax >= S || ay < 0 || ay >= S || az < 0 || az >= S) return false;
         return (s_old[az * S + ay] >> ax) & 1ull;
     };
+    // the nodes ax - 1, ax, ax + 1 of row (ay, az) of a map (0 <= x < S inside) as bits 0..2
+    auto row3 = [&](const uint64_t* map, int ax, int ay, int az) -> unsigned {
+        if (ax < -1 || ax > S || ay < 0 || ay >= S || az < 0 || az >= S) return 0u;
+        const uint64_t w = map[az * S + ay];
+        return (unsigned)(ax >= 1 ? w >> (ax - 1) : w << (1 - ax)) & 7u;
+    };
     // a node (X, Y, Z in the box) in partner j's new or old cube: its local coordinates
     auto ploc = [&](int j, bool nw, int X_, int Y_, int Z_, int& lx, int& ly, int& lz) -> bool {
         const int* ow = nw ? s_pk[j].ow_new : s_pk[j].ow_old;
@@ -148,7 +160,7 @@ __device__ __forceinline__ void boundary_block(const BndParams& P, int p, int c)
     if (tid == 0 && total > cap) atomicOr(P.status, ST_CAPACITY);
     const int count = min(total, cap);
 
-    const long long N = K.N;
+    const int N = (int)K.N;
     const T* A = reinterpret_cast<const T*>(P.src) + K.off;
     const float inv = K.inv_scale, rho0 = K.rho0f, scale = K.scale;
     const unsigned long long pol = l2_evict_normal();
@@ -175,14 +187,14 @@ __device__ __forceinline__ void boundary_block(const BndParams& P, int p, int c)
         const int e = rnd * (BBLOCK / 2) + wpair * 32 + lane;
         bool act = e < count;
         int mx = 0, my = 0, mz = 0, X = 0, Y = 0, Z = 0;
-        long long own = 0;
+        int own = 0;                                // offsets within a box fit 32 bits: 19 N < 2^31
         bool wallrow = false, sol_new = false, sol_old = false;
         int pn = -1, po = -1;
         if (act) {
             const unsigned code = s_list[e];
             mx = code & 0xff; my = (code >> 8) & 0xff; mz = (code >> 16) & 0xff;
             X = wrapd(K.ow_new[0] + mx, nx); Y = wrapd(K.ow_new[1] + my, ny); Z = wrapd(K.ow_new[2] + mz, nz);
-            own = ((long long)Z * ny + Y) * nx + X;
+            own = (Z * ny + Y) * nx + X;
             wallrow = walls && (Y == 0 || Y == ny - 1);
             sol_new = bit_new(mx, my, mz);
             sol_old = !FIRST && bit_old(mx, my, mz);
@@ -242,16 +254,26 @@ __device__ __forceinline__ void boundary_block(const BndParams& P, int p, int c)
             // first collision: the node's initial distributions, no streaming
 #pragma unroll
             for (int i = 0; i < Q; ++i)
-                if (mine(i)) f[i] = St::ld1(A + ((long long)i * N + own), inv, pol);
+                if (mine(i)) f[i] = St::ld1(A + (i * N + own), inv, pol);
         } else if (kind == 4) {
             // fluid at t-1: decide every source first, then issue the loads together
             unsigned bb = 0, wl = 0, pb = 0;        // own, wall and partner bounce-back
+            unsigned ro[3][3];                      // the old map around the node, rows (y + a - 1, z + b - 1)
+            int zy[3][3];
+            const int xs[3] = {wrapd(X - 1, nx), X, wrapd(X + 1, nx)};
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int b = 0; b < 3; ++b) {
+                    ro[a][b] = row3(s_old, mx + dsh[0], my + dsh[1] + a - 1, mz + dsh[2] + b - 1);
+                    zy[a][b] = (wrapd(Z + b - 1, nz) * ny + wrapd(Y + a - 1, ny)) * nx;
+                }
 #pragma unroll
             for (int i = 1; i < Q; ++i) {
                 if (!mine(i)) continue;
                 const int Ys = Y - cy_of(i);
                 if (walls && (Ys == 0 || Ys == ny - 1)) wl |= 1u << i;
-                else if (bit_old(mx - cx_of(i), my - cy_of(i), mz - cz_of(i))) bb |= 1u << i;
+                else bb |= ((ro[1 - cy_of(i)][1 - cz_of(i)] >> (1 - cx_of(i))) & 1u) << i;
             }
             if (nnb > 0) {
                 for (int i = 1; i < Q; ++i) {
@@ -260,62 +282,74 @@ __device__ __forceinline__ void boundary_block(const BndParams& P, int p, int c)
                     for (int j = 0; j < nnb; ++j)
                         if (pbit(j, false, Xs, Ys, Zs)) pb |= 1u << i;
                 }
-                bb |= pb;
             }
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 if (!mine(i)) continue;
-                const bool back = ((bb | wl) >> i) & 1u;
-                const long long src = back ? (long long)opp_of(i) * N + own
-                                           : (long long)i * N + ((long long)wrapd(Z - cz_of(i), nz) * ny + wrapd(Y - cy_of(i), ny)) * nx +
-                                                 wrapd(X - cx_of(i), nx);
-                f[i] = St::ld1(A + src, inv, pol);
+                const bool back = ((bb | wl | pb) >> i) & 1u;
+                f[i] = St::ld1(A + (back ? opp_of(i) * N + own : i * N + zy[1 - cy_of(i)][1 - cz_of(i)] + xs[1 - cx_of(i)]), inv, pol);
             }
-            // mid-link bounce-back terms: + 6 w_i rho0 (u_b . c_i) (Eq. fb, Eq. ub, Eq. ubsquirmer)
-            const float ex[3] = {K.e_old[0], K.e_old[1], K.e_old[2]};
+            // mid-link bounce-back terms: + 6 w_i rho0 (u_b . c_i) (Eq. fb, Eq. ub, Eq. ubsquirmer).  Walls and a passive
+            // body's own links without a branch per direction; the rest (squirmers, partners) in one loop over the
+            // links, so that its code, which most nodes skip, stays small: with all of it once per direction the warps
+            // waited for instructions (an item's nodes 6.3 us after its list, of 23.7 per iteration of a 32^3 box; now 20.1,
+            // and 36.1 -> 32.3 for a channel of 128 x 64 x 128 nodes)
+            if (walls) {
 #pragma unroll
-            for (int i = 1; i < Q; ++i) {
-                if (!mine(i) || !(((bb | wl) >> i) & 1u)) continue;
-                float ubc;
-                if ((wl >> i) & 1u) {
+                for (int i = 1; i < Q; ++i) {
+                    if (!mine(i) || cy_of(i) == 0) continue;
                     const float* uw = (Y - cy_of(i) == 0) ? K.uw_lo : K.uw_hi;
-                    ubc = cx_of(i) * uw[0] + cy_of(i) * uw[1] + cz_of(i) * uw[2];
-                } else if ((pb >> i) & 1u) {
+                    const float ubc = cx_of(i) * uw[0] + cy_of(i) * uw[1] + cz_of(i) * uw[2];
+                    f[i] = (wl >> i) & 1u ? f[i] + 6.0f * w_of(i) * rho0 * ubc : f[i];
+                }
+            }
+            const bool squirmer = K.squirmer != 0;
+            // r_b = x - c_i/2 - x_c(t-1) = ro_old + dsh + m - c_i/2
+            const float p0 = K.ro_old[0] + (float)(dsh[0] + mx), p1 = K.ro_old[1] + (float)(dsh[1] + my),
+                        p2 = K.ro_old[2] + (float)(dsh[2] + mz);
+            if (!squirmer) {
+#pragma unroll
+                for (int i = 1; i < Q; ++i) {
+                    if (!mine(i)) continue;
+                    const float px = p0 - 0.5f * cx_of(i), py = p1 - 0.5f * cy_of(i), pz = p2 - 0.5f * cz_of(i);
+                    const float ux = K.U[0] + (K.W[1] * pz - K.W[2] * py);
+                    const float uy = K.U[1] + (K.W[2] * px - K.W[0] * pz);
+                    const float uz = K.U[2] + (K.W[0] * py - K.W[1] * px);
+                    const float ubc = cx_of(i) * ux + cy_of(i) * uy + cz_of(i) * uz;
+                    f[i] = (bb >> i) & 1u ? f[i] + 6.0f * w_of(i) * rho0 * ubc : f[i];
+                }
+            }
+#pragma unroll 1
+            for (unsigned m = squirmer ? bb | pb : pb; m != 0; m &= m - 1) {
+                const int i = __ffs((int)m) - 1;
+                const int cx = c_of(pack_c(0), i), cy = c_of(pack_c(1), i), cz = c_of(pack_c(2), i);
+                const PartK* Kq = &K;
+                float px = p0 - 0.5f * cx, py = p1 - 0.5f * cy, pz = p2 - 0.5f * cz;
+                if ((pb >> i) & 1u) {
                     // a partner's surface: its velocity at r_b = x - c_i/2 - x_c(t) of that body
-                    const int Xs = wrapd(X - cx_of(i), nx), Ys = wrapd(Y - cy_of(i), ny), Zs = wrapd(Z - cz_of(i), nz);
+                    const int Xs = wrapd(X - cx, nx), Ys = wrapd(Y - cy, ny), Zs = wrapd(Z - cz, nz);
                     int j = 0;
                     while (j < nnb - 1 && !pbit(j, false, Xs, Ys, Zs)) ++j;
-                    const PartK& Kq = s_pk[j];
+                    Kq = &s_pk[j];
                     int l0, l1, l2;
                     ploc(j, false, X, Y, Z, l0, l1, l2);
-                    const float px = Kq.ro_old[0] + (float)l0 - 0.5f * cx_of(i);
-                    const float py = Kq.ro_old[1] + (float)l1 - 0.5f * cy_of(i);
-                    const float pz = Kq.ro_old[2] + (float)l2 - 0.5f * cz_of(i);
-                    float ux = Kq.U[0] + (Kq.W[1] * pz - Kq.W[2] * py);
-                    float uy = Kq.U[1] + (Kq.W[2] * px - Kq.W[0] * pz);
-                    float uz = Kq.U[2] + (Kq.W[0] * py - Kq.W[1] * px);
-                    if (Kq.squirmer) {
-                        float qx, qy, qz;
-                        squirmer_slip(Kq.e_old, Kq.a, Kq.eps2, Kq.B1, Kq.B2, px, py, pz, qx, qy, qz);
-                        ux += qx; uy += qy; uz += qz;
-                    }
-                    ubc = cx_of(i) * ux + cy_of(i) * uy + cz_of(i) * uz;
-                } else {
-                    // r_b = x - c_i/2 - x_c(t-1) = ro_old + dsh + m - c_i/2
-                    const float px = K.ro_old[0] + (float)(dsh[0] + mx) - 0.5f * cx_of(i);
-                    const float py = K.ro_old[1] + (float)(dsh[1] + my) - 0.5f * cy_of(i);
-                    const float pz = K.ro_old[2] + (float)(dsh[2] + mz) - 0.5f * cz_of(i);
-                    float ux = K.U[0] + (K.W[1] * pz - K.W[2] * py);
-                    float uy = K.U[1] + (K.W[2] * px - K.W[0] * pz);
-                    float uz = K.U[2] + (K.W[0] * py - K.W[1] * px);
-                    if (K.squirmer) {
-                        float qx, qy, qz;
-                        squirmer_slip(ex, K.a, K.eps2, K.B1, K.B2, px, py, pz, qx, qy, qz);
-                        ux += qx; uy += qy; uz += qz;
-                    }
-                    ubc = cx_of(i) * ux + cy_of(i) * uy + cz_of(i) * uz;
+                    px = Kq->ro_old[0] + (float)l0 - 0.5f * cx;
+                    py = Kq->ro_old[1] + (float)l1 - 0.5f * cy;
+                    pz = Kq->ro_old[2] + (float)l2 - 0.5f * cz;
                 }
-                f[i] += 6.0f * w_of(i) * rho0 * ubc;
+                float ux = Kq->U[0] + (Kq->W[1] * pz - Kq->W[2] * py);
+                float uy = Kq->U[1] + (Kq->W[2] * px - Kq->W[0] * pz);
+                float uz = Kq->U[2] + (Kq->W[0] * py - Kq->W[1] * px);
+                if (Kq->squirmer) {
+                    float qx, qy, qz;
+                    squirmer_slip(Kq->e_old, Kq->a, Kq->eps2, Kq->B1, Kq->B2, px, py, pz, qx, qy, qz);
+                    ux += qx; uy += qy; uz += qz;
+                }
+                const float ubc = cx * ux + cy * uy + cz * uz;
+                const float t = 6.0f * w_of(i) * rho0 * ubc;
+#pragma unroll
+                for (int k = 1; k < Q; ++k)
+                    if (mine(k)) f[k] = k == i ? f[k] + t : f[k];
             }
         }
         // ---- the node's moments: this warp's part and the partner warp's
@@ -366,20 +400,26 @@ __device__ __forceinline__ void boundary_block(const BndParams& P, int p, int c)
             collide_half<St::GHOST, H>(f, tot, K.omega, rho0, dyn.g[0], dyn.g[1], dyn.g[2], dyn.eps);
 #pragma unroll
             for (int i = 0; i < Q; ++i)
-                if (mine(i)) St::st1(D + (long long)i * N + own, f[i], scale, pol);
+                if (mine(i)) St::st1(D + (i * N + own), f[i], scale, pol);
             // momentum-exchange sums of the new links (x, b), with f*(t)
-            long long fx = 0, fy = 0, fz = 0;
-            bool any = false;
+            unsigned rn[3][3], lk = 0u;             // the new map around the node; the links into it
 #pragma unroll
-            for (int b = 1; b < Q; ++b) {
-                if (!mine(b) || !bit_new(mx + cx_of(b), my + cy_of(b), mz + cz_of(b))) continue;
-                const long long d = fixq(f[b]);
-                any = true;
-                if (cx_of(b) == 1) fx += d; else if (cx_of(b) == -1) fx -= d;
-                if (cy_of(b) == 1) fy += d; else if (cy_of(b) == -1) fy -= d;
-                if (cz_of(b) == 1) fz += d; else if (cz_of(b) == -1) fz -= d;
-            }
-            if (any) {
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int b = 0; b < 3; ++b) rn[a][b] = row3(s_new, mx, my + a - 1, mz + b - 1);
+#pragma unroll
+            for (int b = 1; b < Q; ++b)
+                if (mine(b)) lk |= ((rn[1 + cy_of(b)][1 + cz_of(b)] >> (1 + cx_of(b))) & 1u) << b;
+            if (lk) {
+                long long fx = 0, fy = 0, fz = 0;
+#pragma unroll
+                for (int b = 1; b < Q; ++b) {
+                    if (!mine(b)) continue;
+                    const long long d = fixq((lk >> b) & 1u ? f[b] : 0.0f);
+                    if (cx_of(b) == 1) fx += d; else if (cx_of(b) == -1) fx -= d;
+                    if (cy_of(b) == 1) fy += d; else if (cy_of(b) == -1) fy -= d;
+                    if (cz_of(b) == 1) fz += d; else if (cz_of(b) == -1) fz -= d;
+                }
                 aF[0] += fx; aF[1] += fy; aF[2] += fz;
                 aT[0] += my * fz - mz * fy;
                 aT[1] += mz * fx - mx * fz;
@@ -407,7 +447,7 @@ __device__ __forceinline__ void boundary_block(const BndParams& P, int p, int c)
             // solid now: zero it (never read as a source)
 #pragma unroll
             for (int i = 0; i < Q; ++i)
-                if (mine(i)) St::st1(D + (long long)i * N + own, 0.0f, scale, pol);
+                if (mine(i)) St::st1(D + (i * N + own), 0.0f, scale, pol);
         }
     };
     for (int rnd = 0; rnd < rounds; ++rnd) {

@@ -480,6 +480,16 @@ __device__ __forceinline__ void collide_half(float (&f)[Q], const float (&t)[NT]
     }
 }
 
+// D3Q19 velocity components packed two bits per direction (value + 1), so that
+// a rolled loop over directions stays small in the instruction cache
+__host__ __device__ constexpr unsigned long long pack_c(int comp)
+{
+    unsigned long long v = 0;
+    for (int b = 0; b < Q; ++b) v |= (unsigned long long)((comp == 0 ? cx_of(b) : (comp == 1 ? cy_of(b) : cz_of(b))) + 1) << (2 * b);
+    return v;
+}
+__device__ __forceinline__ int c_of(unsigned long long packed, int b) { return (int)((packed >> (2 * b)) & 3ull) - 1; }
+
 __device__ __forceinline__ long long fixp(float v) { return __float2ll_rn(v * FIXF); }
 
 __device__ __forceinline__ int wrapd(int m, int L) { return m < 0 ? m + L : (m >= L ? m - L : m); }

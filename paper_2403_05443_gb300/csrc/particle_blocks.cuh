@@ -254,9 +254,10 @@ __device__ inline void canon_shape_warp(const double inv[3], const double q[4], 
 // torque for this step and from then on; io_rec (25 doubles) receives its
 // record after the step.  Either may be null.  Both may be pinned host memory
 // that the GPU reads and writes directly.
-__device__ __forceinline__ void crit_block(const PParams& P, int p, const double* io_ft = nullptr,
+static __device__ __noinline__ void crit_block(const PParams& kernel_params, int p, const double* io_ft = nullptr,
                                            double* io_rec = nullptr)
 {
+    const PParams P = kernel_params;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __shared__ PartDev S;
     __shared__ PartK K;
@@ -556,31 +557,12 @@ __device__ __forceinline__ void crit_block(const PParams& P, int p, const double
     __syncthreads();
 
     // ---- warp 0: the shape matrix of the exact test (FP64, needed only if a
-    // node turns out ambiguous, formed while the other warps build the map) and
-    // the force and torque records; warps 1..: occupancy of the new pose, one
-    // row per thread, FP32 test per node, near-surface nodes listed for the
-    // exact test.
+    // node turns out ambiguous, formed while the other warps build the map);
+    // warps 1..: occupancy of the new pose, one row per thread, FP32 test per
+    // node, near-surface nodes listed for the exact test.
     const uint64_t maskS = Sd >= 64 ? ~0ull : ((1ull << Sd) - 1ull);
     if (warp == 0) {
         canon_shape_warp(S.inv_semi2, S.q, s_E, s_A, lane);
-        if (!P.init) {
-            // F = F0 - zeta_FU U' - zeta_FOmega Omega' (Eq. Fsplit) + the
-            // lubrication force, T likewise (Eq. Tsplit)
-            const int row = lane < 6 ? lane : 5;
-            double ft = s_ft0[row] + (row < 3 ? s_FL[row] : 0.0);
-#pragma unroll
-            for (int j = 0; j < 6; ++j) ft -= S.zeta[row * 6 + j] * s_x6[j];
-            if (lane < 6) {
-                S.rec[lane] = s_ft0[lane];
-                S.rec[6 + lane] = ft;
-            }
-            __syncwarp();
-            if (lane < 25) {
-                // exponent all ones: Inf or NaN
-                const unsigned long long b = (unsigned long long)__double_as_longlong(S.rec[lane]);
-                if (((b >> 52) & 0x7ff) == 0x7ff) atomicOr(P.status, ST_NAN);
-            }
-        }
     } else {
         // Along a row the value v(dx) = a dx^2 + 2 b dx + c is a convex quadratic,
         // so the row's solid nodes form one interval between its roots.  Nodes at
@@ -724,6 +706,18 @@ __device__ __forceinline__ void crit_block(const PParams& P, int p, const double
         if (lane == 0 && ns) atomicAdd(&s_nsolid, ns);
     }
     __syncthreads();
+    // ---- the box's uniform terms of the next collision: body force with the
+    // counter force over the fluid nodes, and the mass put back
+    auto box_terms = [&](double fx, double fy, double fz, double dm, long long ns) {
+        const float nf = (float)(K.N - K.nwall - ns);
+        const float inf = nf > 0.0f ? 1.0f / nf : 0.0f;
+        BoxDyn d;
+        d.g[0] = K.body[0] - (K.counter ? (float)fx * inf : 0.0f);
+        d.g[1] = K.body[1] - (K.counter ? (float)fy * inf : 0.0f);
+        d.g[2] = K.body[2] - (K.counter ? (float)fz * inf : 0.0f);
+        d.eps = (float)dm * inf;
+        return d;
+    };
     // ---- redo mask of step t+1 in the new cube: nodes fluid now with a solid
     // neighbour now or before, or solid before (uncovered), and nodes covered now;
     // the bulk kernel of t+1 skips them and the boundary kernel writes them
@@ -747,7 +741,35 @@ __device__ __forceinline__ void crit_block(const PParams& P, int p, const double
         // rows more than one row from every row solid now or before have no
         // solid neighbour: nothing to redo there
         const int ry0 = s_ext[0] - 1, ry1 = s_ext[1] + 1, rz0 = s_ext[2] - 1, rz1 = s_ext[3] + 1;
-        for (int r = tid; r < Sd * Sd; r += CBLOCK) {
+        // the last warp meanwhile: the box terms of a box's only particle, and the
+        // force and torque records (FP64 chains that nothing here waits for)
+        constexpr int RED = CBLOCK - 32;
+        if (warp == CBLOCK / 32 - 1) {
+            if (lane == 0 && K.pcnt == 1) {
+                const BoxDyn d = box_terms(K.Fext[0], K.Fext[1], K.Fext[2], K.dm_return, s_nsolid);
+                P.box_dyn[K.box] = d;
+                P.pdyn[p] = d;
+            }
+            if (!P.init) {
+                // F = F0 - zeta_FU U' - zeta_FOmega Omega' (Eq. Fsplit) + the
+                // lubrication force, T likewise (Eq. Tsplit)
+                const int row = lane < 6 ? lane : 5;
+                double ft = s_ft0[row] + (row < 3 ? s_FL[row] : 0.0);
+#pragma unroll
+                for (int j = 0; j < 6; ++j) ft -= S.zeta[row * 6 + j] * s_x6[j];
+                if (lane < 6) {
+                    S.rec[lane] = s_ft0[lane];
+                    S.rec[6 + lane] = ft;
+                }
+                __syncwarp();
+                if (lane < 25) {
+                    // exponent all ones: Inf or NaN
+                    const unsigned long long b = (unsigned long long)__double_as_longlong(S.rec[lane]);
+                    if (((b >> 52) & 0x7ff) == 0x7ff) atomicOr(P.status, ST_NAN);
+                }
+            }
+        }
+        for (int r = tid; tid < RED && r < Sd * Sd; r += RED) {
             const int my = r % Sd, mz = r / Sd;
             const int Yu = s_o[1] + my;
             uint64_t nd = 0;
@@ -811,27 +833,7 @@ __device__ __forceinline__ void crit_block(const PParams& P, int p, const double
             P.ring[((size_t)p * 2 + (S.step & 1)) * RINGD + tid] =
                 tid < 3 ? S.x[tid] : (tid < 6 ? S.U[tid - 3] : S.q[tid - 6]);
     }
-    // ---- the box's uniform terms of the next collision: body force with the
-    // counter force over the fluid nodes, and the mass put back
-    auto box_terms = [&](double fx, double fy, double fz, double dm, long long ns) {
-        const float nf = (float)(K.N - K.nwall - ns);
-        const float inf = nf > 0.0f ? 1.0f / nf : 0.0f;
-        BoxDyn d;
-        d.g[0] = K.body[0] - (K.counter ? (float)fx * inf : 0.0f);
-        d.g[1] = K.body[1] - (K.counter ? (float)fy * inf : 0.0f);
-        d.g[2] = K.body[2] - (K.counter ? (float)fz * inf : 0.0f);
-        d.eps = (float)dm * inf;
-        return d;
-    };
-    if (K.pcnt == 1) {
-        // the only particle of its box: no other block to wait for
-        if (tid == 0) {
-            const BoxDyn d = box_terms(K.Fext[0], K.Fext[1], K.Fext[2], K.dm_return, K.nsolid);
-            P.box_dyn[K.box] = d;
-            P.pdyn[p] = d;
-        }
-        return;
-    }
+    if (K.pcnt == 1) return;                    // the only particle of its box: written above
     // several particles: the last block of the box sums them
     __threadfence();
     __syncthreads();
@@ -856,16 +858,6 @@ __device__ __forceinline__ void crit_block(const PParams& P, int p, const double
 }
 
 // ---------------------------------------------------------------------------
-// D3Q19 velocity components packed two bits per direction (value + 1), so that
-// a rolled loop over directions stays small in the instruction cache
-__host__ __device__ constexpr unsigned long long pack_c(int comp)
-{
-    unsigned long long v = 0;
-    for (int b = 0; b < Q; ++b) v |= (unsigned long long)((comp == 0 ? cx_of(b) : (comp == 1 ? cy_of(b) : cz_of(b))) + 1) << (2 * b);
-    return v;
-}
-__device__ __forceinline__ int c_of(unsigned long long packed, int b) { return (int)((packed >> (2 * b)) & 3ull) - 1; }
-
 // Auxiliary particle kernel, after the critical one of iteration t and before
 // the critical one of t+1: everything the next solve needs that depends only
 // on the new pose and map.

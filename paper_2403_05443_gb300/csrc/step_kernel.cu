@@ -118,10 +118,10 @@ __device__ __forceinline__ bool grid_barrier(const StepParams& SP, unsigned& s_g
 // add to their accumulators, so no critical block of a cluster may start before
 // every item of the cluster is done.  Returns the lowest index (the cluster's
 // counter) and the members as a mask over the box's particles (at most MAXPB
-// when any particle has partners).  One thread.
-__device__ __forceinline__ int cluster_of(const PartK* pk, int p, unsigned long long& members, int& size)
+// when any particle has partners).  nnb0: p's partner count, read before its item
+// ran (a load less between the item and the critical block).  One thread.
+__device__ __forceinline__ int cluster_of(const PartK* pk, int p, int nnb0, unsigned long long& members, int& size)
 {
-    const int nnb0 = __ldcg(&pk[p].nnb);
     if (nnb0 == 0) {
         members = 0;
         size = 1;
@@ -197,23 +197,28 @@ __global__ void __launch_bounds__(KBLOCK, 2) step_kernel(const __grid_constant__
         // ---- particle items
         for (int item = prank; item < npart; item += gridDim.x) {
             const int p = item / (gx + 1), c = item % (gx + 1);
+            int nnb0 = 0;
+            if (tid == 0) nnb0 = __ldcg(&PP.pk[p].nnb);
             if (c < gx) boundary_block<St, false>(NP, p, c);
             else aux_block(PP, p);                 // a no-op if it already ran for this pose
-            __threadfence();
+            // the item's writes before its count, the other items' before the
+            // critical block's reads: one thread's fences around the count carry
+            // the block's through the block barriers
             __syncthreads();
             if (tid == 0) {
+                __threadfence();
                 // the last item of the particle's cluster runs the cluster's
                 // critical blocks (a single particle: its own), in index order
                 unsigned long long mem;
                 int size;
-                const int root = cluster_of(PP.pk, p, mem, size);
+                const int root = cluster_of(PP.pk, p, nnb0, mem, size);
                 s_root = root;
                 s_members = mem;
                 s_last = atomicAdd(SP.sync + SYNC_PART + root, 1u) == (unsigned)(size * (gx + 1) - 1);
+                __threadfence();
             }
             __syncthreads();
             if (s_last) {
-                __threadfence();
                 const int root = s_root;
                 if (tid == 0) SP.sync[SYNC_PART + root] = 0;
                 unsigned long long mem = s_members;
