@@ -24,6 +24,13 @@ __device__ __forceinline__ long long fixq(float f)
     return (u >> 31) ? -v : v;
 }
 
+// a b - c d with one rounding less; written out, like the bounce-back terms, so that a
+// node's rounding does not depend on which products the compiler finds in common
+__device__ __forceinline__ float cross_term(float a, float b, float c, float d)
+{
+    return __fmaf_rn(a, b, -__fmul_rn(c, d));
+}
+
 __device__ __forceinline__ long long warp_sum(long long v)
 {
 #pragma unroll
@@ -300,7 +307,7 @@ __device__ __noinline__ void boundary_block(const BndParams& kernel_params, int 
                     if (!mine(i) || cy_of(i) == 0) continue;
                     const float* uw = (Y - cy_of(i) == 0) ? K.uw_lo : K.uw_hi;
                     const float ubc = cx_of(i) * uw[0] + cy_of(i) * uw[1] + cz_of(i) * uw[2];
-                    f[i] = (wl >> i) & 1u ? f[i] + 6.0f * w_of(i) * rho0 * ubc : f[i];
+                    f[i] = (wl >> i) & 1u ? __fmaf_rn(6.0f * w_of(i) * rho0, ubc, f[i]) : f[i];
                 }
             }
             const bool squirmer = K.squirmer != 0;
@@ -312,11 +319,11 @@ __device__ __noinline__ void boundary_block(const BndParams& kernel_params, int 
                 for (int i = 1; i < Q; ++i) {
                     if (!mine(i)) continue;
                     const float px = p0 - 0.5f * cx_of(i), py = p1 - 0.5f * cy_of(i), pz = p2 - 0.5f * cz_of(i);
-                    const float ux = K.U[0] + (K.W[1] * pz - K.W[2] * py);
-                    const float uy = K.U[1] + (K.W[2] * px - K.W[0] * pz);
-                    const float uz = K.U[2] + (K.W[0] * py - K.W[1] * px);
+                    const float ux = K.U[0] + cross_term(K.W[1], pz, K.W[2], py);
+                    const float uy = K.U[1] + cross_term(K.W[2], px, K.W[0], pz);
+                    const float uz = K.U[2] + cross_term(K.W[0], py, K.W[1], px);
                     const float ubc = cx_of(i) * ux + cy_of(i) * uy + cz_of(i) * uz;
-                    f[i] = (bb >> i) & 1u ? f[i] + 6.0f * w_of(i) * rho0 * ubc : f[i];
+                    f[i] = (bb >> i) & 1u ? __fmaf_rn(6.0f * w_of(i) * rho0, ubc, f[i]) : f[i];
                 }
             }
 #pragma unroll 1
@@ -337,19 +344,19 @@ __device__ __noinline__ void boundary_block(const BndParams& kernel_params, int 
                     py = Kq->ro_old[1] + (float)l1 - 0.5f * cy;
                     pz = Kq->ro_old[2] + (float)l2 - 0.5f * cz;
                 }
-                float ux = Kq->U[0] + (Kq->W[1] * pz - Kq->W[2] * py);
-                float uy = Kq->U[1] + (Kq->W[2] * px - Kq->W[0] * pz);
-                float uz = Kq->U[2] + (Kq->W[0] * py - Kq->W[1] * px);
+                float ux = Kq->U[0] + cross_term(Kq->W[1], pz, Kq->W[2], py);
+                float uy = Kq->U[1] + cross_term(Kq->W[2], px, Kq->W[0], pz);
+                float uz = Kq->U[2] + cross_term(Kq->W[0], py, Kq->W[1], px);
                 if (Kq->squirmer) {
                     float qx, qy, qz;
                     squirmer_slip(Kq->e_old, Kq->a, Kq->eps2, Kq->B1, Kq->B2, px, py, pz, qx, qy, qz);
                     ux += qx; uy += qy; uz += qz;
                 }
                 const float ubc = cx * ux + cy * uy + cz * uz;
-                const float t = 6.0f * w_of(i) * rho0 * ubc;
+                const float c6 = 6.0f * w_of(i) * rho0;
 #pragma unroll
                 for (int k = 1; k < Q; ++k)
-                    if (mine(k)) f[k] = k == i ? f[k] + t : f[k];
+                    if (mine(k)) f[k] = k == i ? __fmaf_rn(c6, ubc, f[k]) : f[k];
             }
         }
         // ---- the node's moments: this warp's part and the partner warp's
