@@ -262,7 +262,7 @@ lb_status lb_profile_step(lb_ctx* ctx, int32_t nsteps, void* stream, double* ms_
  * 100 KB of shared memory and whose threads still cover every row of the
  * largest bounding cube, those above d while every particle item still gets a
  * block of its own), then (2) the number of consecutive 128-node bulk
- * units a warp takes per fetch from the work counter (1, 2, 4, 8), and keeps the
+ * units a warp takes per fetch from its work counter (1, 2, 4, 8), and keeps the
  * fastest of each for later lb_step calls.  The candidates compute the same
  * values bit for bit, so tuning advances the simulation exactly as lb_step
  * would.  out3 (may be NULL): units per fetch kept, blocks per particle kept,

@@ -600,6 +600,16 @@ extern "C" lb_status lb_create(const lb_box_desc* boxes, int32_t nbox, const lb_
     ctx->total_blocks = blk;
     ctx->total_elems = off;
     ctx->maxp = o.max_particles;
+    // Units a warp takes from its counter at a time: one, so that the last ones to
+    // finish are short; in 16-bit storage, whose units are done in half the time, four
+    // from 20 units per warp upward.  Measured with 1 / 4, us per step: the 32 squirmer
+    // boxes in BF16 (75 per warp) 378 / 367, 16 of 96^3 in FP16 (45) 209 / 204, 24 of
+    // 64^3 in BF16 (20) 95.3 / 94.5, 16 of them (13) 65.6 / 66.2; in FP32 8 of 128^3 (54)
+    // 380 / 384, 40 of 64^3 (34) 244 / 251.
+    int nsm = 0;
+    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || nsm < 1) nsm = 1;
+    const long long warps = 2ll * nsm * (KBLOCK / 32);
+    if (ctx->elem == 2 && (long long)blk * (KBLOCK / 32) >= 20 * warps) ctx->fetch = 4;
     size_t tmp = 0;
     for (auto& h : ctx->hbox) tmp = std::max(tmp, (size_t)(19 * h.N) * sizeof(float));
     ctx->tmp_bytes = tmp;
