@@ -297,8 +297,8 @@ __device__ __noinline__ void boundary_block(const BndParams& kernel_params, int 
                 f[i] = St::ld1(A + (back ? opp_of(i) * N + own : i * N + zy[1 - cy_of(i)][1 - cz_of(i)] + xs[1 - cx_of(i)]), inv, pol);
             }
             // mid-link bounce-back terms: + 6 w_i rho0 (u_b . c_i) (Eq. fb, Eq. ub, Eq. ubsquirmer).  Walls and a passive
-            // body's own links without a branch per direction; the rest (squirmers, partners) in one loop over the
-            // links, so that its code, which most nodes skip, stays small: with all of it once per direction the warps
+            // body's own links without a branch per direction; a squirmer's apart; partners' in one loop over the links,
+            // so that code which most nodes skip stays small: with all of it once per direction the warps
             // waited for instructions (an item's nodes 6.3 us after its list, of 23.7 per iteration of a 32^3 box; now 20.1,
             // and 36.1 -> 32.3 for a channel of 128 x 64 x 128 nodes)
             if (walls) {
@@ -326,24 +326,41 @@ __device__ __noinline__ void boundary_block(const BndParams& kernel_params, int 
                     f[i] = (bb >> i) & 1u ? __fmaf_rn(6.0f * w_of(i) * rho0, ubc, f[i]) : f[i];
                 }
             }
+            if (squirmer) {
+                // its own links one by one: the slip is long, and a link is taken by few lanes
+                const float ex[3] = {K.e_old[0], K.e_old[1], K.e_old[2]};
+#pragma unroll
+                for (int i = 1; i < Q; ++i) {
+                    if (!mine(i) || !((bb >> i) & 1u)) continue;
+                    const float px = K.ro_old[0] + (float)(dsh[0] + mx) - 0.5f * cx_of(i);
+                    const float py = K.ro_old[1] + (float)(dsh[1] + my) - 0.5f * cy_of(i);
+                    const float pz = K.ro_old[2] + (float)(dsh[2] + mz) - 0.5f * cz_of(i);
+                    float ux = K.U[0] + (K.W[1] * pz - K.W[2] * py);
+                    float uy = K.U[1] + (K.W[2] * px - K.W[0] * pz);
+                    float uz = K.U[2] + (K.W[0] * py - K.W[1] * px);
+                    if (K.squirmer) {
+                        float qx, qy, qz;
+                        squirmer_slip(ex, K.a, K.eps2, K.B1, K.B2, px, py, pz, qx, qy, qz);
+                        ux += qx; uy += qy; uz += qz;
+                    }
+                    const float ubc = cx_of(i) * ux + cy_of(i) * uy + cz_of(i) * uz;
+                    f[i] += 6.0f * w_of(i) * rho0 * ubc;
+                }
+            }
 #pragma unroll 1
-            for (unsigned m = squirmer ? bb | pb : pb; m != 0; m &= m - 1) {
+            for (unsigned m = pb; m != 0; m &= m - 1) {
                 const int i = __ffs((int)m) - 1;
                 const int cx = c_of(pack_c(0), i), cy = c_of(pack_c(1), i), cz = c_of(pack_c(2), i);
-                const PartK* Kq = &K;
-                float px = p0 - 0.5f * cx, py = p1 - 0.5f * cy, pz = p2 - 0.5f * cz;
-                if ((pb >> i) & 1u) {
-                    // a partner's surface: its velocity at r_b = x - c_i/2 - x_c(t) of that body
-                    const int Xs = wrapd(X - cx, nx), Ys = wrapd(Y - cy, ny), Zs = wrapd(Z - cz, nz);
-                    int j = 0;
-                    while (j < nnb - 1 && !pbit(j, false, Xs, Ys, Zs)) ++j;
-                    Kq = &s_pk[j];
-                    int l0, l1, l2;
-                    ploc(j, false, X, Y, Z, l0, l1, l2);
-                    px = Kq->ro_old[0] + (float)l0 - 0.5f * cx;
-                    py = Kq->ro_old[1] + (float)l1 - 0.5f * cy;
-                    pz = Kq->ro_old[2] + (float)l2 - 0.5f * cz;
-                }
+                // a partner's surface: its velocity at r_b = x - c_i/2 - x_c(t) of that body
+                const int Xs = wrapd(X - cx, nx), Ys = wrapd(Y - cy, ny), Zs = wrapd(Z - cz, nz);
+                int j = 0;
+                while (j < nnb - 1 && !pbit(j, false, Xs, Ys, Zs)) ++j;
+                const PartK* Kq = &s_pk[j];
+                int l0, l1, l2;
+                ploc(j, false, X, Y, Z, l0, l1, l2);
+                const float px = Kq->ro_old[0] + (float)l0 - 0.5f * cx;
+                const float py = Kq->ro_old[1] + (float)l1 - 0.5f * cy;
+                const float pz = Kq->ro_old[2] + (float)l2 - 0.5f * cz;
                 float ux = Kq->U[0] + cross_term(Kq->W[1], pz, Kq->W[2], py);
                 float uy = Kq->U[1] + cross_term(Kq->W[2], px, Kq->W[0], pz);
                 float uz = Kq->U[2] + cross_term(Kq->W[0], py, Kq->W[1], px);
