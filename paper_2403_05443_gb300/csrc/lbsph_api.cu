@@ -418,7 +418,8 @@ static lb_status q27_set_particles(lb_ctx* ctx, int box, const lb_particle* p, i
 // One step: the first collision, or a context without particles, is one
 // lattice pass over every node and then the particle kernel; afterwards the
 // nodes of the particles' cube unions (near pass) and the particle kernel run
-// on a stream of their own beside the bulk pass over every other node, and the
+// on a stream of their own beside the bulk pass over every other node, the auxiliary
+// kernel on a third one (only the next particle kernel waits for it), and the
 // next step waits for both.  The particle kernel writes the box terms of the
 // next pass into the other slot of d_dyn27, so the bulk pass never reads a slot
 // that is being written.
