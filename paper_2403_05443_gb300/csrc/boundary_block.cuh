@@ -43,7 +43,7 @@ __device__ __forceinline__ long long warp_sum(long long v)
 // loop registers (spilled ones, in some builds; us per step, with and without inlining:
 // 8 boxes of 64^3 in FP32 56.3 / 55.0 and in FP16 39.1 / 37.0, the 32 squirmer boxes in
 // BF16 404 / 380).  The parameters are copied once at its start: read through the
-// reference each is a load on the particle's chain (channel 33.6 / 32.1 us).
+// reference each is a load on the particle's chain (channel 33.6 / 32.1 us in that comparison).
 template <class St, bool FIRST>
 __device__ __noinline__ void boundary_block(const BndParams& kernel_params, int p, int c)
 {
