@@ -653,6 +653,11 @@ __device__ void q27_refine6(const double* A6, const float* Ai, const double* rhs
 // band around 1; the nodes inside the band are collected and then tested by the
 // exact FP64 test in the oracle's operation order, one node per thread, so the
 // map is bit-identical to the oracle's.  Init mode: the map of the current pose.
+// A pose that is not finite, or too far out for 32-bit cube origins, goes no further
+// than the record and the status word: no node index is ever formed from it.  The
+// body then stays where its current map is, at rest, so that the box terms of the
+// next pass (whose slot may never have been written) are valid, and the other
+// boxes' particles go on as if nothing had happened.
 // Measured, a step with its share of the read-back, before (the link sums, the drag
 // matrix and the solve's elimination in this kernel, 54 us of the chain near pass ->
 // particle kernel -> near pass) and after: one 64^3 box 59.7 -> 50.1 us, four 87.5 ->
@@ -670,7 +675,7 @@ __global__ void __launch_bounds__(PBLK, 1) particle27_kernel(const __grid_consta
     __shared__ double s_A[9], s_E[9], s_x[3], s_phi[3];
     __shared__ double s_F0[3], s_T0[3], s_rhs[6], s_x6[6];
     __shared__ float s_A32[9], s_d0[3];
-    __shared__ int s_o[3], s_ow[3], s_ok, s_nsol, s_ncand;
+    __shared__ int s_o[3], s_ow[3], s_ok, s_solved, s_nsol, s_ncand;
     __shared__ int s_cand[NCAND];
     static_assert(sizeof(Part27) % 8 == 0 && sizeof(Box27) % 4 == 0, "staged as words");
     {
@@ -690,7 +695,7 @@ __global__ void __launch_bounds__(PBLK, 1) particle27_kernel(const __grid_consta
     Part27* D = &sD;
     const Box27& B = sB;
     if (warp == 0) {
-        bool solved = true;
+        bool solved = true, finite = true;
         if (!P.init) {
             if (lane == 0) q27_sums(s_acc, D, B, s_F0, s_T0);
             __syncwarp();
@@ -729,6 +734,8 @@ __global__ void __launch_bounds__(PBLK, 1) particle27_kernel(const __grid_consta
                 qstep27(D->q, Wm, qn);
                 const int k = lane % 3;
                 const double xn = D->x[k] + 0.5 * (D->U[k] + s_x6[k]);
+                finite = __all_sync(0xffffffffu, isfinite(xn) && isfinite(s_x6[k]) && isfinite(s_x6[k + 3]) && isfinite(qn[0]) &&
+                                                     isfinite(qn[1]) && isfinite(qn[2]) && isfinite(qn[3]));
                 __syncwarp();
                 if (lane < 3) {
                     D->x[lane] = xn;
@@ -744,27 +751,31 @@ __global__ void __launch_bounds__(PBLK, 1) particle27_kernel(const __grid_consta
         }
         // the cube of the new pose (origin floor(x) - h, side S = 2h + 2), one axis
         // per lane, and the exact inside-test matrix of the new orientation (lanes 0..8)
+        bool in_range = true;
         if (lane < 3) {
             const int k = lane;
             const int L = k == 0 ? B.nx : (k == 1 ? B.ny : B.nz);
-            const int o = (int)floor(D->x[k]) - D->h;
+            int o;
+            in_range = cube_origin27(D->x[k], D->h, o);
             s_o[k] = o;
             s_ow[k] = ((o % L) + L) % L;
             s_phi[k] = (double)o - D->x[k];
             s_d0[k] = (float)s_phi[k];             // d = X - x_c at cube coordinate 0
             s_x[k] = D->x[k];
         }
-        __syncwarp();
+        in_range = __all_sync(0xffffffffu, in_range);
         canon_shape_warp(D->inv2, D->q, s_E, s_A, lane);
         __syncwarp();
         if (lane < 9) s_A32[lane] = (float)s_A[lane];
         if (lane == 0) {
-            if (!solved) atomicOr(P.status, ST_NAN);
-            s_ok = P.init || (solved && !(__ldcg(P.status) & ST_NAN));
+            if (!P.init && !(solved && finite)) atomicOr(P.status, ST_NAN);
+            else if (!P.init && !in_range) atomicOr(P.status, ST_CAPACITY);
+            s_solved = solved;
+            s_ok = P.init || (solved && finite && in_range);
         }
     }
     __syncthreads();
-    if (!P.init && warp == PBLK / 32 - 1 && D->inv_ok) {
+    if (!P.init && warp == PBLK / 32 - 1 && s_solved) {
         // the record F0, T0, F = F0 - zeta_F (U', W'), T likewise, U, W, x, q (finite or ST_NAN), on a warp with few rows
         double v = 0.0;
         if (lane < 12) {
@@ -782,6 +793,22 @@ __global__ void __launch_bounds__(PBLK, 1) particle27_kernel(const __grid_consta
         if (!__all_sync(0xffffffffu, lane >= 25 || isfinite(v)) && lane == 0) atomicOr(P.status, ST_NAN);
     }
     if (!s_ok) {
+        if (tid < 3) {
+            // the next pass sees the current map, at rest
+            const int i = tid, Lk = i == 0 ? B.nx : (i == 1 ? B.ny : B.nz);
+            Dyn27& Y = P.dyn[D->box];
+            cube_union27(D->o[i], D->o[i], D->S, Lk, Y.uo[i], Y.E[i]);
+            Y.o_old[i] = Y.o_new[i] = Y.uo[i];
+            Y.phi_old[i] = Y.phi_new[i] = (float)D->phi[i];
+            Y.U[i] = Y.W[i] = 0.0f;
+            Y.g[i] = (float)B.body[i];
+            if (i == 0) {
+                Y.slot_old = Y.slot_new = D->slot;
+                Y.S = D->S;
+                Y.active = 1;
+                Y.eps = 0.0f;
+            }
+        }
         __syncthreads();
         for (int k = tid; k < (int)(sizeof(Part27) / 8); k += PBLK)
             reinterpret_cast<unsigned long long*>(G)[k] = reinterpret_cast<const unsigned long long*>(&sD)[k];
@@ -876,11 +903,9 @@ __global__ void __launch_bounds__(PBLK, 1) particle27_kernel(const __grid_consta
         Y.phi_old[i] = P.init ? (float)s_phi[i] : (float)D->phi[i];
         Y.o_old[i] = P.init ? s_ow[i] : ((D->o[i] % Lk) + Lk) % Lk;
         // the box that holds both cubes (the near pass covers its nodes)
-        const int lo = P.init ? s_o[i] : min(D->o[i], s_o[i]);
-        const int hi = (P.init ? s_o[i] : max(D->o[i], s_o[i])) + S;
-        Y.E[i] = min(hi - lo, Lk);
-        Y.uo[i] = ((lo % Lk) + Lk) % Lk;
-        if (!P.init && abs(s_o[i] - D->o[i]) > 1) atomicOr(P.status, ST_CAPACITY);
+        const int o_was = P.init ? s_o[i] : D->o[i];
+        cube_union27(o_was, s_o[i], S, Lk, Y.uo[i], Y.E[i]);
+        if (s_o[i] < o_was - 1 || s_o[i] > o_was + 1) atomicOr(P.status, ST_CAPACITY);
         Y.phi_new[i] = (float)s_phi[i];
         Y.o_new[i] = s_ow[i];
         Y.U[i] = (float)D->U[i];

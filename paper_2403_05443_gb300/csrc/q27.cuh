@@ -25,6 +25,7 @@
 // auxiliary kernel on another, beside the bulk pass and the next near pass.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -63,6 +64,27 @@ __host__ __device__ constexpr double wd27(int i)
     return i == 0 ? 8.0 / 27.0 : (i <= 6 ? 2.0 / 27.0 : (i <= 18 ? 1.0 / 54.0 : 1.0 / 216.0));
 }
 __host__ __device__ constexpr float w27(int i) { return (float)wd27(i); }
+
+// Cube origin floor(x) - h along an axis.  False, and the origin a centre at 0 would have, for a
+// centre that is not finite or so far out that the origin's arithmetic could leave 32 bits.
+constexpr double POS_MAX27 = 536870912.0;        // 2^29
+__host__ __device__ inline bool cube_origin27(double x, int h, int& o)
+{
+    const bool ok = x > -POS_MAX27 && x < POS_MAX27;       // false for NaN
+    o = (ok ? (int)floor(x) : 0) - h;
+    return ok;
+}
+
+// Wrapped origin uo and extent E, along an axis of length L, of the range that holds two cubes of
+// side S <= L.  S <= E <= L and 0 <= uo < L whatever the two origins are: uo + m with m < E wraps
+// into the box by one subtraction, which is all that the near pass does.
+__host__ __device__ inline void cube_union27(int o_a, int o_b, int S, int L, int& uo, int& E)
+{
+    const int lo = o_a < o_b ? o_a : o_b, hi = o_a < o_b ? o_b : o_a;
+    const long long e = (long long)hi - lo + S;
+    E = e < L ? (int)e : L;
+    uo = ((lo % L) + L) % L;
+}
 
 // per box, constant
 struct Box27 {
