@@ -195,7 +195,8 @@ lb_status lb_step(lb_ctx* ctx, int32_t nsteps, void* stream);
 /* Writes the fields `what` (one LB_FIELD_* bit) of box `box` at the current
  * time t: f(x, t) is the pre-collision distribution at the start of
  * iteration t.  dst gets dst_bytes bytes (must equal the field's size); it is
- * device memory when dst_is_device != 0.  Waits for completion. */
+ * device memory when dst_is_device != 0 (memory of the context's device, which the
+ * kernel may write in place).  Waits for completion. */
 lb_status lb_get_fields(lb_ctx* ctx, int32_t box, uint32_t what, void* dst, size_t dst_bytes,
                         int32_t dst_is_device, void* stream);
 

@@ -1215,11 +1215,8 @@ extern "C" lb_status lb_get_force_torque_async(lb_ctx* ctx, int32_t box, double*
     return LB_OK;
 }
 
-// Device address of caller memory of `bytes` bytes that the GPU of the
-// context can read and write directly: its own device memory, managed memory,
-// or page-locked host memory (through its mapped address; both ends of the
-// range must lie in the same mapping).  Null when it cannot (pageable host
-// memory, another GPU), and the caller then copies instead.
+// Device address of caller memory that the context's GPU can use in place (in_place_view), or
+// null: the caller then copies instead.
 static void* device_view(lb_ctx* ctx, const void* p, size_t bytes)
 {
     if (!p || bytes == 0) return nullptr;
@@ -1229,12 +1226,7 @@ static void* device_view(lb_ctx* ctx, const void* p, size_t bytes)
         cudaGetLastError();
         return nullptr;
     }
-    if (a.type != b.type || !a.devicePointer || !b.devicePointer) return nullptr;
-    if (static_cast<const char*>(b.devicePointer) - static_cast<const char*>(a.devicePointer) != (ptrdiff_t)(bytes - 1))
-        return nullptr;
-    if (a.type == cudaMemoryTypeDevice && a.device != ctx->device) return nullptr;
-    if (a.type != cudaMemoryTypeDevice && a.type != cudaMemoryTypeManaged && a.type != cudaMemoryTypeHost) return nullptr;
-    return a.devicePointer;
+    return in_place_view(a, b, bytes, ctx->device);
 }
 
 extern "C" lb_status lb_step_io(lb_ctx* ctx, int32_t nsteps, const double* ft, double* rec, void* stream)
@@ -1360,9 +1352,13 @@ extern "C" lb_status lb_init_fluid(lb_ctx* ctx, int32_t box, const float* u, siz
     float* dd = drho ? ctx->d_tmp + 4 * B.N : nullptr;
     CK(cudaStreamWaitEvent(s, ctx->ev_done, 0));
     const float *us = ud, *ds = dd;
-    if (is_device && ((uintptr_t)u | (uintptr_t)drho) % sizeof(float) == 0) {
-        us = u;                                        // read where they are
-        ds = drho;
+    // read where they are, unless they are not aligned to their element type or not this GPU's
+    const bool aligned = is_device && ((uintptr_t)u | (uintptr_t)drho) % sizeof(float) == 0;
+    const float* uv = aligned ? static_cast<const float*>(device_view(ctx, u, u_bytes)) : nullptr;
+    const float* dv = uv && drho ? static_cast<const float*>(device_view(ctx, drho, (size_t)B.N * sizeof(float))) : nullptr;
+    if (uv && (!drho || dv)) {
+        us = uv;
+        ds = dv;
     } else {
         const cudaMemcpyKind kind = is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
         CK(cudaMemcpyAsync(ud, u, u_bytes, kind, s));
@@ -1401,14 +1397,17 @@ extern "C" lb_status lb_stokes_field(lb_ctx* ctx, int32_t box, float* u_dev, flo
     }
     CK(cudaStreamWaitEvent(s, ctx->ev_done, 0));
     CK(owner_field(ctx, box, s));
-    // straight into the caller's fields, unless they are not aligned to their element type
-    const bool direct = ((uintptr_t)u_dev | (uintptr_t)drho_dev) % sizeof(float) == 0;
+    // straight into the caller's fields, unless they are not aligned to their element type or not this GPU's
+    const bool aligned = ((uintptr_t)u_dev | (uintptr_t)drho_dev) % sizeof(float) == 0;
+    float* uv = aligned ? static_cast<float*>(device_view(ctx, u_dev, 3ull * B.N * sizeof(float))) : nullptr;
+    float* dv = uv && drho_dev ? static_cast<float*>(device_view(ctx, drho_dev, (size_t)B.N * sizeof(float))) : nullptr;
+    const bool direct = uv && (!drho_dev || dv);
     float* out = ctx->d_tmp + B.N;                     // [4][N]: u, then drho
     int* counts = reinterpret_cast<int*>(ctx->d_sums + 8);
     CK(launch_stokes(B, reinterpret_cast<int*>(ctx->d_tmp), ctx->d_pd + B.pbeg, B.pcnt, d.counter_force, d.body_force,
                      ctx->d_stokes, reinterpret_cast<int*>(ctx->d_stokes + 2 * B.N), counts,
-                     reinterpret_cast<float*>(counts + ctx->maxp + 1), ctx->d_sums, direct ? u_dev : out,
-                     direct ? drho_dev : out + 3 * B.N, d.tau, s));
+                     reinterpret_cast<float*>(counts + ctx->maxp + 1), ctx->d_sums, direct ? uv : out,
+                     direct ? dv : out + 3 * B.N, d.tau, s));
     if (!direct) {
         CK(cudaMemcpyAsync(u_dev, out, 3ull * B.N * sizeof(float), cudaMemcpyDeviceToDevice, s));
         if (drho_dev) CK(cudaMemcpyAsync(drho_dev, out + 3 * B.N, (size_t)B.N * sizeof(float), cudaMemcpyDeviceToDevice, s));

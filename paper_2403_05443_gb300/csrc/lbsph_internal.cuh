@@ -39,6 +39,7 @@
 //                  critical particle kernel.
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -158,6 +159,20 @@ __host__ __device__ __forceinline__ int div_magic(int n, unsigned m, int s)
 #else
     return s < 0 ? n : (int)((((unsigned long long)(unsigned)n * m) >> 32) >> s);
 #endif
+}
+
+// Device address of caller memory of `bytes` bytes, a and b the attributes of its first and last
+// byte, that kernels on GPU `device` may read and write in place: that GPU's own memory, managed
+// memory, page-locked host memory.  Null for another GPU's (reachable by a copy, but by a kernel
+// only with peer access), for pageable memory, and for a range that is not one mapping.
+inline void* in_place_view(const cudaPointerAttributes& a, const cudaPointerAttributes& b, size_t bytes, int device)
+{
+    if (a.type != b.type || !a.devicePointer || !b.devicePointer) return nullptr;
+    if (static_cast<const char*>(b.devicePointer) - static_cast<const char*>(a.devicePointer) != (ptrdiff_t)(bytes - 1))
+        return nullptr;
+    if (a.type == cudaMemoryTypeDevice && a.device != device) return nullptr;
+    if (a.type != cudaMemoryTypeDevice && a.type != cudaMemoryTypeManaged && a.type != cudaMemoryTypeHost) return nullptr;
+    return a.devicePointer;
 }
 
 // FP32 snapshot of one particle for the lattice kernels, written by the
