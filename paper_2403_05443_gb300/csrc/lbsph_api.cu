@@ -44,6 +44,7 @@ using namespace lbsph;
 
 namespace {
 constexpr int STEP_ITERS = 256;     // iterations per launch of the step kernel
+constexpr int RECS_COPY = 512;      // particle records that come through the page-locked buffer (lb_get_force_torque)
 }
 
 struct lb_ctx {
@@ -72,7 +73,8 @@ struct lb_ctx {
     float* d_tmp = nullptr;
     float2* d_stokes = nullptr;         // lb_stokes_field: complex [2][N] and int [N] of the largest box
     double* d_sums = nullptr;           // its sums, shifts and counters, then node counts and force values per particle
-    unsigned* h_back = nullptr;         // page-locked: the status word, 8 bytes on the records of maxp particles
+    unsigned* d_rec = nullptr;          // the same on the device, for the records of maxp particles
+    unsigned* h_back = nullptr;         // page-locked: the status word, 8 bytes on up to RECS_COPY records
     size_t tmp_bytes = 0;
     bool collided = false;
     bool stepped = false;
@@ -182,7 +184,7 @@ static lb_status read_status(lb_ctx* ctx)
 static lb_status back_buffer(lb_ctx* ctx)
 {
     if (ctx->h_back) return LB_OK;
-    const size_t bytes = 8 + sizeof(double) * LB_RECORD_DOUBLES * (size_t)std::max(ctx->maxp, 1);
+    const size_t bytes = 8 + sizeof(double) * LB_RECORD_DOUBLES * (size_t)RECS_COPY;
     if (cudaHostAlloc((void**)&ctx->h_back, bytes, cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess) return LB_OK;
     cudaGetLastError();
     ctx->h_back = nullptr;
@@ -198,13 +200,16 @@ static lb_status finish(lb_ctx* ctx, cudaStream_t s)
     return judge_status(ctx, *ctx->h_back);
 }
 
-// records of n particles, `stride` bytes apart, and the status word (out: its device address)
+// Records of n particles, `stride` bytes apart, and the status word (out: its device address).
+// One double per thread: bound by the latency of a load and a store to host memory, so as many
+// of them in flight as there are.
 __global__ void records_kernel(const char* rec, size_t stride, int n, const unsigned* status, unsigned* out)
 {
-    double* d = reinterpret_cast<double*>(out + 2);
-    for (int e = threadIdx.x; e < n * LB_RECORD_DOUBLES; e += blockDim.x)
-        d[e] = reinterpret_cast<const double*>(rec + (size_t)(e / LB_RECORD_DOUBLES) * stride)[e % LB_RECORD_DOUBLES];
-    if (threadIdx.x == 0) *out = *status;
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < n * LB_RECORD_DOUBLES)
+        reinterpret_cast<double*>(out + 2)[e] =
+            reinterpret_cast<const double*>(rec + (size_t)(e / LB_RECORD_DOUBLES) * stride)[e % LB_RECORD_DOUBLES];
+    if (e == 0) *out = *status;
 }
 
 // ---------------------------------------------------------------------------
@@ -1183,14 +1188,29 @@ extern "C" lb_status lb_get_force_torque(lb_ctx* ctx, int32_t box, double* out, 
     if (ctx->last_user_stream && ctx->last_user_stream != ctx->stream) CK(cudaStreamSynchronize(ctx->last_user_stream));
     const lb_status r = back_buffer(ctx);
     if (r != LB_OK) return r;
-    unsigned* back = nullptr;
-    CK(cudaHostGetDevicePointer((void**)&back, ctx->h_back, 0));
     const bool d27 = ctx->lattice == 27;
     const int slot = all ? 0 : (d27 ? ctx->box27_part[box] : ctx->hbox[box].pbeg);
     const char* rec = d27 ? (const char*)&ctx->d_part27[slot].rec[0] : (const char*)&ctx->d_pd[slot].rec[0];
+    const size_t stride = d27 ? sizeof(q27::Part27) : sizeof(PartDev);
+    // A few records come with the status word into the page-locked buffer.  From there on the host's
+    // own copy out of that buffer costs more than gathering on the device and one copy into the
+    // caller's array.  us per call for 64 / 512 / 1,024 / 4,096 / 8,192 records: page-locked 12.4 /
+    // 17.7 / 24 / 61 / 114, copied 24 at 1,024, 28 and 32 (a strided copy straight out of the states 24 / 36 / 56 from
+    // 1,024 on; one block for all records 13.5 / 27 / 42 / 137 / 268).
+    const bool few = n <= RECS_COPY;
+    if (!few && !ctx->d_rec) {
+        ctx->d_rec = (unsigned*)dev_alloc(ctx, 8 + sizeof(double) * LB_RECORD_DOUBLES * ctx->maxp);
+        if (!ctx->d_rec) return fail(ctx, LB_ENOMEM, "record staging buffer");
+    }
+    unsigned* to = ctx->d_rec;
+    if (few) CK(cudaHostGetDevicePointer((void**)&to, ctx->h_back, 0));
     clear_stale_error();
-    records_kernel<<<1, 256, 0, ctx->stream>>>(rec, d27 ? sizeof(q27::Part27) : sizeof(PartDev), n, ctx->d_status, back);
+    records_kernel<<<(n * LB_RECORD_DOUBLES + 255) / 256, 256, 0, ctx->stream>>>(rec, stride, n, ctx->d_status, to);
     CK(cudaGetLastError());
+    if (!few) {
+        CK(cudaMemcpyAsync(out, to + 2, sizeof(double) * LB_RECORD_DOUBLES * n, cudaMemcpyDeviceToHost, ctx->stream));
+        return finish(ctx, ctx->stream);
+    }
     CK(cudaStreamSynchronize(ctx->stream));
     std::memcpy(out, ctx->h_back + 2, sizeof(double) * LB_RECORD_DOUBLES * n);
     return judge_status(ctx, *ctx->h_back);
