@@ -363,7 +363,10 @@ __device__ __forceinline__ float softplus(float y) { return y > 20.0f ? y : log1
 __device__ __forceinline__ float sigmoid(float y) { return 1.0f / (1.0f + expf(-y)); }
 
 // ---- PTX helpers
-// programmatic dependent launch: wait for the kernels before this one; let the next one start its prologue
+// programmatic dependent launch: wait for the kernels before this one; let the next one start its prologue.
+// A kernel launched like that may be running while the one before it still writes, so what that one writes is
+// read by plain (or .cg) loads after the wait and never by non-coherent ones (__ldg), which ask for data that
+// nobody writes while the reading kernel runs; a caller's inputs may be the outputs of the call before.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void mbar_init(unsigned long long* b)
@@ -566,7 +569,7 @@ __device__ __forceinline__ float head_row(const float* T, int i, const float* rt
         if (R_out) R_out[j] = a;
         dR[j] = 0.0f;
         if (rt) {
-            const float d = a - __ldg(rt + j);
+            const float d = a - rt[j];
             err += d * d;
             dR[j] = c * d;
         }
@@ -619,11 +622,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) net_kernel(const NetArgs A)
         float f[NIN];
         const float* xs = A.x + (long long)s * NIN;
         if (live && (reinterpret_cast<uintptr_t>(A.x) & 15u) == 0) {
-            const float4 u = __ldg(reinterpret_cast<const float4*>(xs)), v = __ldg(reinterpret_cast<const float4*>(xs) + 1);
+            const float4 u = *reinterpret_cast<const float4*>(xs), v = *(reinterpret_cast<const float4*>(xs) + 1);
             f[0] = u.x; f[1] = u.y; f[2] = u.z; f[3] = u.w; f[4] = v.x; f[5] = v.y; f[6] = v.z; f[7] = v.w;
         } else {
 #pragma unroll
-            for (int k = 0; k < NIN; ++k) f[k] = live ? __ldg(xs + k) : 0.0f;
+            for (int k = 0; k < NIN; ++k) f[k] = live ? xs[k] : 0.0f;
         }
         const uint4 c0 = make_uint4(pack2(f[0], f[1]), pack2(f[2], f[3]), pack2(f[4], f[5]), pack2(f[6], f[7]));
         const uint4 c1 = make_uint4(0u, 0u, 0u, 0u);
@@ -635,7 +638,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) net_kernel(const NetArgs A)
         }
     }
     for (int k = tid; k < 2 * NH + NOUTP; k += NTHREADS)
-        sb[k] = __ldg(A.p + (k < NH ? OFF_B1 + k : (k < 2 * NH ? OFF_B2 + k - NH : OFF_B3 + k - 2 * NH)));
+        sb[k] = A.p[k < NH ? OFF_B1 + k : (k < 2 * NH ? OFF_B2 + k - NH : OFF_B3 + k - 2 * NH)];
     fence_async();
     tc_before();
     __syncthreads();
@@ -907,7 +910,7 @@ __global__ void __launch_bounds__(GTHREADS_N, 1) grad_kernel(const GradArgs G)
         } else {
             if (warp > 0) return;
 #pragma unroll 8
-            for (int t = 0; t < 4 * G.tiles; ++t) v += __ldg(G.act.b_part + (long long)t * NSUM + c0 + lane);
+            for (int t = 0; t < 4 * G.tiles; ++t) v += __ldcg(G.act.b_part + (long long)t * NSUM + c0 + lane);
         }
         if (!ok) {
             if (lane == 0) {
