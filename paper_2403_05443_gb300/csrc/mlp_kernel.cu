@@ -897,7 +897,7 @@ __global__ void __launch_bounds__(GTHREADS_N, 1) grad_kernel(const GradArgs G)
             __syncthreads();
             if (warp > 0) return;
             bulk_load(sm + lane * (bytes + 16), G.act.d32 + (long long)(c0 + lane) * G.act.ns, (unsigned)bytes, full);
-            ok = mbar_wait(full, 0u);
+            ok = __all_sync(0xffffffffu, mbar_wait(full, 0u));
             const float4* d = reinterpret_cast<const float4*>(sm + lane * (bytes + 16));
 #pragma unroll 8
             for (int t = 0; t < G.tiles * TILE / 4; ++t) {
@@ -913,6 +913,8 @@ __global__ void __launch_bounds__(GTHREADS_N, 1) grad_kernel(const GradArgs G)
             for (int t = 0; t < 4 * G.tiles; ++t) v += __ldcg(G.act.b_part + (long long)t * NSUM + c0 + lane);
         }
         if (!ok) {
+            // a second bounded wait for the copies in flight before leaving
+            (void)mbar_wait(full, 0u);
             if (lane == 0) {
                 atomicOr(&g_gemm_status, 1u);
                 if (G.status) atomicOr(G.status, 1u);
@@ -971,17 +973,20 @@ __global__ void __launch_bounds__(GTHREADS_N, 1) grad_kernel(const GradArgs G)
     pdl_wait();
     const unsigned tmem = s_tmem;
     bool ok = true;
+    int issued = 0;                             // stages this thread has loaded, or passed to the tensor core
     if (warp == 16) {
         // loads: one column group (2 KiB of a tile) per lane
         const int ng = 16 + ncol / 8;
         for (int t = t0; t < t1; ++t) {
             const int st = (t - t0) % GST, use = (t - t0) / GST;
-            if (use > 0 && !mbar_wait(empty + st, (unsigned)(use - 1) & 1u)) { ok = false; break; }
+            // one decision per warp: lanes whose waits ended differently would part at the barrier below
+            if (!__all_sync(0xffffffffu, use == 0 || mbar_wait(empty + st, (unsigned)(use - 1) & 1u))) { ok = false; break; }
             unsigned char* d = sm + st * (GS_A + GS_B);
             if (lane == 0) mbar_expect(full + st, (unsigned)(ng * CS_T));
             __syncwarp();
             if (lane < 16) bulk_load(d + lane * CS_T, a + lane * G.act.cs + (long long)t * CS_T, CS_T, full + st);
             else if (lane < ng) bulk_load(d + GS_A + (lane - 16) * CS_T, b + (lane - 16) * G.act.cs + (long long)t * CS_T, CS_T, full + st);
+            ++issued;
         }
     } else if (tid == 17 * 32) {
         const unsigned idesc = idesc_bf16(TILE, ncol) | (1u << 15) | (1u << 16);     // both MN-major
@@ -992,6 +997,7 @@ __global__ void __launch_bounds__(GTHREADS_N, 1) grad_kernel(const GradArgs G)
             const unsigned ad = smem_u32(sm + st * (GS_A + GS_B)), bd = ad + GS_A;
             mma_chain(tmem, sdesc(ad, 128u, CS_T), 256 / 16, sdesc(bd, 128u, CS_T), 256 / 16, idesc, TILE / 16, t > t0);
             mma_commit(empty + st);
+            ++issued;
         }
         if (ok) {
             mma_commit(&done);
@@ -1014,7 +1020,13 @@ __global__ void __launch_bounds__(GTHREADS_N, 1) grad_kernel(const GradArgs G)
             atomicOr(&g_gemm_status, 1u);
             if (G.status) atomicOr(G.status, 1u);
         }
-        for (int k = 0; k < GST; ++k) (void)mbar_wait(full + k, 0u);
+        // a second bounded wait for what is in flight: the last copies into every stage, and the products (which
+        // complete in order, so the last one's arrival covers them all)
+        if (warp == 16)
+            for (int k = max(0, issued - GST); k < issued; ++k) (void)mbar_wait(full + k % GST, (unsigned)(k / GST) & 1u);
+        else if (tid == 17 * 32 && issued > 0)
+            (void)mbar_wait(empty + (issued - 1) % GST, (unsigned)((issued - 1) / GST) & 1u);
+        __syncthreads();
     }
     if (nrank > 1) {
         // the other blocks' parts into the first one's stages: column j of row m at (j * 128 + m) floats

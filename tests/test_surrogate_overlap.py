@@ -1,7 +1,11 @@
 """The network's kernels start while the kernel before them may still be writing (programmatic launch).  What that one
 writes must not be read by non-coherent loads (__ldg: read-only for the whole life of the reading kernel).  It may be a
 caller's buffer as well: the prediction of one forward pass as the targets of the next call, all of it queued without
-a wait, gives the same bits as with a wait after every call."""
+a wait, gives the same bits as with a wait after every call.
+
+Every wait in them is bounded.  One that gives up must do so for the whole warp (lanes that part would meet at
+different barriers), and the block must wait again for the copies and products it has in flight before it leaves; no
+such wait can be made to run out here without holding up the GPU, so this is checked in the source."""
 import os
 import re
 
@@ -17,6 +21,21 @@ def test_no_non_coherent_load_in_kernels_that_start_early(kernel):
         text = f.read()
     m = re.search(r"\n[^\n/]*\b%s\(.*?\n}\n" % kernel, text, re.S)
     assert m and "__ldg(" not in m.group(0)
+
+
+def test_a_wait_that_gives_up_leaves_nothing_in_flight():
+    with open(os.path.join(ROOT, "paper_2403_05443_gb300", "csrc", "mlp_kernel.cu")) as f:
+        text = f.read()
+    body = re.search(r"\n[^\n/]*\bgrad_kernel\(.*?\n}\n", text, re.S).group(0)
+    bias, tiles = body.split("// ---- operands and place of this tile")
+    # waits by a whole warp: decided together
+    assert len(re.findall(r"__all_sync\(0xffffffffu, mbar_wait\(full", bias)) == 1
+    assert len(re.findall(r"__all_sync\(0xffffffffu, use == 0 \|\| mbar_wait\(empty", tiles)) == 1
+    # the second waits: the biases' copies; the last copies into every stage and the last product of a tile's
+    assert re.search(r"if \(!ok\) \{[^}]*\(void\)mbar_wait\(full, 0u\);", bias)
+    fail = tiles.split("if (fail) {", 1)[1].split("if (nrank > 1)", 1)[0]
+    assert "k = max(0, issued - GST); k < issued; ++k) (void)mbar_wait(full + k % GST, (unsigned)(k / GST) & 1u)" in fail
+    assert "(void)mbar_wait(empty + (issued - 1) % GST, (unsigned)((issued - 1) / GST) & 1u)" in fail
 
 
 @pytest.mark.gpu
