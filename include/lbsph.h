@@ -334,8 +334,11 @@ lb_status lb_init_fluid(lb_ctx* ctx, int32_t box, const float* u, size_t u_bytes
  * the balancing -sum F_ext / N_fluid on the fluid nodes; a net mean force is
  * dropped.  The flow is the exact steady state of the linear lattice dynamics
  * itself (D3Q19 BGK with Guo forcing at the box's tau and rho0), solved mode by
- * mode in Fourier space (DFTs on the device, a 4 x 4 system in the conserved
- * moments per mode in FP64): at the scales of a few nodes the lattice's own
+ * mode in Fourier space (FP32 transforms on the device; per mode a symmetric
+ * 3 x 3 system for the velocity and a scalar equation for the density, the
+ * directions' terms in FP32, their sums and the solve with twice FP32's digits;
+ * the result is within 4e-7 of the 64-bit one, normwise, for edges without
+ * large prime factors, also near tau = 1/2): at the scales of a few nodes the lattice's own
  * viscous and pressure operators differ from a Stokes stencil by several per
  * cent, and only a start on the lattice's own steady state avoids the slow
  * relaxation of that difference.  Then a uniform velocity is added on the
