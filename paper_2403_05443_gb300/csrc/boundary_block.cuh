@@ -338,11 +338,9 @@ __device__ __noinline__ void boundary_block(const BndParams& kernel_params, int 
                     float ux = K.U[0] + (K.W[1] * pz - K.W[2] * py);
                     float uy = K.U[1] + (K.W[2] * px - K.W[0] * pz);
                     float uz = K.U[2] + (K.W[0] * py - K.W[1] * px);
-                    if (K.squirmer) {
-                        float qx, qy, qz;
-                        squirmer_slip(ex, K.a, K.eps2, K.B1, K.B2, px, py, pz, qx, qy, qz);
-                        ux += qx; uy += qy; uz += qz;
-                    }
+                    float qx, qy, qz;
+                    squirmer_slip(ex, K.a, K.eps2, K.B1, K.B2, px, py, pz, qx, qy, qz);
+                    ux += qx; uy += qy; uz += qz;
                     const float ubc = cx_of(i) * ux + cy_of(i) * uy + cz_of(i) * uz;
                     f[i] += 6.0f * w_of(i) * rho0 * ubc;
                 }

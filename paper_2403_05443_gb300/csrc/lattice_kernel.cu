@@ -51,9 +51,7 @@ __device__ __forceinline__ bool hits(int lo, int hi, int ow, int S, int L)
 // ---------------------------------------------------------------------------
 enum { FK_F = 0, FK_MOMENTS = 1, FK_SOLID = 2 };
 
-// blocks per SM the registers are held to
-template <class St, int WHAT>
-constexpr int FIELD_BLOCKS = 2;
+constexpr int FIELD_BLOCKS = 2;             // blocks per SM the registers are held to
 
 // Density deviation and momentum of one node's populations, in this order of additions.
 __device__ __forceinline__ void node_moments(const float (&f)[Q], float rho0, const float* g, float& drho, float& ux,
@@ -238,7 +236,7 @@ __device__ __forceinline__ void surface_node(const KParams& P, const BoxDev& B, 
 }
 
 template <class St, int WHAT>
-__global__ void __launch_bounds__(KBLOCK, FIELD_BLOCKS<St, WHAT>) fields_kernel(const __grid_constant__ KParams P)
+__global__ void __launch_bounds__(KBLOCK, FIELD_BLOCKS) fields_kernel(const __grid_constant__ KParams P)
 {
     using T = typename St::T;
     __shared__ float s_g[3];

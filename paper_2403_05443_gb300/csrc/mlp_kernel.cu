@@ -51,11 +51,9 @@ struct GemmArgs {
     int M, N, K;
     const float* bias;
     int relu;
-    const __nv_bfloat16* mask;          // if set: C *= (mask(m, n) > 0), same strides as C
     float* C32;
     __nv_bfloat16* C16;
     long long c_sm, c_sn;
-    unsigned* status;
 };
 
 __device__ unsigned g_gemm_status;      // bit 0: a completion wait gave up
@@ -227,10 +225,7 @@ __global__ void __launch_bounds__(GTHREADS) gemm_kernel(const GemmArgs g)
     }
     if (!ok) {
         // give the issued products a second bounded wait before freeing TMEM
-        if (tid == 0) {
-            atomicOr(&g_gemm_status, 1u);
-            if (g.status) atomicOr(g.status, 1u);
-        }
+        if (tid == 0) atomicOr(&g_gemm_status, 1u);
         (void)mbar_wait(&bar, phase ^ 1u);
     } else {
         const int m = m0 + warp * 32 + lane;
@@ -252,7 +247,6 @@ __global__ void __launch_bounds__(GTHREADS) gemm_kernel(const GemmArgs g)
                     if (g.bias) v += g.bias[n];
                     if (g.relu) v = fmaxf(v, 0.0f);
                     const long long o = m * g.c_sm + n * g.c_sn;
-                    if (g.mask && !(__bfloat162float(g.mask[o]) > 0.0f)) v = 0.0f;
                     if (g.C32) g.C32[o] = v;
                     if (g.C16) g.C16[o] = __float2bfloat16(v);
                 }
@@ -453,7 +447,6 @@ struct NetArgs {
     float* loss;                        // !BWD: the loss is summed here by the last tile
     Acts act;
     int n;
-    unsigned* status;
 };
 
 constexpr int NS_W2 = 0, NS_W3 = NS_W2 + NH * NH * 2, NS_H = NS_W3 + NOUTP * NH * 2, NS_BIAS = NS_H + TILE * NH * 2,
@@ -798,10 +791,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) net_kernel(const NetArgs A)
     } while (false);
     if (!ok) {
         // a completion never came: give what is in flight a second bounded wait before leaving
-        if (tid == 0) {
-            atomicOr(&g_gemm_status, 1u);
-            if (A.status) atomicOr(A.status, 1u);
-        }
+        if (tid == 0) atomicOr(&g_gemm_status, 1u);
         (void)mbar_wait(bar, 0u);
         if (pending) (void)mbar_wait(bar + 1, 0u);
         (void)mbar_wait(bar + 2, phase ^ 1u);
@@ -849,7 +839,6 @@ struct GradArgs {
     unsigned char* w;
     float lr, c1, c2;
     float* loss;
-    unsigned* status;
 };
 
 constexpr int GST = 5, GS_A = 16 * CS_T, GS_B = 4 * CS_T, GRAD_SMEM = GST * (GS_A + GS_B);
@@ -915,10 +904,7 @@ __global__ void __launch_bounds__(GTHREADS_N, 1) grad_kernel(const GradArgs G)
         if (!ok) {
             // a second bounded wait for the copies in flight before leaving
             (void)mbar_wait(full, 0u);
-            if (lane == 0) {
-                atomicOr(&g_gemm_status, 1u);
-                if (G.status) atomicOr(G.status, 1u);
-            }
+            if (lane == 0) atomicOr(&g_gemm_status, 1u);
             return;
         }
         if (c0 + lane >= 2 * NH + NOUT) v = 0.0f;     // padding
@@ -1016,10 +1002,7 @@ __global__ void __launch_bounds__(GTHREADS_N, 1) grad_kernel(const GradArgs G)
 #pragma unroll
     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(acc[j >> 4][j & 15]);
     if (fail) {
-        if (tid == 0) {
-            atomicOr(&g_gemm_status, 1u);
-            if (G.status) atomicOr(G.status, 1u);
-        }
+        if (tid == 0) atomicOr(&g_gemm_status, 1u);
         // a second bounded wait for what is in flight: the last copies into every stage, and the products (which
         // complete in order, so the last one's arrival covers them all)
         if (warp == 16)
