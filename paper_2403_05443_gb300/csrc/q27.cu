@@ -734,8 +734,9 @@ __global__ void __launch_bounds__(PBLK, 1) particle27_kernel(const __grid_consta
                 qstep27(D->q, Wm, qn);
                 const int k = lane % 3;
                 const double xn = D->x[k] + 0.5 * (D->U[k] + s_x6[k]);
-                finite = __all_sync(0xffffffffu, isfinite(xn) && isfinite(s_x6[k]) && isfinite(s_x6[k + 3]) && isfinite(qn[0]) &&
-                                                     isfinite(qn[1]) && isfinite(qn[2]) && isfinite(qn[3]));
+                int ex = max(exponent27(xn), max(exponent27(s_x6[k]), exponent27(s_x6[k + 3])));
+                for (int c = 0; c < 4; ++c) ex = max(ex, exponent27(qn[c]));
+                finite = __all_sync(0xffffffffu, ex != 0x7ff);
                 __syncwarp();
                 if (lane < 3) {
                     D->x[lane] = xn;

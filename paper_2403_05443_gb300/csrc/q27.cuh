@@ -27,6 +27,7 @@
 
 #include <cmath>
 #include <cstdint>
+#include <cstring>
 #include <cuda_runtime.h>
 
 #include "lbsph_internal.cuh"
@@ -68,9 +69,22 @@ __host__ __device__ constexpr float w27(int i) { return (float)wd27(i); }
 // Cube origin floor(x) - h along an axis.  False, and the origin a centre at 0 would have, for a
 // centre that is not finite or so far out that the origin's arithmetic could leave 32 bits.
 constexpr double POS_MAX27 = 536870912.0;        // 2^29
+// The biased exponent: 0x7ff for NaN and Inf, 1023 + 29 and more from |x| = 2^29 on.  Integer tests of it
+// instead of FP64 comparisons, which issue at this part's slow FP64 rate on the particle's chain (141 steps of five
+// boxes with their read-back: 8,922 us with comparisons, 8,806-8,906 like this, 8,884-8,889 without any test).
+__host__ __device__ inline int exponent27(double x)
+{
+#ifdef __CUDA_ARCH__
+    return (__double2hiint(x) >> 20) & 0x7ff;
+#else
+    unsigned long long b;
+    memcpy(&b, &x, 8);
+    return (int)(b >> 52) & 0x7ff;
+#endif
+}
 __host__ __device__ inline bool cube_origin27(double x, int h, int& o)
 {
-    const bool ok = x > -POS_MAX27 && x < POS_MAX27;       // false for NaN
+    const bool ok = exponent27(x) < 1023 + 29;             // |x| < POS_MAX27
     o = (ok ? (int)floor(x) : 0) - h;
     return ok;
 }
