@@ -94,6 +94,7 @@ __device__ __forceinline__ void box_force(const KParams& P, const BoxDev& B, int
 }
 
 // A 256-quad tile may meet at most MAXC particles (grown by one node; old and new cubes): else ST_CAPACITY.  One warp.
+// The blocks here would do with any number; callers have always been refused beyond MAXC, and still are.
 __device__ __forceinline__ void tile_capacity(const KParams& P, const BoxDev& B, int q0, int lane)
 {
     const int ny = B.ny, nz = B.nz;
